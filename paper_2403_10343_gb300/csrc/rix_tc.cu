@@ -157,42 +157,61 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
 }
 
-// The MMAs of one K stage: slice pairs (s, u) with s + u < S, each into
-// accumulator min(s + u, NACC - 1), two K steps of 16.  ad0 / bd0 are the
-// descriptors of slice 0 of the stage; the others follow at fixed offsets (the
-// start-address field counts 16-byte units and stays below 2^14 in shared
-// memory).  In this order the first MMA into every accumulator is the one with
-// s = 0, kk = 0 and u <= NACC - 1; for the accumulators whose bit is set in
-// open (a group of them starts at this stage) it overwrites the accumulator.
-template <int S>
-__device__ __forceinline__ void issue_stage(uint32_t tmem, uint64_t ad0, uint64_t bd0, uint32_t idesc,
-                                            uint32_t open) {
-#pragma unroll
-  for (int s = 0; s < S; s++)
-#pragma unroll
-    for (int u = 0; u < S - s; u++) {
-      const int a = s + u < NACC - 1 ? s + u : NACC - 1;
-#pragma unroll
-      for (int kk = 0; kk < KC / 16; kk++) {
-        const uint64_t ad = ad0 + (uint64_t)((s * A_TILE + kk * 256) >> 4);
-        const uint64_t bd = bd0 + (uint64_t)((u * B_TILE + kk * 256) >> 4);
-        const bool first = s == 0 && kk == 0 && u <= NACC - 1;
-        mma_bf16(tmem + (uint32_t)(a * TN), ad, bd, idesc, first ? 1u - ((open >> a) & 1u) : 1u);
-      }
-    }
+// Widest run of B slices one MMA takes (N = RUN x 80, at most 256 columns).
+constexpr int RUN = 3;
+__host__ __device__ constexpr int run_width(int left) {  // next run of `left` slices: 3, or 2 + 2 for four
+  return left <= RUN ? left : left == RUN + 1 ? 2 : RUN;
 }
 
-__device__ __forceinline__ void issue_stage_s(int S, uint32_t tmem, uint64_t ad0, uint64_t bd0, uint32_t idesc,
-                                              uint32_t open) {
+// The MMAs of one K stage: slice pairs (s, u) with s + u < S, each into
+// accumulator min(s + u, NACC - 1), two K steps of 16.  The B tiles of
+// consecutive slices lie back to back in shared memory (one K-major matrix of
+// 80 rows per slice) and their accumulators s + u, s + u + 1, ... back to back
+// in tensor memory, so one MMA with N = 80 w columns multiplies A slice s by w
+// B slices at once.  With N = 80 each MMA reads 4 KB of A and 2.5 KB of B for
+// 40 tensor cycles, more than the 128 B per clock shared memory gives (51
+// cycles); at N = 240 it reads 11.5 KB for 120, and the tensor pipe is the
+// bound.  (GB300, (H2O)64 build at six slices: the 13 GEMM launches 142 ms with
+// single pairs, 128 ms with runs; the build 183.0 and 169.3 ms.)  The pairs beyond the last accumulator (S > NACC) go one by one.
+// ad0 / bd0 are the descriptors of slice 0 of the stage; the others follow at
+// fixed offsets (the start-address field counts 16-byte units and stays below
+// 2^14 in shared memory).  With open set (a group of accumulations starts at
+// this stage) the MMAs of A slice 0 and the first K step overwrite their
+// accumulators; they come first and cover all of them.
+template <int S>
+__device__ __forceinline__ void issue_stage(uint32_t tmem, uint64_t ad0, uint64_t bd0, uint32_t open) {
+#pragma unroll
+  for (int s = 0; s < S; s++) {
+    const int top = S < NACC ? S : NACC;  // accumulators in use
+    const int nu = top - s;               // slices u with an accumulator of their own
+#pragma unroll
+    for (int u = 0; u < nu; u += run_width(nu - u)) {
+      const int w = run_width(nu - u);
+#pragma unroll
+      for (int kk = 0; kk < KC / 16; kk++)
+        mma_bf16(tmem + (uint32_t)((s + u) * TN), ad0 + (uint64_t)((s * A_TILE + kk * 256) >> 4),
+                 bd0 + (uint64_t)((u * B_TILE + kk * 256) >> 4), idesc_bf16(TM, w * TN),
+                 s == 0 && kk == 0 ? 1u - open : 1u);
+    }
+#pragma unroll
+    for (int u = nu > 0 ? nu : 0; u < S - s; u++)
+#pragma unroll
+      for (int kk = 0; kk < KC / 16; kk++)
+        mma_bf16(tmem + (uint32_t)((NACC - 1) * TN), ad0 + (uint64_t)((s * A_TILE + kk * 256) >> 4),
+                 bd0 + (uint64_t)((u * B_TILE + kk * 256) >> 4), idesc_bf16(TM, TN), 1u);
+  }
+}
+
+__device__ __forceinline__ void issue_stage_s(int S, uint32_t tmem, uint64_t ad0, uint64_t bd0, uint32_t open) {
   switch (S) {
-    case 1: issue_stage<1>(tmem, ad0, bd0, idesc, open); break;
-    case 2: issue_stage<2>(tmem, ad0, bd0, idesc, open); break;
-    case 3: issue_stage<3>(tmem, ad0, bd0, idesc, open); break;
-    case 4: issue_stage<4>(tmem, ad0, bd0, idesc, open); break;
-    case 5: issue_stage<5>(tmem, ad0, bd0, idesc, open); break;
-    case 6: issue_stage<6>(tmem, ad0, bd0, idesc, open); break;
-    case 7: issue_stage<7>(tmem, ad0, bd0, idesc, open); break;
-    default: issue_stage<8>(tmem, ad0, bd0, idesc, open); break;
+    case 1: issue_stage<1>(tmem, ad0, bd0, open); break;
+    case 2: issue_stage<2>(tmem, ad0, bd0, open); break;
+    case 3: issue_stage<3>(tmem, ad0, bd0, open); break;
+    case 4: issue_stage<4>(tmem, ad0, bd0, open); break;
+    case 5: issue_stage<5>(tmem, ad0, bd0, open); break;
+    case 6: issue_stage<6>(tmem, ad0, bd0, open); break;
+    case 7: issue_stage<7>(tmem, ad0, bd0, open); break;
+    default: issue_stage<8>(tmem, ad0, bd0, open); break;
   }
 }
 
@@ -651,7 +670,6 @@ __global__ void __launch_bounds__(NTHR, 1) k_gemm_sliced(GemmArgs g) {
       atomicAdd(g.chunks, (unsigned long long)cg * (unsigned long long)(S * (S + 1) / 2) * (KC / 16));
   } else if (warp == 1 && lane == 0) {
     // ------------------------------------------------------------ MMA issuer
-    const uint32_t idesc = idesc_bf16(TM, TN);
     uint32_t cg = 0, gg = 0;  // chunks consumed, accumulation groups completed
     bool issued = false;
     if (g.stall && !mbar_wait(never, 0, g.wait_ns)) atomicExch(abort_flag, 1);
@@ -676,8 +694,8 @@ __global__ void __launch_bounds__(NTHR, 1) k_gemm_sliced(GemmArgs g) {
         const uint32_t sa = smem_u32(smem + st * stage_bytes);
         const uint32_t sb = sa + S * A_TILE;
         // K step kk covers core-matrix columns 2kk, 2kk+1 (LBO = 128 B apart)
-        const uint32_t open = lc % GROUP == 0 ? 0xFFu : 0u;  // every accumulator starts a group
-        issue_stage_s(S, tmem, sdesc(sa, 128, (KC / 8) * 128), sdesc(sb, 128, (KC / 8) * 128), idesc, open);
+        const uint32_t open = lc % GROUP == 0 ? 1u : 0u;  // every accumulator starts a group
+        issue_stage_s(S, tmem, sdesc(sa, 128, (KC / 8) * 128), sdesc(sb, 128, (KC / 8) * 128), open);
         issued = true;
         mma_commit(&empty[st]);
         if (lc % GROUP == GROUP - 1 || lc == ti.nlive - 1) {
