@@ -358,8 +358,10 @@ rix_status rix_stats(const rix_ctx *ctx, rix_stats_t *out);
  * one rix_build_K with the density matrix D_dev (device, packed) performs
  * after block screening (Sec. "Screening": products whose C, V or D block has
  * no element of magnitude >= tau are skipped).  Terms 1 and 4 are symmetric
- * under the transposition of their block (Eq. 11), so the build evaluates them
- * for one orientation of each pair / K block and these counts do the same.  The counts of rix_stats_t
+ * under the transposition of their block (Eq. 11), and these counts take them
+ * once per pair / K block, with every Z product; where the build halves term 4
+ * in Z instead of in the K blocks (chosen at setup) it performs other and
+ * fewer products than [3] and [4] say.  The counts of rix_stats_t
  * include every product; these depend on D.  flops (host, 10 doubles):
  * [0] T, [1] U2, [2] terms 1+2, [3] Z, [4] terms 3+4, [5] symmetrise, [6] the
  * term-2 part of [2], [7] the part of [2] for the column atoms whose term 1

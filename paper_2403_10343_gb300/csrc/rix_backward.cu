@@ -132,14 +132,14 @@ __global__ void __launch_bounds__(NT) kb_Z34(const int4 *items, const int64_t *p
 }
 
 // ---------------------------------------------------------------- Vbar(B,G') from term 4
-// Fbar[P][k][l] = 1/2 sum_j D(B,G')[j][k] Zbar(B,E')[P][j][l];  Vbar[P][Q] += sum_kl Fbar C(G',E')[Q on G'][k][l]
+// Fbar[P][k][l] = w sum_j D(B,G')[j][k] Zbar(B,E')[P][j][l] (w: wZ of the pair);  Vbar[P][Q] += sum_kl Fbar C(G',E')[Q on G'][k][l]
 __global__ void __launch_bounds__(NT) kb_ZV(const int4 *items, const int64_t *ptr, const int2 *L, const int32_t *pA,
                                             const int32_t *pB, const int32_t *nb, const int32_t *na,
                                             const double *__restrict__ C, const int64_t *offC,
                                             const double *__restrict__ D, const int64_t *offD,
                                             const uint8_t *keepC, const uint8_t *keepV, const uint8_t *keepD,
-                                            const double *__restrict__ Zbar, const int64_t *off2,
-                                            const int64_t *offV, Win w, double *dV) {
+                                            const uint8_t *wZ, const double *__restrict__ Zbar, const int64_t *off2,
+                                            const int64_t *offV, Win win, double *dV) {
   extern __shared__ double sm[];
   const int4 it = items[blockIdx.x];
   const int p2 = it.x, p0 = it.y;
@@ -150,16 +150,17 @@ __global__ void __launch_bounds__(NT) kb_ZV(const int4 *items, const int64_t *pt
   const int pe = min(naB, p0 + tile_rows(per));
   const int nel = (pe - p0) * per;
   const double *Dbg = D + offD[p2];
+  const double w = wZ[p2] == 2 ? 0.5 : 1.0;
   double acc[MAXE];
 #pragma unroll
   for (int r = 0; r < MAXE; r++) acc[r] = 0.0;
   for (int64_t x = ptr[p2]; x < ptr[p2 + 1]; x++) {
     const int2 en = L[x];
-    if (!keepC[en.x] || !in_win(w, en.y)) continue;
+    if (!keepC[en.x] || !in_win(win, en.y)) continue;
     const int e = pB[en.x];
     const int nbE = nb[e];
     const double *Cg = C + offC[en.x];
-    const double *Zb = Zbar + (off2[en.y] - w.base);
+    const double *Zb = Zbar + (off2[en.y] - win.base);
     const int fper = nbG * nbE;
     const int ft = max(1, min(pe - p0, SM_BIG / fper));
     for (int ps = p0; ps < pe; ps += ft) {
@@ -171,7 +172,7 @@ __global__ void __launch_bounds__(NT) kb_ZV(const int4 *items, const int64_t *pt
         const double *zr = Zb + (int64_t)(ps + pp) * nbB * nbE + l;
         double f = 0.0;
         for (int j = 0; j < nbB; j++) f = fma(Dbg[j * nbG + k], zr[j * nbE], f);
-        sm[el] = 0.5 * f;
+        sm[el] = w * f;
       }
       __syncthreads();
 #pragma unroll
@@ -207,8 +208,8 @@ __global__ void __launch_bounds__(NT) kb_ZC(const int4 *items, const int64_t *pt
                                             const double *__restrict__ V, const int64_t *offV,
                                             const double *__restrict__ D, const int64_t *offD,
                                             const uint8_t *keepC, const uint8_t *keepV, const uint8_t *keepD,
-                                            const double *__restrict__ Zbar, const int64_t *off2,
-                                            const int64_t *offC, Win w, double *dC) {
+                                            const uint8_t *wZ, const double *__restrict__ Zbar, const int64_t *off2,
+                                            const int64_t *offC, Win win, double *dC) {
   extern __shared__ double sm[];
   const int4 it = items[blockIdx.x];
   const int p3 = it.x, q0 = it.y;
@@ -223,12 +224,13 @@ __global__ void __launch_bounds__(NT) kb_ZC(const int4 *items, const int64_t *pt
   for (int r = 0; r < MAXE; r++) acc[r] = 0.0;
   for (int64_t x = ptr[p3]; x < ptr[p3 + 1]; x++) {
     const int2 en = L[x];
-    if (!keepD[en.x] || !keepV[en.x] || !in_win(w, en.y)) continue;
+    if (!keepD[en.x] || !keepV[en.x] || !in_win(win, en.y)) continue;
     const int b = pA[en.x];
     const int nbB = nb[b], naB = na[b];
     const double *Dbg = D + offD[en.x];
     const double *Vbg = V + offV[en.x];
-    const double *Zb = Zbar + (off2[en.y] - w.base);
+    const double w = wZ[en.x] == 2 ? 0.5 : 1.0;
+    const double *Zb = Zbar + (off2[en.y] - win.base);
     const int pc = max(1, min(naB, SM_BIG / per));
     for (int P0 = 0; P0 < naB; P0 += pc) {
       const int pn = min(pc, naB - P0);
@@ -239,7 +241,7 @@ __global__ void __launch_bounds__(NT) kb_ZC(const int4 *items, const int64_t *pt
         const double *zr = Zb + (int64_t)(P0 + pp) * nbB * nbE + l;
         double f = 0.0;
         for (int j = 0; j < nbB; j++) f = fma(Dbg[j * nbG + k], zr[j * nbE], f);
-        sm[el] = 0.5 * f;
+        sm[el] = w * f;
       }
       __syncthreads();
 #pragma unroll
@@ -801,14 +803,14 @@ extern "C" rix_status rix_backward(rix_ctx *ctx, const double *D, double gEx, do
     if (dC && ctx->n_itB[3]) {
       kb_ZC<<<(unsigned)ctx->n_itB[3], NT, SM_BIG * 8, st>>>(
           ctx->d_itB[3], ctx->d_ptrBZC, ctx->d_LBZC, ctx->d_pA, ctx->d_pB, ctx->d_nb, ctx->d_na, ctx->d_V,
-          ctx->d_offV, D, ctx->d_offD, ctx->d_keepC, ctx->d_keepV, ctx->d_keepD, ctx->d_Z, ctx->d_off2,
+          ctx->d_offV, D, ctx->d_offD, ctx->d_keepC, ctx->d_keepV, ctx->d_keepD, ctx->d_wZ, ctx->d_Z, ctx->d_off2,
           ctx->d_offC, w, dC);
       if ((s = last_err(ctx, "kb_ZC")) != RIX_OK) return s;
     }
     if (dV && ctx->n_itB[2]) {
       kb_ZV<<<(unsigned)ctx->n_itB[2], NT, SM_BIG * 8, st>>>(
           ctx->d_itB[2], ctx->d_ptrBZV, ctx->d_LBZV, ctx->d_pA, ctx->d_pB, ctx->d_nb, ctx->d_na, ctx->d_C,
-          ctx->d_offC, D, ctx->d_offD, ctx->d_keepC, ctx->d_keepV, ctx->d_keepD, ctx->d_Z, ctx->d_off2,
+          ctx->d_offC, D, ctx->d_offD, ctx->d_keepC, ctx->d_keepV, ctx->d_keepD, ctx->d_wZ, ctx->d_Z, ctx->d_off2,
           ctx->d_offV, w, dV);
       if ((s = last_err(ctx, "kb_ZV")) != RIX_OK) return s;
     }

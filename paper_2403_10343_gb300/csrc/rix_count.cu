@@ -85,42 +85,33 @@ __global__ void k_cnt_X12(int64_t n2, const int64_t *ptr, const rix::X12Entry *L
   add_out(out, 7, t1tc_s);
 }
 
-// Z(B,E') <- D(B,G') V(B,G') C(G',E'): 2 na_B na_G nb_G nb_E + 2 na_B nb_B nb_G nb_E per kept product.
-__global__ void k_cnt_Z(int64_t n2, const int64_t *ptrZ, const int2 *LZ, const int32_t *atomA2,
-                        const int32_t *atomB2, const int32_t *pB, const int32_t *nb, const int32_t *na,
-                        const uint8_t *keepC, const uint8_t *keepV, const uint8_t *keepD, const uint8_t *ztc,
-                        rix::PScreen ps, double *out) {
+// Z(B,E') <- D(B,G') V(B,G') C(G',E'), (G',E') not on-site: 2 na_B na_G nb_G nb_E +
+// 2 na_B nb_B nb_G nb_E per kept product, every pair (B,G') of the grouping (a build that halves
+// term 4 in Z runs one of each two), so the walk is over the pairs and not over the Z list.
+__global__ void k_cnt_Z(int64_t np, const int64_t *row1, const int32_t *pA, const int32_t *pB, const uint8_t *onsite,
+                        const int32_t *nb, const int32_t *na, const uint8_t *keepC, const uint8_t *keepV,
+                        const uint8_t *keepD, const uint8_t *ztc, rix::PScreen ps, double *out) {
   double all = 0.0, tc = 0.0;
-  for (int64_t z = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; z < n2; z += (int64_t)gridDim.x * blockDim.x) {
-    const int b = atomA2[z], e = atomB2[z];
-    for (int64_t x = ptrZ[z]; x < ptrZ[z + 1]; x++) {
-      const int2 en = LZ[x];
-      if (!keepD[en.x] || !keepV[en.x] || !keepC[en.y] || ps.drop3(en.x, en.x, en.y)) continue;
-      const int g = pB[en.x];
-      const double f = 2.0 * na[b] * na[g] * nb[g] * nb[e] + 2.0 * na[b] * nb[b] * nb[g] * nb[e];
-      all += f;
-      if (ztc && ztc[g]) tc += f;
-    }
+  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < np; p += (int64_t)gridDim.x * blockDim.x) {
+    if (!keepD[p] || !keepV[p]) continue;
+    const int b = pA[p], g = pB[p];
+    double f = 0.0;
+    for (int64_t x = row1[g]; x < row1[g + 1]; x++)
+      if (!onsite[x] && keepC[x] && !ps.drop3((int)p, (int)p, (int)x))
+        f += 2.0 * na[b] * nb[g] * nb[pB[x]] * (na[g] + nb[b]);
+    all += f;
+    if (ztc && ztc[g]) tc += f;
   }
   add_out(out, 3, all);
   add_out(out, 8, tc);
 }
 
-// X(A,E') <- C(A,B') Z(B,E'): 2 na_B nb_B nb_A nb_E per product with a kept C.
-__global__ void k_cnt_X34(int64_t nk, const int64_t *ptr, const int2 *L, const int32_t *atomA3,
-                          const int32_t *atomB3, const int32_t *pB, const int32_t *nb, const int32_t *na,
-                          const uint8_t *keepC, const uint8_t *rep3, double *out) {
+// X(A,E') <- C(A,B') Z(B,E'): 2 na_B nb_B nb_A nb_E per product with a kept C, one orientation
+// of each K block; summed per pair (A,B') at setup.
+__global__ void k_cnt_X34(int64_t np, const double *f34, const uint8_t *keepC, double *out) {
   double s = 0.0;
-  for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < nk; x += (int64_t)gridDim.x * blockDim.x) {
-    if (!rep3[x]) continue;  // one orientation per K block
-    const int a = atomA3[x], e = atomB3[x];
-    for (int64_t it = ptr[x]; it < ptr[x + 1]; it++) {
-      const int2 en = L[it];
-      if (!keepC[en.x]) continue;
-      const int b = pB[en.x];
-      s += 2.0 * na[b] * nb[b] * nb[a] * nb[e];
-    }
-  }
+  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < np; p += (int64_t)gridDim.x * blockDim.x)
+    if (keepC[p]) s += f34[p];
   add_out(out, 4, s);
 }
 
@@ -148,7 +139,7 @@ extern "C" rix_status rix_count_flops(rix_ctx *ctx, const double *D, double *flo
   rix_status r = RIX_OK;
   do {
     if (cudaMemsetAsync(d_out, 0, 10 * sizeof(double), st) != cudaSuccess) { r = RIX_ECUDA; break; }
-    const int64_t n2 = ctx->stats.n_pairs2, nk = ctx->stats.n_kblocks;
+    const int64_t n2 = ctx->stats.n_pairs2;
     k_cnt_T<<<grid_for(n2), CNT_THREADS, 0, st>>>(n2, ctx->d_ptrT, ctx->d_LT, ctx->d_atomA2, ctx->d_atomB2,
                                                   ctx->d_pB, ctx->d_nb, ctx->d_na, ctx->d_keepC, ctx->d_keepD,
                                                   ctx->d_ttc, rix_pscreen(ctx), d_out);
@@ -157,12 +148,10 @@ extern "C" rix_status rix_count_flops(rix_ctx *ctx, const double *D, double *flo
     k_cnt_X12<<<grid_for(n2), CNT_THREADS, 0, st>>>(n2, ctx->d_ptrX12, ctx->d_LX12, ctx->d_atomA2,
                                                     ctx->d_atomB2, ctx->d_map2to1, ctx->d_pA, ctx->d_nb, ctx->d_na, ctx->d_keepC, ctx->d_keepV,
                                                     ctx->d_t1tc, ctx->d_rep1, d_out);
-    k_cnt_Z<<<grid_for(n2), CNT_THREADS, 0, st>>>(n2, ctx->d_ptrZ, ctx->d_LZ, ctx->d_atomA2, ctx->d_atomB2,
-                                                  ctx->d_pB, ctx->d_nb, ctx->d_na, ctx->d_keepC, ctx->d_keepV,
-                                                  ctx->d_keepD, ctx->d_ztc, rix_pscreen(ctx), d_out);
-    k_cnt_X34<<<grid_for(nk), CNT_THREADS, 0, st>>>(nk, ctx->d_ptrX34, ctx->d_LX34, ctx->d_atomA3,
-                                                    ctx->d_atomB3, ctx->d_pB, ctx->d_nb, ctx->d_na, ctx->d_keepC,
-                                                    ctx->d_rep3, d_out);
+    k_cnt_Z<<<grid_for(ctx->np), CNT_THREADS, 0, st>>>(ctx->np, ctx->d_row1, ctx->d_pA, ctx->d_pB, ctx->d_onsite,
+                                                       ctx->d_nb, ctx->d_na, ctx->d_keepC, ctx->d_keepV,
+                                                       ctx->d_keepD, ctx->d_ztc, rix_pscreen(ctx), d_out);
+    k_cnt_X34<<<grid_for(ctx->np), CNT_THREADS, 0, st>>>(ctx->np, ctx->d_f34, ctx->d_keepC, d_out);
     if (cudaGetLastError() != cudaSuccess) { r = RIX_ECUDA; break; }
     if (cudaMemcpyAsync(flops, d_out, 10 * sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess) {

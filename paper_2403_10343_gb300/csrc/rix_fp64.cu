@@ -9,6 +9,7 @@
 //   X(A,E')   = 1/2 sum_G' [V(A,E')^T T(A,G')]^{Q on E'} C(G',E')^{Q on E'}   term 1
 //             +     sum_G'!=E' U2(A,G') C(G',E')^{Q on G'}                     term 2
 //   Z(B,E')   = 1/2 sum_G'!=E' [V(B,G') C(G',E')^{Q on G'}] applied to D(B,G') (H = F*D)
+//               (or over the unordered pairs {B,G'}: rix_ctx::z_half)
 //   X(A,E')  +=     sum_B'!=A C(A,B')^{P on B'} Z(B,E')                        term 4
 //   K(A,E',n) = X(A,E',n) + X(E',A,-n)^T
 //
@@ -319,8 +320,9 @@ __global__ void __launch_bounds__(NT) k_X12(const int32_t *ord, const int64_t *p
 }
 
 // ------------------------------------------------------------------ term 4 intermediate
-// Z(B,E')[P][j][l] = 1/2 sum over (pair (B,G'), pair (G',E') not on-site) of
-//   sum_k D(B,G')[j][k] F[P][k][l],  F[P][k][l] = sum_Q V(B,G')[P][Q] C(G',E')[Q on G'][k][l].
+// Z(B,E')[P][j][l] = sum over (pair (B,G'), pair (G',E') not on-site) of
+//   w sum_k D(B,G')[j][k] F[P][k][l],  F[P][k][l] = sum_Q V(B,G')[P][Q] C(G',E')[Q on G'][k][l],
+// w the pair's weight (wZ: 1/2, or 1 for the pairs that stand for both orientations).
 __global__ void __launch_bounds__(NT) k_Z(const int2 *items, const int64_t *ptrZ, const int2 *LZ,
                                           const int32_t *atomA2, const int32_t *atomB2, const int64_t *off2,
                                           const int32_t *pB, const int32_t *nb, const int32_t *na,
@@ -328,7 +330,8 @@ __global__ void __launch_bounds__(NT) k_Z(const int2 *items, const int64_t *ptrZ
                                           const double *__restrict__ V, const int64_t *offV,
                                           const double *__restrict__ D, const int64_t *offD,
                                           const uint8_t *keepC, const uint8_t *keepV, const uint8_t *keepD,
-                                          double *Z, int64_t zbase, int smb, const uint8_t *ztc, PScreen ps) {
+                                          double *Z, int64_t zbase, int smb, const uint8_t *ztc,
+                                          const uint8_t *wZ, PScreen ps) {
   extern __shared__ double sm[];
   const int tid = threadIdx.x;
   const int2 it = items[blockIdx.x];
@@ -351,6 +354,7 @@ __global__ void __launch_bounds__(NT) k_Z(const int2 *items, const int64_t *ptrZ
     const double *Dbg = D + offD[en.x];
     const double *Vbg = V + offV[en.x];
     const double *Cge = C + offC[en.y];
+    const double w = wZ[en.x] == 2 ? 0.5 : 1.0;
     const int fper = nbG * nbE;
     const int ft = max(1, min(pe - p0, smb / fper));
     for (int ps = p0; ps < pe; ps += ft) {
@@ -361,7 +365,7 @@ __global__ void __launch_bounds__(NT) k_Z(const int2 *items, const int64_t *ptrZ
         const double *vr = Vbg + (int64_t)(ps + pp) * naG;
         double f = 0.0;
         for (int Q = 0; Q < naG; Q++) f = fma(__ldg(vr + Q), __ldg(Cge + (int64_t)Q * fper + c), f);
-        sm[el] = f;
+        sm[el] = w * f;
       }
       __syncthreads();
 #pragma unroll
@@ -387,7 +391,7 @@ __global__ void __launch_bounds__(NT) k_Z(const int2 *items, const int64_t *ptrZ
 #pragma unroll
   for (int r = 0; r < MAXE; r++) {
     const int el = tid + r * NT;
-    if (el < nel) out[el] = 0.5 * acc[r];
+    if (el < nel) out[el] = acc[r];
   }
 }
 
@@ -403,8 +407,9 @@ __global__ void __launch_bounds__(NT) k_X34(const int32_t *ord, const int64_t *p
   extern __shared__ double sm[];
   const int tid = threadIdx.x;
   const int x = ord[blockIdx.x];
-  // one orientation of each K block (the transpose partner carries the other), with
-  // twice the weight of Z's 1/2; the self block keeps it
+  // term 4 halved in the K blocks: one orientation of each (the transpose partner carries
+  // the other), with twice the weight of Z's 1/2; the self block keeps it.  Halved in Z
+  // (rep3 = 2 everywhere): every block with weight 1.
   const uint8_t r3 = rep3[x];
   if (!r3) return;
   const double w4 = r3 == 2 ? 1.0 : 2.0;
@@ -612,7 +617,7 @@ rix_status launch_Z_items(rix_ctx *ctx, const double *D, int b, int64_t first, i
                                             ctx->d_atomA2, ctx->d_atomB2, ctx->d_off2, ctx->d_pB, ctx->d_nb,
                                             ctx->d_na, ctx->d_C, ctx->d_offC, ctx->d_V, ctx->d_offV, D, ctx->d_offD,
                                             ctx->d_keepC, ctx->d_keepV, ctx->d_keepD, ctx->d_Z, ctx->blk_base[b],
-                                            smb, ctx->have_mx ? ctx->d_ztc : nullptr, rix_pscreen(ctx));
+                                            smb, ctx->have_mx ? ctx->d_ztc : nullptr, ctx->d_wZ, rix_pscreen(ctx));
   return last(ctx, "k_Z");
 }
 

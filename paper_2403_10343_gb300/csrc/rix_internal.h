@@ -133,11 +133,18 @@ struct rix_ctx {
   // with weight 1/2 (on-site pair), 0 = left to the transpose partner
   std::vector<uint8_t> rep1;
   uint8_t *d_rep1 = nullptr;
-  // the same for term 4 per K block (A, E', n) of the 3-hop pattern: 1 = computed with
-  // twice the weight of the four-term grouping, 2 = the self block (A, A, 0), weight as
-  // in the grouping, 0 = left to the transpose partner
-  std::vector<uint8_t> rep3;
-  uint8_t *d_rep3 = nullptr;
+  // Term 4 is symmetric as well, and the build evaluates half of it in one of two ways
+  // (z_half, chosen at setup by the estimated cost of both):
+  //   z_half = false: Z sums over every pair (B, G') with weight 1/2, and X takes the K
+  //     blocks (A, E', n) in one orientation with twice that weight;
+  //   z_half = true: Z sums over the unordered pairs {B, G'} with weight 1 (1/2 on-site),
+  //     and X takes every K block.
+  // rep3 per K block: 1 = weight 2, 2 = weight 1, 0 = left to the transpose partner; wZ per
+  // pair (B, G'): 1 = weight 1, 2 = weight 1/2, 0 = left to the partner pair.
+  bool z_half = false;
+  std::vector<uint8_t> rep3, wZ;
+  uint8_t *d_rep3 = nullptr, *d_wZ = nullptr;
+  double *d_f34 = nullptr;             // per pair (A, B'): FLOPs of its terms-3+4 products (rix_count_flops)
   int64_t *d_offC = nullptr, *d_offV = nullptr, *d_offD = nullptr, *d_offU = nullptr;
   int32_t *d_map1to2 = nullptr, *d_map1to3 = nullptr;
   // 2-hop and 3-hop lists
@@ -185,7 +192,6 @@ struct rix_ctx {
   bool fwd_valid = false;
   // mixed precision: terms 3+4 and term 2 as batched sliced GEMMs on the tensor cores
   bool have_mx = false;
-  int32_t mx_S = 5;
   struct rix_mx_plan *mx34 = nullptr, *mx2 = nullptr;
   struct rix_t1_plan *mx1 = nullptr;           // term 1 for the column atoms where it pays
   struct rix_mx_plan *mxz = nullptr;            // term-4 intermediate for the middle atoms where it pays
@@ -270,6 +276,7 @@ inline rix_status rix_upload(rix_ctx *ctx, T **p, const std::vector<T> &v) {
 
 // mixed precision (rix_tc.cu)
 rix_status rix_mixed_plan(rix_ctx *ctx, const std::vector<int64_t> &ptrZ);
+int rix_plan_slices(const rix_ctx *ctx, int kind);  // slices of the mixed plans of a kind
 int64_t rix_mixed_bytes(rix_ctx *ctx, const std::vector<int64_t> &ptrZ);
 rix_status rix_mixed_x34(rix_ctx *ctx, int blk, int64_t zbase, cudaStream_t st);
 rix_status rix_mixed_z(rix_ctx *ctx, int blk, int64_t zbase, const double *D, cudaStream_t st);

@@ -281,6 +281,66 @@ static rix_status build_backward_lists(rix_ctx *ctx, const std::vector<int2> &LT
   return RIX_OK;
 }
 
+// Which half of term 4 the build evaluates (rix_ctx::z_half) and the pair weights wZ.
+// Both forms cost one stage in full and the other in half; the estimates below count
+// every product of the lists (D, which screens Z, is not known yet).  FP64: the FLOPs of
+// the two stages.  Mixed: the sliced products, Z as Kronecker rows (na nb per row atom and
+// nb_B na_G nb_G per column), which makes Z the larger one by far except where few
+// atoms lie within the cutoff.  (GB300, mixed, start and with Z halved: (H2O)64 cluster 169.3 and
+// 123.0 ms, 192-atom ice cell 379 and 330 ms, 12-atom perovskite 239 and 210 ms.  FP64: the 24-atom
+// ice cell, whose K blocks outweigh Z (245 and 31 ms), stays with the halved K blocks.)
+static void choose_term4(rix_ctx *ctx) {
+  const int nat = ctx->nat;
+  const bool mixed = ctx->opt.precision == RIX_MIXED_BF16;
+  std::vector<double> sE(nat, 0.0), s2(nat, 0.0);
+  for (int64_t p = 0; p < ctx->np; p++)
+    if (!ctx->onsite[p]) sE[ctx->pA[p]] += ctx->nb_at[ctx->pB[p]];
+  for (int64_t z = 0; z < ctx->n2; z++) s2[key_a(ctx->keys2[z])] += ctx->nb_at[key_b(ctx->keys2[z])];
+  auto fz = [&](int64_t p) {  // FP64 FLOPs of the Z products of pair (B, G')
+    const double naB = ctx->na_at[ctx->pA[p]], nbB = ctx->nb_at[ctx->pA[p]];
+    const double naG = ctx->na_at[ctx->pB[p]], nbG = ctx->nb_at[ctx->pB[p]];
+    return 2.0 * naB * nbG * (naG + nbB) * sE[ctx->pB[p]];
+  };
+  ctx->wZ.assign(ctx->np, 0);
+  double z_all = 0, z_rep = 0, zk_all = 0, zk_rep = 0, x_all = 0;
+  for (int64_t p = 0; p < ctx->np; p++) {
+    const int b = ctx->pA[p], g = ctx->pB[p];
+    // one pair of {(B, G'), (G', B)}: in FP64 the one that applies V from the side that
+    // costs less; index order in the mixed plans, which keeps molecules together
+    bool rep = ctx->rep1[p] != 0;
+    if (!mixed && !ctx->onsite[p]) {
+      const double f = fz(p), fq = fz(ctx->partner1[p]);
+      if (f != fq) rep = f < fq;
+    }
+    ctx->wZ[p] = ctx->onsite[p] ? 2 : rep ? 1 : 0;
+    const double zk = 2.0 * ctx->na_at[b] * ctx->nb_at[b] * ctx->na_at[g] * ctx->nb_at[g] * sE[g];
+    z_all += fz(p);
+    zk_all += zk;
+    if (ctx->wZ[p]) {
+      z_rep += fz(p);
+      zk_rep += zk;
+    }
+  }
+  for (int a = 0; a < nat; a++) x_all += 2.0 * ctx->na_at[a] * ctx->nb_at[a] * sE[a] * s2[a];
+  double full, half;  // costs with Z in full, with Z halved
+  if (mixed && !ctx->opt.deterministic) {
+    const int S = rix_plan_slices(ctx, 0), R = rix_plan_slices(ctx, 2);
+    const double px = 0.5 * S * (S + 1), pz = 0.5 * R * (R + 1);
+    full = zk_all * pz + 0.5 * x_all * px;
+    half = zk_rep * pz + x_all * px;
+  } else if (mixed) {  // deterministic: Z on the FP64 pipe, ~600 times slower per FLOP than a sliced product
+    const int S = rix_plan_slices(ctx, 0);
+    const double px = 0.5 * S * (S + 1) / 600.0;
+    full = z_all + 0.5 * x_all * px;
+    half = z_rep + x_all * px;
+  } else {
+    full = z_all + 0.5 * x_all;
+    half = z_rep + x_all;
+  }
+  ctx->z_half = half < full;
+  if (!ctx->z_half) ctx->wZ.assign(ctx->np, 2);
+}
+
 static rix_status build_lists(rix_ctx *ctx) {
   const int nat = ctx->nat;
   const int64_t np = ctx->np;
@@ -373,15 +433,14 @@ static rix_status build_lists(rix_ctx *ctx) {
     return RIX_EINVAL;
   }
   for (int64_t x = 0; x < nk; x++) ctx->offK[x + 1] = ctx->offK[x] + szk[x];
-  // Term 4 (like term 1) is symmetric under (A, E', n) -> (E', A, -n) with
-  // transposition: it is computed for one orientation of each K block (twice the 1/2
-  // of the grouping), the self block (A, A, 0) being its own partner.
-  ctx->rep3.assign(nk, 0);
+  // K blocks in their representative orientation (1; 2 = the self block, its own
+  // partner): the ones that take term 4, and its FLOP count, when it is halved there.
+  std::vector<uint8_t> rep3c(nk, 0);
   for (int64_t x = 0; x < nk; x++) {
     const int a = key_a(keys3[x]), e = key_b(keys3[x]);
     const int n0 = key_n(keys3[x], 0), n1 = key_n(keys3[x], 1), n2 = key_n(keys3[x], 2);
     const bool pos = n0 > 0 || (n0 == 0 && (n1 > 0 || (n1 == 0 && n2 > 0)));
-    ctx->rep3[x] = partner3[x] == x ? 2 : (a < e || (a == e && pos)) ? 1 : 0;
+    rep3c[x] = partner3[x] == x ? 2 : (a < e || (a == e && pos)) ? 1 : 0;
   }
   std::vector<int32_t> map1to2(np), map1to3(np);
   std::vector<int64_t> offU(np + 1, 0);
@@ -497,9 +556,18 @@ static rix_status build_lists(rix_ctx *ctx) {
   ptrX12[n2] = baseX[nat];
   for (int64_t p = 0; p < np; p++) flU2 += 2.0 * NA(pA[p]) * NA(pB[p]) * NB(pA[p]) * NB(pB[p]);
 
+  // ---------------------------------------------------------------- term 4: which half
+  choose_term4(ctx);
+  ctx->rep3.assign(nk, 2);
+  if (!ctx->z_half) ctx->rep3 = rep3c;
+
   // ---------------------------------------------------------------- Z list (term 4): Z(B,E') <- (pair (B,G'), pair (G',E'))
   // and the X34 list: X(A,E') <- (C(A,B') not on-site, Z(B,E'-n1)).  Z blocks that no
-  // product reaches (possible only without neighbours) are left out of the X34 list.
+  // product reaches are left out of the X34 list.  The FLOP counts are those of the
+  // grouping (every Z product, one orientation of each K block), whichever half runs;
+  // f34 splits the latter by the pair (A, B').
+  std::vector<uint8_t> reach(n2, 0);   // Z blocks that a product of either orientation reaches
+  std::vector<double> f34(np, 0.0);
   std::vector<std::vector<int2>> lz(nat), lxx(nat);
   std::vector<std::vector<int64_t>> lzp(nat), lxp(nat);
   double flZ = 0, flX34 = 0;
@@ -513,8 +581,12 @@ static rix_status build_lists(rix_ctx *ctx) {
       for (int64_t p3 = row1[g]; p3 < row1[g + 1]; p3++) {
         if (ctx->onsite[p3]) continue;
         int e = pB[p3];
-        key.push_back(find2(key_add(b, e, &pn[3 * p2], &pn[3 * p3], &lok)));
-        pay.push_back(make_int2((int)p2, (int)p3));
+        const int64_t z = find2(key_add(b, e, &pn[3 * p2], &pn[3 * p3], &lok));
+        reach[z] = 1;
+        if (ctx->wZ[p2]) {
+          key.push_back(z);
+          pay.push_back(make_int2((int)p2, (int)p3));
+        }
         flZ += 2.0 * NA(b) * NA(g) * NB(g) * NB(e) + 2.0 * NA(b) * NB(b) * NB(g) * NB(e);
       }
     }
@@ -549,15 +621,17 @@ static rix_status build_lists(rix_ctx *ctx) {
       if (ctx->onsite[p1]) continue;
       int b = pB[p1];
       for (int64_t z = row2[b]; z < row2[b + 1]; z++) {
-        if (ptrZ[z + 1] == ptrZ[z]) continue;
+        if (!reach[z]) continue;
         int e = key_b(keys2[z]);
         int8_t m[3];
         decode_n(keys2[z], m);
         const int64_t x3 = find3(key_add(a, e, &pn[3 * p1], m, &lok));
+        if (rep3c[x3]) f34[p1] += 2.0 * NA(b) * NB(b) * NB(a) * NB(e);  // one orientation
+        if (ptrZ[z + 1] == ptrZ[z]) continue;
         key.push_back(x3);
         pay.push_back(make_int2((int)p1, (int)z));
-        if (x3 >= 0 && ctx->rep3[x3]) flX34 += 2.0 * NA(b) * NB(b) * NB(a) * NB(e);  // one orientation
       }
+      flX34 += f34[p1];
     }
     std::vector<int64_t> rel(row3[a + 1] - row3[a] + 1);
     lxx[a].resize(key.size());
@@ -696,6 +770,8 @@ static rix_status build_lists(rix_ctx *ctx) {
   TRY(rix_upload(ctx, &ctx->d_map2to3, map2to3));
   TRY(rix_upload(ctx, &ctx->d_atomA3, atomA3));
   TRY(rix_upload(ctx, &ctx->d_rep3, ctx->rep3));
+  TRY(rix_upload(ctx, &ctx->d_wZ, ctx->wZ));
+  TRY(rix_upload(ctx, &ctx->d_f34, f34));
   TRY(rix_upload(ctx, &ctx->d_atomB3, atomB3));
   TRY(rix_upload(ctx, &ctx->d_offK, ctx->offK));
   TRY(rix_upload(ctx, &ctx->d_partner3, partner3));

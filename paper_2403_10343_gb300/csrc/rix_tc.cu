@@ -443,8 +443,9 @@ void launch_pack(const double *X, int64_t sr, int64_t sk, int R, int Kd, int Rpa
 // ------------------------------------------------------------------ the GEMM
 // Middle atoms batched into one problem of the plans of terms 2, 3+4 and Z (at most).
 constexpr int GMAX = 4;
-// xmap entries of the terms-3+4 plan: output block index, with this bit set for the self
-// block (A, A, 0), which takes half the weight of the other blocks
+// xmap entries of the terms-3+4 plan: output block index, with this bit set for the blocks of
+// weight 1 (rep3 = 2), half the plan's weight; Src flags of the Z plan: pair index, with this bit
+// set for the pairs of weight 1/2 beside pairs of weight 1 (on-site pairs when Z is halved)
 constexpr int32_t XHALF = 1 << 30;
 
 // One problem of a batched launch: its packed operands, exponents and the
@@ -998,7 +999,8 @@ extern "C" rix_status rix_test_stalled_gemm(rix_ctx *ctx, int64_t wait_ns, void 
 //     rows (A', i) over G's neighbours (U2 of the pair (A', G)), K = (Q, k),
 //     columns (E', l) over G's neighbours E' != G;
 //   term 4 intermediate (middle atom G, rows of one block):
-//     Z(B,E')[P][j][l] += 1/2 sum_{Q on G, k} V(B,G')[P][Q] D(B,G')[j][k] C(G',E')[Q on G][k][l]
+//     Z(B,E')[P][j][l] += w sum_{Q on G, k} V(B,G')[P][Q] D(B,G')[j][k] C(G',E')[Q on G][k][l]
+//       (w = 1/2 over all B, or 1 over one pair of each {B, G'}: rix_ctx::z_half);
 //     rows (B, P, j), K = (Q, k), columns (E', l) as for term 2.  The row
 //     operand is the Kronecker product of the V and D blocks, formed while
 //     slicing; this costs about nb_B times the FLOPs of the FP64 grouping, so a
@@ -1012,7 +1014,7 @@ namespace rixtc {
 // One packed row (A operand) or column (B operand): element k < K of it is
 //   X[off - shift + o * outer + in * inner_st] * (off2 < 0 ? 1 : X2[off2 + in]),
 // o = k / inner_n, in = k % inner_n.  off < 0 marks padding; flag >= 0 zeroes
-// the row unless keep[flag] (and keep2[flag] when given).
+// the row unless keep[flag] (and keep2[flag] when given); XHALF in flag halves the element.
 struct Src {
   int64_t off, off2;
   int32_t outer, inner_st, inner_n, flag;
@@ -1173,11 +1175,13 @@ struct SrcAcc {
     const int m = (k >= R.pr.kb[1]) + (k >= R.pr.kb[2]) + (k >= R.pr.kb[3]);
     const int k0 = m == 0 ? 0 : m == 1 ? R.pr.kb[1] : m == 2 ? R.pr.kb[2] : R.pr.kb[3];
     const Src sr = R.s[m];
-    if (sr.off < 0 || (sr.flag >= 0 && !(keep[sr.flag] && (!keep2 || keep2[sr.flag])))) return 0.0;
+    const int f = sr.flag & ~XHALF;
+    if (sr.off < 0 || (sr.flag >= 0 && !(keep[f] && (!keep2 || keep2[f])))) return 0.0;
     const int kl = k - k0;
     const int o = kl / sr.inner_n, in = kl - o * sr.inner_n;
     const double v = X[sr.off - shift + (int64_t)o * sr.outer + (int64_t)in * sr.inner_st];
-    return sr.off2 >= 0 ? v * X2[sr.off2 + in] : v;
+    if (sr.off2 < 0) return v;
+    return sr.flag & XHALF ? 0.5 * (v * X2[sr.off2 + in]) : v * X2[sr.off2 + in];
   }
 };
 
@@ -1194,14 +1198,15 @@ __global__ void k_kron_exp(int64_t n0, int64_t n, SrcAcc acc, int *e) {
   int m = -2000;
   for (int k = 0; k < R.pr.ng; k++) {
     const Src sr = R.s[k];
-    if (sr.off < 0 || (sr.flag >= 0 && !(acc.keep[sr.flag] && (!acc.keep2 || acc.keep2[sr.flag])))) continue;
+    const int f = sr.flag & ~XHALF;
+    if (sr.off < 0 || (sr.flag >= 0 && !(acc.keep[f] && (!acc.keep2 || acc.keep2[f])))) continue;
     const int kn = (k == 0 ? R.pr.kb[1] : k == 1 ? R.pr.kb[2] - R.pr.kb[1] : k == 2 ? R.pr.kb[3] - R.pr.kb[2]
                                                                                    : R.pr.kb[4] - R.pr.kb[3]);
     const int nq = kn / sr.inner_n;
     double mv = 0.0, md = 0.0;
     for (int q = 0; q < nq; q++) mv = fmax(mv, fabs(acc.X[sr.off - acc.shift + (int64_t)q * sr.outer]));
     for (int i = 0; i < sr.inner_n; i++) md = fmax(md, fabs(acc.X2[sr.off2 + i]));
-    m = max(m, exp_of(mv * md));
+    m = max(m, exp_of(sr.flag & XHALF ? 0.5 * (mv * md) : mv * md));
   }
   e[R.pr.eaoff + R.r] = m;
 }
@@ -1336,14 +1341,21 @@ struct PlanHost {
 
 }  // namespace
 
+// Slices per operand when rix_options.n_slices is 0: with balanced digits five
+// slices (six for the regrouped plans) keep the mixed build within 1e-8 in K and
+// 1e-6 Ha in E_x on the water, ice and perovskite workloads measured (largest
+// difference 1.1e-7 Ha, the 1,536-atom perovskite).
+constexpr int DEFAULT_SLICES = 5;
+
 // Slices per plan: the regrouped forms (term 1 as T x C, Z with Kronecker rows)
 // sum many more products of widely ranging size per output than the FP64
 // grouping, and T feeds every term, so these take one slice more than the
 // GEMMs of terms 2-4 (capped at 8).
 int rix_plan_slices(const rix_ctx *ctx, int kind) {
-  if (kind < 2) return ctx->mx_S;
+  const int S = ctx->opt.n_slices > 0 ? ctx->opt.n_slices : DEFAULT_SLICES;
+  if (kind < 2) return S;
   const int r = ctx->opt.n_slices_regrouped;
-  return r > 0 ? std::min(r, (int)rixtc::MAXS) : std::min(ctx->mx_S + 1, (int)rixtc::MAXS);
+  return r > 0 ? std::min(r, (int)rixtc::MAXS) : std::min(S + 1, (int)rixtc::MAXS);
 }
 
 namespace {
@@ -1377,11 +1389,15 @@ rix_status plan_host(rix_ctx *ctx, int kind, const std::vector<int64_t> &ptrZ, P
   h.use.assign(nat, kind == 2 ? 0 : 1);
   if (kind == 2) {
     for (int g = 0; g < nat; g++) {
-      double sB1 = 0, sB2 = 0, sE = 0, M = 0;
+      double sB1 = 0, sB2 = 0, sE = 0, M = 0, a1 = 0, a2 = 0;
       for (int64_t q = row1[g]; q < row1[g + 1]; q++) {
         const int b = ctx->pB[q];
-        sB1 += ctx->na_at[b];
-        sB2 += (double)ctx->na_at[b] * ctx->nb_at[b];
+        a1 += ctx->na_at[b];
+        a2 += (double)ctx->na_at[b] * ctx->nb_at[b];
+        if (ctx->wZ[ctx->partner1[q]]) {  // the pairs (B, G') that run
+          sB1 += ctx->na_at[b];
+          sB2 += (double)ctx->na_at[b] * ctx->nb_at[b];
+        }
         if (!ctx->onsite[q]) sE += ctx->nb_at[b];
       }
       M = sB2;
@@ -1394,7 +1410,7 @@ rix_status plan_host(rix_ctx *ctx, int kind, const std::vector<int64_t> &ptrZ, P
       // contributions of many middle atoms, which the tensor-core plan does with atomics)
       if (sE > 0 && tc / TC_RATE < f64 / FP64_RATE_Z && !ctx->opt.deterministic) {
         h.use[g] = 1;
-        h.fl64 += f64;
+        h.fl64 += 2.0 * a1 * naG * nbG * sE + 2.0 * a2 * nbG * sE;  // of the grouping, every pair (B, G')
       }
     }
   }
@@ -1486,6 +1502,7 @@ rix_status plan_host(rix_ctx *ctx, int kind, const std::vector<int64_t> &ptrZ, P
         for (int64_t q = row1[b]; q < row1[b + 1]; q++) {
           if (kind == 0 && ctx->onsite[q]) continue;
           if (kind == 2 && mblk[ctx->pB[q]] != blk && nblk > 1) continue;
+          if (kind == 2 && !ctx->wZ[ctx->partner1[q]]) continue;  // left to the pair (G', B)
           int M[3];
           for (int c = 0; c < 3; c++) M[c] = ctx->pn[3 * q + c] + gm[k].o[c];
           slot(rm, node_key(ctx->pB[q], M))[k] = q;
@@ -1596,6 +1613,7 @@ rix_status plan_host(rix_ctx *ctx, int kind, const std::vector<int64_t> &ptrZ, P
             if (kind == 2) {  // rows (P, j) of V(B,G')[P][.] x D(B,G')[j][.]
               const int P = y / nbA, j = y - P * nbA;
               sr = Src{ctx->offV[pq] + (int64_t)P * naB, ctx->offD[pq] + (int64_t)j * nbB, 1, 0, nbB, (int32_t)pq};
+              if (ctx->z_half && ctx->wZ[pq] == 2) sr.flag |= XHALF;
             } else if (kind == 0) {  // C(A,B)[naA + P][i][j]
               sr = Src{ctx->offC[pq] + ((int64_t)naA * nbA + y) * nbB, -1, nbA * nbB, 1, nbB, (int32_t)pq};
             } else {  // U2(A,G)[Q][i][k]
@@ -1709,15 +1727,8 @@ int64_t group_budget(int64_t maxp, int64_t total) {
 
 }  // namespace
 
-// Slices per operand when rix_options.n_slices is 0: with balanced digits five
-// slices (six for the regrouped plans) keep the mixed build within 1e-8 in K and
-// 1e-6 Ha in E_x on the water, ice and perovskite workloads measured (largest
-// difference 1.1e-7 Ha, the 1,536-atom perovskite).
-constexpr int DEFAULT_SLICES = 5;
-
 // Device bytes the mixed-precision plans will need (their maps plus one slice buffer).
 int64_t rix_mixed_bytes(rix_ctx *ctx, const std::vector<int64_t> &ptrZ) {
-  ctx->mx_S = ctx->opt.n_slices > 0 ? ctx->opt.n_slices : DEFAULT_SLICES;
   int64_t maps = 0, buf = 0;
   {
     int64_t t1 = 0, tt = 0;
@@ -1738,11 +1749,6 @@ int64_t rix_mixed_bytes(rix_ctx *ctx, const std::vector<int64_t> &ptrZ) {
 
 rix_status rix_mixed_plan(rix_ctx *ctx, const std::vector<int64_t> &ptrZ) {
   using namespace rixtc;
-  ctx->mx_S = ctx->opt.n_slices > 0 ? ctx->opt.n_slices : DEFAULT_SLICES;
-  if (ctx->mx_S > MAXS) {
-    ctx->last_error = "n_slices above 8";
-    return RIX_EINVAL;
-  }
   int64_t buf = 0;
   double tflops = 0;
   for (int kind = 0; kind < 3; kind++) {
@@ -2013,7 +2019,7 @@ rix_status rix_mixed_x34(rix_ctx *ctx, int blk, int64_t zbase, cudaStream_t st) 
   rt_masks(ctx, pl, ctx->d_keepC, nullptr, false, st);
   for (size_t g = 0; g + 1 < pl->grp.size(); g++) {
     if (pl->grp_blk[g] != blk) continue;
-    // weight 2: term 4 in one orientation of each K block (Z carries the grouping's 1/2)
+    // weight 2 (1 for the blocks marked XHALF): see rix_ctx::z_half
     rix_status s = run_group(ctx, pl, g, rows, cols, ctx->d_offK, ctx->d_X, 0, 2.0, st);
     if (s != RIX_OK) return s;
   }
@@ -2044,7 +2050,7 @@ rix_status rix_mixed_z(rix_ctx *ctx, int blk, int64_t zbase, const double *D, cu
   rt_masks(ctx, pl, ctx->d_keepV, ctx->d_keepD, true, st);
   for (size_t g = 0; g + 1 < pl->grp.size(); g++) {
     if (pl->grp_blk[g] != blk) continue;
-    rix_status s = run_group(ctx, pl, g, rows, cols, ctx->d_off2, ctx->d_Z, zbase, 0.5, st);
+    rix_status s = run_group(ctx, pl, g, rows, cols, ctx->d_off2, ctx->d_Z, zbase, ctx->z_half ? 1.0 : 0.5, st);
     if (s != RIX_OK) return s;
   }
   return RIX_OK;
