@@ -9,7 +9,7 @@
 //   X(A,E')   = 1/2 sum_G' [V(A,E')^T T(A,G')]^{Q on E'} C(G',E')^{Q on E'}   term 1
 //             +     sum_G'!=E' U2(A,G') C(G',E')^{Q on G'}                     term 2
 //   Z(B,E')   = 1/2 sum_G'!=E' [V(B,G') C(G',E')^{Q on G'}] applied to D(B,G') (H = F*D)
-//               (or over the unordered pairs {B,G'}: rix_ctx::z_half)
+//               (or over the unordered pairs {B,G'}: rix_ctx::wZ)
 //   X(A,E')  +=     sum_B'!=A C(A,B')^{P on B'} Z(B,E')                        term 4
 //   K(A,E',n) = X(A,E',n) + X(E',A,-n)^T
 //
@@ -20,6 +20,8 @@
 // Each kernel is output-stationary: one CTA owns an output block (or a row
 // tile of it), walks its product list and keeps the sums in registers, so no
 // atomics are needed and every run sums in the same order.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cstdio>
 #include <string>
@@ -27,12 +29,14 @@
 #include "rix_internal.h"
 
 using namespace rix;
+namespace cg = cooperative_groups;
 
 namespace {
 
 constexpr int NT = 256;      // threads per CTA
-constexpr int MAXE = 32;     // output elements per thread in tiled kernels (NT * MAXE = 8192)
-constexpr int XMAXE = 16;    // output elements per thread for K blocks (64 x 64 / 256)
+constexpr int MAXE = 32;     // output elements per thread in tiled kernels
+static_assert(NT * MAXE == CAP_MAX, "row tiles");
+constexpr int XMAXE = 16;    // output elements per thread for K blocks above 256 elements (64 x 64 / 256)
 constexpr int SM_MAX = 16384;  // largest shared-memory tile budget in doubles (128 KB)
 
 // ------------------------------------------------------------------ pair list (a1)
@@ -155,7 +159,7 @@ __global__ void __launch_bounds__(NT) k_T(const int2 *items, const int64_t *ptrT
                                           const double *__restrict__ C, const int64_t *offC,
                                           const double *__restrict__ D, const int64_t *offD,
                                           const uint8_t *keepC, const uint8_t *keepD, double *T,
-                                          int64_t tbase, const uint8_t *ttc, PScreen ps) {
+                                          int64_t tbase, const uint8_t *ttc, int cap, PScreen ps) {
   extern __shared__ double sm[];
   const int tid = threadIdx.x;
   const int2 it = items[blockIdx.x];
@@ -164,7 +168,7 @@ __global__ void __launch_bounds__(NT) k_T(const int2 *items, const int64_t *ptrT
   if (ttc && ttc[a]) return;  // this row atom's T comes from the tensor cores
   const int nbA = nb[a], naA = na[a], nbG = nb[g];
   const int per = nbA * nbG;
-  const int pt = max(1, NT * MAXE / per);
+  const int pt = max(1, cap / per);
   const int pe = min(naA, p0 + pt);
   const int nel = (pe - p0) * per;
   double acc[MAXE];
@@ -212,7 +216,7 @@ __global__ void __launch_bounds__(NT) k_U2(const int2 *items, const int32_t *pA,
   const int a = pA[p], g = pB[p];
   const int nbA = nb[a], naA = na[a], nbG = nb[g], naG = na[g];
   const int per = nbA * nbG;
-  const int qt = max(1, NT * MAXE / per);
+  const int qt = max(1, CAP_MIN / per);
   const int qe = min(naG, q0 + qt);
   const int nel = (qe - q0) * per;
   const double *Vb = V + offV[p];
@@ -226,97 +230,252 @@ __global__ void __launch_bounds__(NT) k_U2(const int2 *items, const int32_t *pA,
   }
 }
 
+// ------------------------------------------------------------------ K-block outputs (terms 1+2, terms 3+4)
+// A K block has few elements (196 for a pair of O, 25 for a pair of H) and sums
+// long products, so a CTA splits the contraction and not only the output:
+// thread tid works on element tid % nel in group tid / nel, each group sums its own
+// share of every product, and the shares are added in a fixed order at the end.  Two
+// DFMA per clock and SM leave 64 clocks to a warp instruction, so what counts is
+// that every lane has work and that warps of several CTAs overlap the loads; the
+// products that need no staging run without a barrier.  Where a system has few or very
+// uneven outputs, a cluster of ns CTAs shares one output (the launch classes of rix_ctx).
+// R elements per thread: 1 up to 256 elements, else 16 (and one group).
+// GB300, one group with staged operands and now: (H2O)64 terms 1+2 652 and 309 ms (1.14 TFLOP/s
+// of the products it keeps, FP64 pipe 1.25), 24-atom ice cell terms 3+4 245 and 115 ms (1.13);
+// (H2O)8, split over 2^c CTAs, terms 1+2 5.34 and 1.99 ms.
+struct Split {
+  int ng, grp, el0;  // groups of the CTA, this thread's group (ng: no work) and first element
+  int part, parts;   // share of this thread's group among the shares of the whole cluster
+};
+
+template <int R>
+__device__ __forceinline__ Split split_of(int nel, int rank, int ns) {
+  Split s;
+  s.ng = R == 1 ? NT / nel : 1;
+  s.grp = R == 1 ? (int)threadIdx.x / nel : 0;
+  s.el0 = R == 1 ? (int)threadIdx.x - s.grp * nel : (int)threadIdx.x;
+  s.part = rank * s.ng + s.grp;
+  s.parts = ns * s.ng;
+  return s;
+}
+
+// acc[r] += sum over this share of the rows (P, j) of a[P][i][j] b[P][j][l] (a: nP x nbA x nbJ,
+// b: nP x nbJ x nbE); element el = i nbE + l.
+template <int R>
+__device__ __forceinline__ void dot_share(double (&acc)[R], const Split &s, int nel, const double *__restrict__ a,
+                                          const double *__restrict__ b, int nP, int nbA, int nbJ, int nbE) {
+  if (s.grp >= s.ng) return;
+  const int K = nP * nbJ;
+  const int k0 = (int)((int64_t)K * s.part / s.parts), k1 = (int)((int64_t)K * (s.part + 1) / s.parts);
+  const int P0 = k0 / nbJ, j0 = k0 - P0 * nbJ;
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    const int el = s.el0 + r * NT;
+    if (el < nel) {
+      const int i = el / nbE, l = el - i * nbE;
+      const double *ap = a + ((int64_t)P0 * nbA + i) * nbJ + j0;
+      const double *bp = b + (int64_t)k0 * nbE + l;
+      double v = acc[r];
+      int j = j0;
+#pragma unroll 4
+      for (int k = k0; k < k1; k++) {
+        v = fma(__ldg(ap), __ldg(bp), v);
+        bp += nbE;
+        ap++;
+        if (++j == nbJ) {  // the next P: same row i
+          j = 0;
+          ap += (nbA - 1) * nbJ;
+        }
+      }
+      acc[r] = v;
+    }
+  }
+}
+
+// The sum of all shares of a cluster's output, in rank 0: groups first, then ranks.
+// red: NT (R == 1) or nel doubles of shared memory.
+template <int R, class F>
+__device__ __forceinline__ void gather_shares(double (&acc)[R], const Split &s, int nel, int ns, double *red, F store) {
+  if (R == 1 && s.ng > 1) {
+    __syncthreads();
+    red[threadIdx.x] = acc[0];
+    __syncthreads();
+    if ((int)threadIdx.x < nel) {
+      double v = acc[0];
+      for (int g = 1; g < s.ng; g++) v += red[g * nel + threadIdx.x];
+      acc[0] = v;
+    }
+  }
+  if (ns > 1) {
+    cg::cluster_group cl = cg::this_cluster();
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      const int el = threadIdx.x + r * NT;
+      if (el < nel) red[el] = acc[r];
+    }
+    cl.sync();
+    if (cl.block_rank() == 0) {
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        const int el = threadIdx.x + r * NT;
+        if (el < nel)
+          for (int q = 1; q < ns; q++) acc[r] += cl.map_shared_rank(red, q)[el];
+      }
+    }
+    cl.sync();
+    if (cl.block_rank() != 0) return;
+  }
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    const int el = threadIdx.x + r * NT;
+    if (el < nel) store(el, acc[r]);
+  }
+}
+
 // ------------------------------------------------------------------ terms 1 and 2
-__global__ void __launch_bounds__(NT) k_X12(const int32_t *ord, const int64_t *ptr, const X12Entry *L,
-                                            const int32_t *atomA2, const int32_t *atomB2,
-                                            const int32_t *map2to1, const int32_t *map2to3,
-                                            const int32_t *pA, const uint8_t *onsite, const int32_t *nb,
-                                            const int32_t *na, const double *__restrict__ C,
-                                            const int64_t *offC, const double *__restrict__ V,
-                                            const int64_t *offV, const uint8_t *keepC, const uint8_t *keepV,
-                                            const double *__restrict__ T, const int64_t *off2,
-                                            const double *__restrict__ U, const int64_t *offU,
-                                            const int64_t *offK, double *X, int64_t tbase, int smb, int t2,
-                                            const uint8_t *t1tc, const uint8_t *rep1) {
+// Term 1, U1[Q][i][k] = sum_P V(A,E')[P][Q] T(A,G')[P][i][k] (Q on E') and X += U1 C(G',E'), takes
+// the columns (G', k) of several entries at once: a table of the columns' T and C offsets, U1 of a
+// few Q over all of them in shared memory (full warps whatever the species), then the split product.
+// Term 2 is a split product per entry.
+constexpr int XCOL = 192;    // columns of a batch at most
+constexpr int XENT = 32;     // entries of a batch at most (one warp builds the table)
+struct XCols {
+  int64_t t[XCOL], c[XCOL];  // offsets of T(A,G')[0][0][k] and C(G',E')[Q = 0 on E'][k][0]
+  int nb[XCOL];              // nb of G'
+  int n, next;               // columns; first list entry after the batch
+};
+
+// XCols of the list entries from it on that term 1 uses, at most maxcol columns (one warp)
+__device__ __forceinline__ void x12_batch(XCols &tb, int64_t it, int64_t end, int maxcol, const X12Entry *L,
+                                          const uint8_t *keepC, const int32_t *pA, const int32_t *nb,
+                                          const int32_t *na, const uint8_t *onsite, const int64_t *off2,
+                                          int64_t tbase, const int64_t *offC, int nbE) {
+  const int lane = threadIdx.x & 31;
+  const bool in = it + lane < end;
+  const X12Entry en = L[in ? it + lane : it];
+  const int g = pA[en.p3];
+  const int w = in && en.t1 && keepC[en.p3] ? nb[g] : 0;
+  int s = w;  // columns up to and including this entry's
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, s, o);
+    if (lane >= o) s += v;
+  }
+  const unsigned fit = __ballot_sync(0xffffffffu, in && s <= maxcol);
+  const int take = __popc(fit);  // s does not decrease, so the entries that fit come first
+  if (lane < take) {
+    const int64_t t0 = off2[en.t] - tbase, c0 = offC[en.p3] + (int64_t)(onsite[en.p3] ? 0 : na[g]) * w * nbE;
+    for (int k = 0; k < w; k++) {
+      tb.t[s - w + k] = t0 + k;
+      tb.c[s - w + k] = c0 + (int64_t)k * nbE;
+      tb.nb[s - w + k] = w;
+    }
+  }
+  if (lane == take - 1) {
+    tb.n = s;
+    tb.next = take;
+  }
+}
+
+template <int R>
+__global__ void __launch_bounds__(NT, R == 1 ? 4 : 1)
+    k_X12(const int32_t *ord, const int64_t *ptr, const X12Entry *L, const int32_t *atomA2, const int32_t *atomB2,
+          const int32_t *map2to1, const int32_t *map2to3, const int32_t *pA, const uint8_t *onsite, const int32_t *nb,
+          const int32_t *na, const double *__restrict__ C, const int64_t *offC, const double *__restrict__ V,
+          const int64_t *offV, const uint8_t *keepC, const uint8_t *keepV, const double *__restrict__ T,
+          const int64_t *off2, const double *__restrict__ U, const int64_t *offU, const int64_t *offK, double *X,
+          int64_t tbase, int smb, int t2, const uint8_t *t1tc, const uint8_t *rep1, int ns) {
   extern __shared__ double sm[];
+  __shared__ XCols tb;
   const int tid = threadIdx.x;
-  const int s = ord[blockIdx.x];
+  const int s = ord[blockIdx.x / ns];
+  const int rank = blockIdx.x % ns;
   const int a = atomA2[s], e = atomB2[s];
   const int nbA = nb[a], naA = na[a], nbE = nb[e], naE = na[e];
   const int nel = nbA * nbE;
+  if ((R == 1) != (nel <= NT)) return;  // the other instance's output
   const int pae = map2to1[s];
   // term 1 in one orientation of each pair (rep1; else the transpose partner's block
   // carries it), and not for the column atoms whose term 1 runs on the tensor cores
   const bool has1 = pae >= 0 && keepV[pae] && rep1[pae] && !(t1tc && t1tc[e]);
   const double w1 = has1 && rep1[pae] == 2 ? 0.5 : 1.0;
   if (!has1 && !t2) return;
-  double acc[XMAXE];
+  const Split sp = split_of<R>(nel, rank, ns);
+  double acc[R];
 #pragma unroll
-  for (int r = 0; r < XMAXE; r++) acc[r] = 0.0;
-  for (int64_t it = ptr[s]; it < ptr[s + 1]; it++) {
-    const X12Entry en = L[it];
-    if (!keepC[en.p3]) continue;
-    const int g = pA[en.p3];
-    const int nbG = nb[g], naG = na[g];
-    const double *Cge = C + offC[en.p3];
-    if (en.t1 && has1) {
-      // term 1: U1[Q][i][k] = sum_P V(A,E')[P][Q] T(A,G')[P][i][k], Q on E', in tiles of Q
-      const int qE0 = onsite[en.p3] ? 0 : naG;
-      const double *Tt = T + (off2[en.t] - tbase);
-      const double *Vae = V + offV[pae];
-      const int per = nbA * nbG;
-      const int qt = min(naE, max(1, smb / per));
-      for (int q0 = 0; q0 < naE; q0 += qt) {
-        const int qn = min(qt, naE - q0);
-        __syncthreads();
+  for (int r = 0; r < R; r++) acc[r] = 0.0;
+  if (has1) {
+    const double *Vae = V + offV[pae];
+    const int qlo = naE * rank / ns, qhi = naE * (rank + 1) / ns;  // this rank's Q on E'
+    for (int64_t it = ptr[s]; it < ptr[s + 1];) {
+      __syncthreads();
+      if (tid < 32)
+        x12_batch(tb, it, ptr[s + 1], min(XCOL, smb / nbA), L, keepC, pA, nb, na, onsite, off2, tbase, offC, nbE);
+      __syncthreads();
+      const int n = tb.n;
+      it += tb.next;
+      if (n == 0) continue;
+      const int per = nbA * n;
+      const int qt = max(1, smb / per);
+      for (int q0 = qlo; q0 < qhi; q0 += qt) {
+        const int qn = min(qt, qhi - q0);
+        if (q0 > qlo) __syncthreads();
         for (int el = tid; el < qn * per; el += NT) {
-          const int q = el / per, c = el - q * per;
+          const int q = el / per, rem = el - q * per;
+          const int i = rem / n, c = rem - i * n;
+          const int nbG = tb.nb[c];
+          const double *tp = T + tb.t[c] + (int64_t)i * nbG;
+          const double *vp = Vae + q0 + q;
+          const int st = nbA * nbG;
           double u = 0.0;
-          for (int P = 0; P < naA; P++) u = fma(__ldg(Vae + P * naE + q0 + q), __ldg(Tt + (int64_t)P * per + c), u);
-          sm[el] = u;
+#pragma unroll 4
+          for (int P = 0; P < naA; P++) {
+            u = fma(__ldg(vp), __ldg(tp), u);
+            vp += naE;
+            tp += st;
+          }
+          sm[el] = w1 * u;
         }
         __syncthreads();
+        if (sp.grp < sp.ng) {
+          const int K = qn * n;
+          const int k0 = K * sp.grp / sp.ng, k1 = K * (sp.grp + 1) / sp.ng;
 #pragma unroll
-        for (int r = 0; r < XMAXE; r++) {
-          const int el = tid + r * NT;
-          if (el < nel) {
-            const int i = el / nbE, l = el - i * nbE;
-            double v = 0.0;
-            for (int q = 0; q < qn; q++) {
-              const double *cq = Cge + ((int64_t)(qE0 + q0 + q) * nbG) * nbE + l;
-              const double *uq = sm + (q * nbA + i) * nbG;
-              for (int k = 0; k < nbG; k++) v = fma(uq[k], __ldg(cq + k * nbE), v);
+          for (int r = 0; r < R; r++) {
+            const int el = sp.el0 + r * NT;
+            if (el < nel) {
+              const int i = el / nbE, l = el - i * nbE;
+              int q = k0 / n, c = k0 - q * n;
+              const double *up = sm + ((int64_t)q * nbA + i) * n + c;
+              double v = acc[r];
+#pragma unroll 4
+              for (int k = k0; k < k1; k++) {
+                v = fma(*up, __ldg(C + tb.c[c] + (int64_t)(q0 + q) * (tb.nb[c] * nbE) + l), v);
+                up++;
+                if (++c == n) {  // the next Q: same row i
+                  c = 0;
+                  q++;
+                  up += (nbA - 1) * n;
+                }
+              }
+              acc[r] = v;
             }
-            acc[r] = fma(w1, v, acc[r]);
           }
         }
       }
     }
-    if (t2 && en.u2 >= 0 && keepV[en.u2]) {
-      // term 2: X += U2(A,G')[Q][i][k] C(G',E')[Q on G'][k][l] (on the tensor cores in mixed precision)
-      const double *U2 = U + offU[en.u2];
-#pragma unroll
-      for (int r = 0; r < XMAXE; r++) {
-        const int el = tid + r * NT;
-        if (el < nel) {
-          const int i = el / nbE, l = el - i * nbE;
-          double v = acc[r];
-          for (int q = 0; q < naG; q++) {
-            const double *cq = Cge + ((int64_t)q * nbG) * nbE + l;
-            const double *uq = U2 + ((int64_t)q * nbA + i) * nbG;
-            for (int k = 0; k < nbG; k++) v = fma(__ldg(uq + k), __ldg(cq + k * nbE), v);
-          }
-          acc[r] = v;
-        }
-      }
+  }
+  if (t2) {
+    // term 2: X += U2(A,G')[Q][i][k] C(G',E')[Q on G'][k][l] (on the tensor cores in mixed precision)
+    for (int64_t it = ptr[s]; it < ptr[s + 1]; it++) {
+      const X12Entry en = L[it];
+      if (en.u2 < 0 || !keepC[en.p3] || !keepV[en.u2]) continue;
+      const int g = pA[en.p3];
+      dot_share<R>(acc, sp, nel, U + offU[en.u2], C + offC[en.p3], na[g], nbA, nb[g], nbE);
     }
   }
   double *out = X + offK[map2to3[s]];
-#pragma unroll
-  for (int r = 0; r < XMAXE; r++) {
-    const int el = tid + r * NT;
-    if (el < nel) out[el] += acc[r];
-  }
+  gather_shares<R>(acc, sp, nel, ns, sm, [&](int el, double v) { out[el] += v; });
 }
 
 // ------------------------------------------------------------------ term 4 intermediate
@@ -331,7 +490,7 @@ __global__ void __launch_bounds__(NT) k_Z(const int2 *items, const int64_t *ptrZ
                                           const double *__restrict__ D, const int64_t *offD,
                                           const uint8_t *keepC, const uint8_t *keepV, const uint8_t *keepD,
                                           double *Z, int64_t zbase, int smb, const uint8_t *ztc,
-                                          const uint8_t *wZ, PScreen ps) {
+                                          const uint8_t *wZ, int cap, PScreen ps) {
   extern __shared__ double sm[];
   const int tid = threadIdx.x;
   const int2 it = items[blockIdx.x];
@@ -339,7 +498,7 @@ __global__ void __launch_bounds__(NT) k_Z(const int2 *items, const int64_t *ptrZ
   const int b = atomA2[z], e = atomB2[z];
   const int nbB = nb[b], naB = na[b], nbE = nb[e];
   const int per = nbB * nbE;
-  const int pt = max(1, NT * MAXE / per);
+  const int pt = max(1, cap / per);
   const int pe = min(naB, p0 + pt);
   const int nel = (pe - p0) * per;
   double acc[MAXE];
@@ -397,16 +556,15 @@ __global__ void __launch_bounds__(NT) k_Z(const int2 *items, const int64_t *ptrZ
 
 // ------------------------------------------------------------------ term 4 (and term 3 via the transpose)
 // X(A,E') += sum over (C(A,B') not on-site, Z(B,E'')) of C(A,B')[P on B'][i][j] Z[P][j][l].
-__global__ void __launch_bounds__(NT) k_X34(const int32_t *ord, const int64_t *ptr, const int2 *L,
-                                            const int32_t *atomA3, const int32_t *atomB3, const int32_t *pB,
-                                            const int32_t *nb, const int32_t *na,
-                                            const double *__restrict__ C, const int64_t *offC,
-                                            const uint8_t *keepC, const double *__restrict__ Z,
-                                            const int64_t *off2, const int64_t *offK, double *X, int64_t zbase,
-                                            int64_t zlo, int64_t zhi, int smb, const uint8_t *rep3) {
-  extern __shared__ double sm[];
-  const int tid = threadIdx.x;
-  const int x = ord[blockIdx.x];
+template <int R>
+__global__ void __launch_bounds__(NT, R == 1 ? 6 : 1)
+    k_X34(const int32_t *ord, const int64_t *ptr, const int2 *L, const int32_t *atomA3, const int32_t *atomB3,
+          const int32_t *pB, const int32_t *nb, const int32_t *na, const double *__restrict__ C, const int64_t *offC,
+          const uint8_t *keepC, const double *__restrict__ Z, const int64_t *off2, const int64_t *offK, double *X,
+          int64_t zbase, int64_t zlo, int64_t zhi, const uint8_t *rep3, int ns) {
+  __shared__ double red[R == 1 ? NT : NT * R];
+  const int x = ord[blockIdx.x / ns];
+  const int rank = blockIdx.x % ns;
   // term 4 halved in the K blocks: one orientation of each (the transpose partner carries
   // the other), with twice the weight of Z's 1/2; the self block keeps it.  Halved in Z
   // (rep3 = 2 everywhere): every block with weight 1.
@@ -416,47 +574,21 @@ __global__ void __launch_bounds__(NT) k_X34(const int32_t *ord, const int64_t *p
   const int a = atomA3[x], e = atomB3[x];
   const int nbA = nb[a], naA = na[a], nbE = nb[e];
   const int nel = nbA * nbE;
-  double acc[XMAXE];
+  if ((R == 1) != (nel <= NT)) return;  // the other instance's output
+  const Split sp = split_of<R>(nel, rank, ns);
+  double acc[R];
 #pragma unroll
-  for (int r = 0; r < XMAXE; r++) acc[r] = 0.0;
+  for (int r = 0; r < R; r++) acc[r] = 0.0;
   for (int64_t it = ptr[x]; it < ptr[x + 1]; it++) {
     const int2 en = L[it];
     if (!keepC[en.x] || en.y < zlo || en.y >= zhi) continue;
     const int b = pB[en.x];
-    const int nbB = nb[b], naB = na[b];
-    const double *Cb = C + offC[en.x] + (int64_t)naA * nbA * nbB;
-    const double *Zb = Z + (off2[en.y] - zbase);
-    const int csz = nbA * nbB, zsz = nbB * nbE;
-    const int pc = max(1, min(naB, smb / (csz + zsz)));
-    for (int P0 = 0; P0 < naB; P0 += pc) {
-      const int pn = min(pc, naB - P0);
-      __syncthreads();
-      for (int i = tid; i < pn * csz; i += NT) sm[i] = Cb[(int64_t)P0 * csz + i];
-      for (int i = tid; i < pn * zsz; i += NT) sm[pn * csz + i] = Zb[(int64_t)P0 * zsz + i];
-      __syncthreads();
-      const double *Zs = sm + pn * csz;
-#pragma unroll
-      for (int r = 0; r < XMAXE; r++) {
-        const int el = tid + r * NT;
-        if (el < nel) {
-          const int i = el / nbE, l = el - i * nbE;
-          double v = acc[r];
-          for (int P = 0; P < pn; P++) {
-            const double *cr = sm + (P * nbA + i) * nbB;
-            const double *zr = Zs + P * zsz + l;
-            for (int j = 0; j < nbB; j++) v = fma(cr[j], zr[j * nbE], v);
-          }
-          acc[r] = v;
-        }
-      }
-    }
+    const int nbB = nb[b];
+    dot_share<R>(acc, sp, nel, C + offC[en.x] + (int64_t)naA * nbA * nbB, Z + (off2[en.y] - zbase), na[b], nbA, nbB,
+                 nbE);
   }
   double *out = X + offK[x];
-#pragma unroll
-  for (int r = 0; r < XMAXE; r++) {
-    const int el = tid + r * NT;
-    if (el < nel) out[el] += w4 * acc[r];
-  }
+  gather_shares<R>(acc, sp, nel, ns, red, [&](int el, double v) { out[el] += w4 * v; });
 }
 
 // ------------------------------------------------------------------ K = X + X^T (image flipped)
@@ -543,13 +675,14 @@ __global__ void k_fold(int64_t ng, const int64_t *fold, const int32_t *atomA3, c
   }
 }
 
+rix_status fail_cuda(rix_ctx *ctx, const char *what, cudaError_t e) {
+  ctx->last_error = std::string(what) + ": " + cudaGetErrorString(e);
+  return RIX_ECUDA;
+}
+
 rix_status last(rix_ctx *ctx, const char *what) {
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) {
-    ctx->last_error = std::string(what) + ": " + cudaGetErrorString(e);
-    return RIX_ECUDA;
-  }
-  return RIX_OK;
+  return e == cudaSuccess ? RIX_OK : fail_cuda(ctx, what, e);
 }
 
 bool g_attr_done = false;
@@ -601,9 +734,9 @@ namespace {
 
 void set_attrs() {
   if (!g_attr_done) {
-    cudaFuncSetAttribute(k_X12, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_MAX * 8);
+    cudaFuncSetAttribute(k_X12<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_MAX * 8);
+    cudaFuncSetAttribute(k_X12<XMAXE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_MAX * 8);
     cudaFuncSetAttribute(k_Z, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_MAX * 8);
-    cudaFuncSetAttribute(k_X34, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_MAX * 8);
     g_attr_done = true;
   }
 }
@@ -617,35 +750,89 @@ rix_status launch_Z_items(rix_ctx *ctx, const double *D, int b, int64_t first, i
                                             ctx->d_atomA2, ctx->d_atomB2, ctx->d_off2, ctx->d_pB, ctx->d_nb,
                                             ctx->d_na, ctx->d_C, ctx->d_offC, ctx->d_V, ctx->d_offV, D, ctx->d_offD,
                                             ctx->d_keepC, ctx->d_keepV, ctx->d_keepD, ctx->d_Z, ctx->blk_base[b],
-                                            smb, ctx->have_mx ? ctx->d_ztc : nullptr, ctx->d_wZ, rix_pscreen(ctx));
+                                            smb, ctx->have_mx ? ctx->d_ztc : nullptr, ctx->d_wZ, ctx->cap_Z,
+                                            rix_pscreen(ctx));
   return last(ctx, "k_Z");
+}
+
+// a launch of count outputs, each shared by a cluster of ns CTAs
+template <class... P, class... A>
+cudaError_t launch_split(void (*kernel)(P...), int64_t count, int ns, int smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(count * ns));
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = ns;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = ns > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// outputs of terms 1+2 in block b
+int64_t n_X12(const rix_ctx *ctx, int b) {
+  return ctx->segX12[rix_ctx::NCLS * (b + 1)] - ctx->segX12[rix_ctx::NCLS * b];
 }
 
 // terms 1+2 for the output blocks [first, first + count) of block b's launch order.
 rix_status launch_X12_items(rix_ctx *ctx, int b, int64_t first, int64_t count, int smb, cudaStream_t st) {
   set_attrs();
-  if (!count) return RIX_OK;
-  k_X12<<<(unsigned)count, NT, smb * 8, st>>>(
-      ctx->d_ordX12 + ctx->segX12[b] + first, ctx->d_ptrX12, ctx->d_LX12, ctx->d_atomA2, ctx->d_atomB2,
-      ctx->d_map2to1, ctx->d_map2to3, ctx->d_pA, ctx->d_onsite, ctx->d_nb, ctx->d_na, ctx->d_C, ctx->d_offC,
-      ctx->d_V, ctx->d_offV, ctx->d_keepC, ctx->d_keepV, ctx->d_T, ctx->d_off2, ctx->d_U, ctx->d_offU, ctx->d_offK,
-      ctx->d_X, ctx->blk_base[b], smb, ctx->have_mx ? 0 : 1, ctx->have_mx ? ctx->d_t1tc : nullptr, ctx->d_rep1);
+  smb = std::max(smb, 64 * 64);  // one column entry of 64 functions over 64 rows, or a 64 x 64 output
+  const int64_t *seg = &ctx->segX12[rix_ctx::NCLS * b];
+  for (int c = 0; c < rix_ctx::NCLS; c++) {  // the class's part of [first, first + count)
+    const int64_t lo = std::max(seg[c], seg[0] + first), hi = std::min(seg[c + 1], seg[0] + first + count);
+    if (hi <= lo) continue;
+    auto go = [&](auto *kernel) {
+      return launch_split(kernel, hi - lo, 1 << c, smb * 8, st, ctx->d_ordX12 + lo, ctx->d_ptrX12, ctx->d_LX12,
+                          ctx->d_atomA2, ctx->d_atomB2, ctx->d_map2to1, ctx->d_map2to3, ctx->d_pA, ctx->d_onsite,
+                          ctx->d_nb, ctx->d_na, ctx->d_C, ctx->d_offC, ctx->d_V, ctx->d_offV, ctx->d_keepC,
+                          ctx->d_keepV, ctx->d_T, ctx->d_off2, ctx->d_U, ctx->d_offU, ctx->d_offK, ctx->d_X,
+                          ctx->blk_base[b], smb, ctx->have_mx ? 0 : 1, ctx->have_mx ? ctx->d_t1tc : nullptr,
+                          ctx->d_rep1, 1 << c);
+    };
+    cudaError_t e = go(k_X12<1>);
+    if (e == cudaSuccess && ctx->max_nel > NT) e = go(k_X12<XMAXE>);
+    if (e != cudaSuccess) return fail_cuda(ctx, "k_X12", e);
+  }
   return last(ctx, "k_X12");
 }
 
-// terms 3+4 (FP64) for the K blocks [first, first + count) of the launch order, Z of block b.
-rix_status launch_X34_items(rix_ctx *ctx, int b, int64_t first, int64_t count, int smb, cudaStream_t st) {
-  set_attrs();
-  if (!count) return RIX_OK;
+// terms 3+4 (FP64) for every K block, Z of block b.
+rix_status launch_X34(rix_ctx *ctx, int b, cudaStream_t st) {
   const int64_t zlo = ctx->row2[ctx->blk_atom[b]], zhi = ctx->row2[ctx->blk_atom[b + 1]];
-  k_X34<<<(unsigned)count, NT, smb * 8, st>>>(ctx->d_ordX34 + first, ctx->d_ptrX34, ctx->d_LX34, ctx->d_atomA3,
-                                              ctx->d_atomB3, ctx->d_pB, ctx->d_nb, ctx->d_na, ctx->d_C, ctx->d_offC,
-                                              ctx->d_keepC, ctx->d_Z, ctx->d_off2, ctx->d_offK, ctx->d_X,
-                                              ctx->blk_base[b], zlo, zhi, smb, ctx->d_rep3);
+  for (int c = 0; c < rix_ctx::NCLS; c++) {
+    const int64_t lo = ctx->segX34[c], n = ctx->segX34[c + 1] - lo;
+    if (!n) continue;
+    auto go = [&](auto *kernel) {
+      return launch_split(kernel, n, 1 << c, 0, st, ctx->d_ordX34 + lo, ctx->d_ptrX34, ctx->d_LX34, ctx->d_atomA3,
+                          ctx->d_atomB3, ctx->d_pB, ctx->d_nb, ctx->d_na, ctx->d_C, ctx->d_offC, ctx->d_keepC,
+                          ctx->d_Z, ctx->d_off2, ctx->d_offK, ctx->d_X, ctx->blk_base[b], zlo, zhi, ctx->d_rep3,
+                          1 << c);
+    };
+    cudaError_t e = go(k_X34<1>);
+    if (e == cudaSuccess && ctx->max_nel > NT) e = go(k_X34<XMAXE>);
+    if (e != cudaSuccess) return fail_cuda(ctx, "k_X34", e);
+  }
   return last(ctx, "k_X34");
 }
 
 }  // namespace
+
+// one launch per class that has outputs, and a second one for the K blocks above 256 elements
+int32_t rix_x12_launches(const rix_ctx *ctx) {
+  int32_t n = 0;
+  for (size_t i = 0; i + 1 < ctx->segX12.size(); i++) n += ctx->segX12[i + 1] > ctx->segX12[i];
+  return ctx->max_nel > NT ? 2 * n : n;
+}
+
+int32_t rix_x34_launches(const rix_ctx *ctx) {
+  int32_t n = 0;
+  for (int c = 0; c < rix_ctx::NCLS; c++) n += ctx->segX34[c + 1] > ctx->segX34[c];
+  return ctx->max_nel > NT ? 2 * n : n;
+}
 
 // T(A,G') for the row atoms of block b (T buffer holds that block).  In mixed
 // precision the buffer is cleared first and the tensor cores add the T blocks
@@ -661,7 +848,7 @@ rix_status rix_launch_T_block(rix_ctx *ctx, const double *D, int b, cudaStream_t
     k_T<<<(unsigned)nT, NT, 64 * 64 * 8, st>>>(ctx->d_itT + ctx->segT[b], ctx->d_ptrT, ctx->d_LT, ctx->d_atomA2,
                                                ctx->d_atomB2, ctx->d_off2, ctx->d_pB, ctx->d_nb, ctx->d_na,
                                                ctx->d_C, ctx->d_offC, D, ctx->d_offD, ctx->d_keepC, ctx->d_keepD,
-                                               ctx->d_T, ctx->blk_base[b], tc ? ctx->d_ttc : nullptr,
+                                               ctx->d_T, ctx->blk_base[b], tc ? ctx->d_ttc : nullptr, ctx->cap_T,
                                                rix_pscreen(ctx));
     rix_status s = last(ctx, "k_T");
     if (s != RIX_OK) return s;
@@ -707,7 +894,7 @@ rix_status rix_fp64_build(rix_ctx *ctx, const double *D, double *K, cudaStream_t
     }
     if (b == 0 && (s = rix_prof_mark(ctx, 3, st)) != RIX_OK) return s;
     if ((!ctx->have_mx || ctx->n_t1tc < ctx->nat) &&
-        (s = launch_X12_items(ctx, b, 0, ctx->segX12[b + 1] - ctx->segX12[b], ctx->tile_X12, st)) != RIX_OK)
+        (s = launch_X12_items(ctx, b, 0, n_X12(ctx, b), ctx->tile_X12, st)) != RIX_OK)
       return s;
     // mixed precision, several row blocks: term 1 on the tensor cores while T of the block is resident
     if (ctx->have_mx && ctx->nblk > 1 && (s = rix_mixed_t1(ctx, b, tbase, st)) != RIX_OK) return s;
@@ -724,7 +911,7 @@ rix_status rix_fp64_build(rix_ctx *ctx, const double *D, double *K, cudaStream_t
     if (b == 0 && (s = rix_prof_mark(ctx, 6, st)) != RIX_OK) return s;
     if (ctx->have_mx) {
       if ((s = rix_mixed_x34(ctx, b, zbase, st)) != RIX_OK) return s;
-    } else if ((s = launch_X34_items(ctx, b, 0, ctx->n_ordX34, ctx->tile_X34, st)) != RIX_OK) {
+    } else if ((s = launch_X34(ctx, b, st)) != RIX_OK) {
       return s;
     }
   }
@@ -736,8 +923,8 @@ rix_status rix_fp64_build(rix_ctx *ctx, const double *D, double *K, cudaStream_t
 }
 
 // ------------------------------------------------------------------ autotuner
-// Picks the shared-memory tile budget of k_X12, k_Z and k_X34 (and with it
-// their tile shapes and CTAs per SM) by timing each candidate on a slice of
+// Picks the shared-memory tile budget of k_X12 and k_Z (and with it their
+// tile shapes and CTAs per SM; k_X34 stages nothing and keeps its entry) by timing each candidate on a slice of
 // the real work items of the first memory-plan block; the choice is cached
 // per system in a text file.  The analogue of the paper's auto-tuned Fock
 // block size (Sec. "Initialization"), at the level of one GPU's tiles.
@@ -831,7 +1018,7 @@ extern "C" rix_status rix_autotune(rix_ctx *ctx, const double *D, const char *ca
   }
   float ms = 0.f;
   {
-    const int64_t n = ctx->segX12[b + 1] - ctx->segX12[b], cnt = std::min(n, SAMPLE), first = (n - cnt) / 2;
+    const int64_t n = n_X12(ctx, b), cnt = std::min(n, SAMPLE), first = (n - cnt) / 2;
     if (cnt && (s = pick(ctx, st, [&](int c) { return launch_X12_items(ctx, b, first, cnt, c, st); },
                          &ctx->tile_X12, &ms)) != RIX_OK)
       return s;
@@ -840,13 +1027,6 @@ extern "C" rix_status rix_autotune(rix_ctx *ctx, const double *D, const char *ca
     const int64_t n = ctx->segZ[b + 1] - ctx->segZ[b], cnt = std::min(n, SAMPLE), first = (n - cnt) / 2;
     if (cnt && (s = pick(ctx, st, [&](int c) { return launch_Z_items(ctx, D, b, first, cnt, c, st); },
                          &ctx->tile_Z, &ms)) != RIX_OK)
-      return s;
-  }
-  if (!ctx->have_mx && ctx->n_ordX34) {
-    if ((s = rix_launch_Z_block(ctx, D, b, st)) != RIX_OK) return s;
-    const int64_t n = ctx->n_ordX34, cnt = std::min(n, SAMPLE), first = (n - cnt) / 2;
-    if ((s = pick(ctx, st, [&](int c) { return launch_X34_items(ctx, b, first, cnt, c, st); }, &ctx->tile_X34,
-                  &ms)) != RIX_OK)
       return s;
   }
   RIX_CUDA_TRY(ctx, cudaStreamSynchronize(st));

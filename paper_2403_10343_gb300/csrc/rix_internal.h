@@ -88,6 +88,9 @@ struct BX12Entry {
   int32_t t1;    // 1 if term 1
 };
 
+// Output elements of a row-tiled work item: 32 or 4 per thread of a 256-thread CTA.
+constexpr int CAP_MAX = 8192, CAP_MIN = 1024;
+
 // Device allocation tracked for the workspace statistics.
 struct DevBuf {
   void *p = nullptr;
@@ -133,15 +136,14 @@ struct rix_ctx {
   // with weight 1/2 (on-site pair), 0 = left to the transpose partner
   std::vector<uint8_t> rep1;
   uint8_t *d_rep1 = nullptr;
-  // Term 4 is symmetric as well, and the build evaluates half of it in one of two ways
-  // (z_half, chosen at setup by the estimated cost of both):
-  //   z_half = false: Z sums over every pair (B, G') with weight 1/2, and X takes the K
-  //     blocks (A, E', n) in one orientation with twice that weight;
-  //   z_half = true: Z sums over the unordered pairs {B, G'} with weight 1 (1/2 on-site),
-  //     and X takes every K block.
+  // Term 4 is symmetric as well, and the build evaluates half of it in one of two ways,
+  // chosen at setup by the estimated cost of both:
+  //   Z sums over every pair (B, G') with weight 1/2, and X takes the K blocks (A, E', n)
+  //     in one orientation with twice that weight; or
+  //   Z sums over the unordered pairs {B, G'} with weight 1 (1/2 on-site), and X takes
+  //     every K block.
   // rep3 per K block: 1 = weight 2, 2 = weight 1, 0 = left to the transpose partner; wZ per
   // pair (B, G'): 1 = weight 1, 2 = weight 1/2, 0 = left to the partner pair.
-  bool z_half = false;
   std::vector<uint8_t> rep3, wZ;
   uint8_t *d_rep3 = nullptr, *d_wZ = nullptr;
   double *d_f34 = nullptr;             // per pair (A, B'): FLOPs of its terms-3+4 products (rix_count_flops)
@@ -218,7 +220,9 @@ struct rix_ctx {
   int32_t nblk = 1;
   std::vector<int32_t> blk_atom;                  // [nblk+1]
   std::vector<int64_t> blk_base;                  // off2 of the block's first 2-hop block
-  std::vector<int64_t> segT, segU, segX12, segZ;  // [nblk+1] ranges in the item arrays
+  std::vector<int64_t> segT, segU, segZ;          // [nblk+1] ranges in the item arrays
+  std::vector<int64_t> segX12;                    // [NCLS nblk + 1], see NCLS
+  int32_t cap_T = 0, cap_Z = 0;                   // output elements per T and Z item (CAP_MAX or CAP_MIN)
 
   // ------------------------------------------------------------ backward plan (opt.backward)
   bool have_bwd = false;
@@ -237,8 +241,19 @@ struct rix_ctx {
 
   rix_stats_t stats{};
 
-  // shared-memory tile budgets (doubles) of k_X12, k_Z and k_X34; rix_autotune picks them
-  int32_t tile_X12 = 12288, tile_Z = 12288, tile_X34 = 12288;
+  // shared-memory tile budgets (doubles) of k_X12 and k_Z; rix_autotune picks them (tile_X34
+  // stays as it is: k_X34 stages nothing)
+  int32_t tile_X12 = 4096, tile_Z = 12288, tile_X34 = 4096;
+  // Launch classes of k_X12 and k_X34: class c holds the outputs shared by a cluster of 2^c CTAs
+  // (segX12[4 b + c] .. of block b, segX34[c] ..); max_nel: the largest K block (elements)
+  static constexpr int NCLS = 4;
+  std::vector<int64_t> segX34;
+  int32_t max_nel = 0;
+  // connected component of the pair list of every atom.  What changes the order of a sum is
+  // decided per component, so that systems batched in one context (batch.py) give the bits that
+  // each gives alone.
+  std::vector<int32_t> comp;
+  int32_t ncomp = 0;
 
   // stage timing (rix_options.profile): 8 events per build, pooled
   static constexpr int NSTAGE = 8;
@@ -294,6 +309,8 @@ int32_t rix_tt_launches(const rix_ctx *ctx);
 
 // FP64 path launches (rix_fp64.cu)
 rix_status rix_fp64_build(rix_ctx *ctx, const double *D, double *K, cudaStream_t st, int accumulate = 0);
+int32_t rix_x12_launches(const rix_ctx *ctx);  // of one build
+int32_t rix_x34_launches(const rix_ctx *ctx);  // per block of middle atoms
 rix_status rix_launch_T_block(rix_ctx *ctx, const double *D, int b, cudaStream_t st);
 rix_status rix_launch_Z_block(rix_ctx *ctx, const double *D, int b, cudaStream_t st);
 rix_status rix_launch_flags(rix_ctx *ctx, const double *arr, const int64_t *off, int64_t n,

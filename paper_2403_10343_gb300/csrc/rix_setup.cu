@@ -281,15 +281,37 @@ static rix_status build_backward_lists(rix_ctx *ctx, const std::vector<int2> &LT
   return RIX_OK;
 }
 
-// Which half of term 4 the build evaluates (rix_ctx::z_half) and the pair weights wZ.
-// Both forms cost one stage in full and the other in half; the estimates below count
-// every product of the lists (D, which screens Z, is not known yet).  FP64: the FLOPs of
-// the two stages.  Mixed: the sliced products, Z as Kronecker rows (na nb per row atom and
-// nb_B na_G nb_G per column), which makes Z the larger one by far except where few
-// atoms lie within the cutoff.  (GB300, mixed, start and with Z halved: (H2O)64 cluster 169.3 and
-// 123.0 ms, 192-atom ice cell 379 and 330 ms, 12-atom perovskite 239 and 210 ms.  FP64: the 24-atom
-// ice cell, whose K blocks outweigh Z (245 and 31 ms), stays with the halved K blocks.)
-static void choose_term4(rix_ctx *ctx) {
+// Connected components of the pair list (rix_ctx::comp), numbered by their first atom.
+static void find_components(rix_ctx *ctx) {
+  ctx->comp.assign(ctx->nat, -1);
+  std::vector<int> stack;
+  for (int s = 0; s < ctx->nat; s++) {
+    if (ctx->comp[s] >= 0) continue;
+    ctx->comp[s] = ctx->ncomp;
+    stack.push_back(s);
+    while (!stack.empty()) {
+      const int a = stack.back();
+      stack.pop_back();
+      for (int64_t p = ctx->row1[a]; p < ctx->row1[a + 1]; p++)
+        if (ctx->comp[ctx->pB[p]] < 0) {
+          ctx->comp[ctx->pB[p]] = ctx->ncomp;
+          stack.push_back(ctx->pB[p]);
+        }
+    }
+    ctx->ncomp++;
+  }
+}
+
+// Which half of term 4 the build evaluates, as the pair weights wZ; returns per component
+// whether Z is the halved stage.  Both forms cost one stage in full and the other in half;
+// the estimates below count every product of the lists (D, which screens Z, is not known
+// yet).  FP64: the FLOPs of the two stages.  Mixed: the sliced products, Z as Kronecker rows
+// (na nb per row atom and nb_B na_G nb_G per column), which makes Z the larger one by far
+// except where few atoms lie within the cutoff.  (GB300, mixed, K blocks halved and Z halved:
+// (H2O)64 cluster 169.3 and 123.0 ms, 192-atom ice cell 379 and 330 ms, 12-atom perovskite 239
+// and 210 ms.  FP64: the 24-atom ice cell, whose K blocks outweigh Z (245 and 31 ms), stays with
+// the halved K blocks.)
+static std::vector<uint8_t> choose_term4(rix_ctx *ctx) {
   const int nat = ctx->nat;
   const bool mixed = ctx->opt.precision == RIX_MIXED_BF16;
   std::vector<double> sE(nat, 0.0), s2(nat, 0.0);
@@ -301,8 +323,17 @@ static void choose_term4(rix_ctx *ctx) {
     const double naG = ctx->na_at[ctx->pB[p]], nbG = ctx->nb_at[ctx->pB[p]];
     return 2.0 * naB * nbG * (naG + nbB) * sE[ctx->pB[p]];
   };
+  // Weight of a sliced-product FLOP against a Z FLOP.  Deterministic mixed builds run Z on the
+  // FP64 pipe, about 600 times slower per FLOP than the tensor cores.
+  double px = 1.0, pz = 1.0;
+  const bool kron = mixed && !ctx->opt.deterministic;
+  if (mixed) {
+    const int S = rix_plan_slices(ctx, 0), R = rix_plan_slices(ctx, 2);
+    px = 0.5 * S * (S + 1) / (kron ? 1.0 : 600.0);
+    if (kron) pz = 0.5 * R * (R + 1);
+  }
   ctx->wZ.assign(ctx->np, 0);
-  double z_all = 0, z_rep = 0, zk_all = 0, zk_rep = 0, x_all = 0;
+  std::vector<double> z_all(ctx->ncomp, 0.0), z_rep(ctx->ncomp, 0.0), x_all(ctx->ncomp, 0.0);
   for (int64_t p = 0; p < ctx->np; p++) {
     const int b = ctx->pA[p], g = ctx->pB[p];
     // one pair of {(B, G'), (G', B)}: in FP64 the one that applies V from the side that
@@ -313,32 +344,16 @@ static void choose_term4(rix_ctx *ctx) {
       if (f != fq) rep = f < fq;
     }
     ctx->wZ[p] = ctx->onsite[p] ? 2 : rep ? 1 : 0;
-    const double zk = 2.0 * ctx->na_at[b] * ctx->nb_at[b] * ctx->na_at[g] * ctx->nb_at[g] * sE[g];
-    z_all += fz(p);
-    zk_all += zk;
-    if (ctx->wZ[p]) {
-      z_rep += fz(p);
-      zk_rep += zk;
-    }
+    const double f = kron ? 2.0 * ctx->na_at[b] * ctx->nb_at[b] * ctx->na_at[g] * ctx->nb_at[g] * sE[g] : fz(p);
+    z_all[ctx->comp[b]] += f;
+    if (ctx->wZ[p]) z_rep[ctx->comp[b]] += f;
   }
-  for (int a = 0; a < nat; a++) x_all += 2.0 * ctx->na_at[a] * ctx->nb_at[a] * sE[a] * s2[a];
-  double full, half;  // costs with Z in full, with Z halved
-  if (mixed && !ctx->opt.deterministic) {
-    const int S = rix_plan_slices(ctx, 0), R = rix_plan_slices(ctx, 2);
-    const double px = 0.5 * S * (S + 1), pz = 0.5 * R * (R + 1);
-    full = zk_all * pz + 0.5 * x_all * px;
-    half = zk_rep * pz + x_all * px;
-  } else if (mixed) {  // deterministic: Z on the FP64 pipe, ~600 times slower per FLOP than a sliced product
-    const int S = rix_plan_slices(ctx, 0);
-    const double px = 0.5 * S * (S + 1) / 600.0;
-    full = z_all + 0.5 * x_all * px;
-    half = z_rep + x_all * px;
-  } else {
-    full = z_all + 0.5 * x_all;
-    half = z_rep + x_all;
-  }
-  ctx->z_half = half < full;
-  if (!ctx->z_half) ctx->wZ.assign(ctx->np, 2);
+  for (int a = 0; a < nat; a++) x_all[ctx->comp[a]] += 2.0 * ctx->na_at[a] * ctx->nb_at[a] * sE[a] * s2[a];
+  std::vector<uint8_t> half(ctx->ncomp);
+  for (int c = 0; c < ctx->ncomp; c++) half[c] = z_rep[c] * pz + x_all[c] * px < z_all[c] * pz + 0.5 * x_all[c] * px;
+  for (int64_t p = 0; p < ctx->np; p++)
+    if (!half[ctx->comp[ctx->pA[p]]]) ctx->wZ[p] = 2;
+  return half;
 }
 
 static rix_status build_lists(rix_ctx *ctx) {
@@ -557,9 +572,11 @@ static rix_status build_lists(rix_ctx *ctx) {
   for (int64_t p = 0; p < np; p++) flU2 += 2.0 * NA(pA[p]) * NA(pB[p]) * NB(pA[p]) * NB(pB[p]);
 
   // ---------------------------------------------------------------- term 4: which half
-  choose_term4(ctx);
-  ctx->rep3.assign(nk, 2);
-  if (!ctx->z_half) ctx->rep3 = rep3c;
+  find_components(ctx);
+  const std::vector<uint8_t> z_half = choose_term4(ctx);
+  ctx->rep3 = rep3c;
+  for (int64_t x = 0; x < nk; x++)
+    if (z_half[ctx->comp[atomA3[x]]]) ctx->rep3[x] = 2;
 
   // ---------------------------------------------------------------- Z list (term 4): Z(B,E') <- (pair (B,G'), pair (G',E'))
   // and the X34 list: X(A,E') <- (C(A,B') not on-site, Z(B,E'-n1)).  Z blocks that no
@@ -664,34 +681,36 @@ static rix_status build_lists(rix_ctx *ctx) {
   }
 
   // ---------------------------------------------------------------- work items and launch orders
-  const int64_t CAP = 8192;  // output elements per work item (256 threads x 32)
+  // Row tiles of T and Z (a block's P rows, CAP output elements per item at most) and of U2.
+  // 8192 elements (32 per thread) re-read the operands least; a system whose stage would have
+  // fewer than 32 items per SM takes 1024, so that its longest item does not run on alone (the
+  // sums do not depend on the tile).  U2 has one product per output and always takes 1024.
   std::vector<int2> itT, itZ, itU;
   std::vector<double> cT, cZ;
-  for (int64_t t = 0; t < n2; t++) {
-    int a = atomA2[t], g = atomB2[t];
-    int64_t per = NB(a) * NB(g);
-    int64_t pt = std::max<int64_t>(1, CAP / per);
-    double len = (double)(ptrT[t + 1] - ptrT[t]);
-    for (int64_t p0 = 0; p0 < NA(a); p0 += pt) {
-      itT.push_back(make_int2((int)t, (int)p0));
-      cT.push_back(len * std::min(pt, NA(a) - p0) * per);
+  auto tile2 = [&](const std::vector<int64_t> &ptr, std::vector<int2> &it, std::vector<double> &c, bool empty) {
+    int64_t cap = CAP_MAX;
+    for (;; cap = CAP_MIN) {
+      for (int64_t t = 0; t < n2; t++) {
+        const int a = atomA2[t];
+        const int64_t per = NB(a) * NB(atomB2[t]), pt = std::max<int64_t>(1, cap / per);
+        const double len = (double)(ptr[t + 1] - ptr[t]);
+        if (len == 0 && !empty) continue;
+        for (int64_t p0 = 0; p0 < NA(a); p0 += pt) {
+          it.push_back(make_int2((int)t, (int)p0));
+          c.push_back(len * std::min(pt, NA(a) - p0) * per);
+        }
+      }
+      if (cap == CAP_MIN || it.size() >= 32 * 152) return (int32_t)cap;
+      it.clear();
+      c.clear();
     }
-  }
-  for (int64_t z = 0; z < n2; z++) {
-    int b = atomA2[z], e = atomB2[z];
-    int64_t per = NB(b) * NB(e);
-    int64_t pt = std::max<int64_t>(1, CAP / per);
-    double len = (double)(ptrZ[z + 1] - ptrZ[z]);
-    if (len == 0) continue;
-    for (int64_t p0 = 0; p0 < NA(b); p0 += pt) {
-      itZ.push_back(make_int2((int)z, (int)p0));
-      cZ.push_back(len * std::min(pt, NA(b) - p0) * per);
-    }
-  }
+  };
+  ctx->cap_T = tile2(ptrT, itT, cT, true);
+  ctx->cap_Z = tile2(ptrZ, itZ, cZ, false);
   for (int64_t p = 0; p < np; p++) {
     int a = pA[p], g = pB[p];
     int64_t per = NB(a) * NB(g);
-    int64_t qt = std::max<int64_t>(1, CAP / per);
+    int64_t qt = std::max<int64_t>(1, CAP_MIN / per);
     for (int64_t q0 = 0; q0 < NA(g); q0 += qt) itU.push_back(make_int2((int)p, (int)q0));
   }
   // launch order: most expensive first (longest processing time first)
@@ -710,8 +729,29 @@ static rix_status build_lists(rix_ctx *ctx) {
   for (int64_t s = 0; s < n2; s++)
     if (ptrX12[s + 1] > ptrX12[s]) {
       ordX12.push_back((int32_t)s);
-      cX12.push_back((double)(ptrX12[s + 1] - ptrX12[s]) * NA(atomA2[s]) * NB(atomA2[s]));
+      // multiply-adds per column (G', k) of the list
+      const int a = atomA2[s], e = atomB2[s];
+      const int64_t pae = map2to1[s];
+      const double t1 = pae >= 0 && ctx->rep1[pae] ? (double)NA(e) * NB(a) * (NA(a) + NB(e)) : 0.0;
+      cX12.push_back((double)(ptrX12[s + 1] - ptrX12[s]) * (t1 + (double)NA(a) * NB(a) * NB(e)));
     }
+  // A cluster of 2^c CTAs per output (1, 2, 4 or 8) where the longest output of its component
+  // would otherwise take more than half of an even share of the stage on the 152 SMs: its CTA
+  // would run on alone at the end.
+  auto clusters = [&](const std::vector<int32_t> &ord, const std::vector<double> &c, auto atom) {
+    std::vector<double> tot(ctx->ncomp, 0.0), top(ctx->ncomp, 0.0);
+    for (size_t i = 0; i < ord.size(); i++) {
+      const int m = ctx->comp[atom(ord[i])];
+      tot[m] += c[i];
+      top[m] = std::max(top[m], c[i]);
+    }
+    std::vector<int> cls(ctx->ncomp, 0);
+    for (int m = 0; m < ctx->ncomp; m++)
+      while (cls[m] + 1 < rix_ctx::NCLS && 2.0 * top[m] * 152 > tot[m] * (1 << cls[m])) cls[m]++;
+    return cls;
+  };
+  const std::vector<int> cls12 = clusters(ordX12, cX12, [&](int32_t s) { return atomA2[s]; });
+  for (int a = 0; a < nat; a++) ctx->max_nel = std::max(ctx->max_nel, (int32_t)(NB(a) * NB(a)));
   {
     std::vector<int64_t> idx(ordX12.size());
     std::iota(idx.begin(), idx.end(), 0);
@@ -727,12 +767,18 @@ static rix_status build_lists(rix_ctx *ctx) {
         ordX34.push_back((int32_t)x);
         c.push_back((double)(ptrX34[x + 1] - ptrX34[x]) * NB(atomA3[x]) * NB(atomB3[x]));
       }
+    const std::vector<int> cls = clusters(ordX34, c, [&](int32_t x) { return atomA3[x]; });
     std::vector<int64_t> idx(ordX34.size());
     std::iota(idx.begin(), idx.end(), 0);
     std::stable_sort(idx.begin(), idx.end(), [&](int64_t x, int64_t y) { return c[x] > c[y]; });
     std::vector<int32_t> o(idx.size());
     for (size_t i = 0; i < idx.size(); i++) o[i] = ordX34[idx[i]];
     ordX34.swap(o);
+    auto of = [&](int32_t x) { return cls[ctx->comp[atomA3[x]]]; };
+    std::stable_sort(ordX34.begin(), ordX34.end(), [&](int32_t x, int32_t y) { return of(x) < of(y); });
+    ctx->segX34.assign(rix_ctx::NCLS + 1, 0);
+    for (int32_t x : ordX34) ctx->segX34[of(x) + 1]++;
+    for (int q = 0; q < rix_ctx::NCLS; q++) ctx->segX34[q + 1] += ctx->segX34[q];
   }
   // fold groups: consecutive K blocks of one atom pair
   std::vector<int64_t> fold;
@@ -868,11 +914,11 @@ static rix_status build_lists(rix_ctx *ctx) {
   seg_sort(itZ, [&](const int2 &v) { return blk_of[atomA2[v.x]]; }, ctx->segZ);
   seg_sort(itU, [&](const int2 &v) { return blk_of[pA[v.x]]; }, ctx->segU);
   {
-    std::stable_sort(ordX12.begin(), ordX12.end(),
-                     [&](int32_t x, int32_t y) { return blk_of[atomA2[x]] < blk_of[atomA2[y]]; });
-    ctx->segX12.assign(nblk + 1, 0);
-    for (auto v : ordX12) ctx->segX12[blk_of[atomA2[v]] + 1]++;
-    for (int b = 0; b < nblk; b++) ctx->segX12[b + 1] += ctx->segX12[b];
+    auto of = [&](int32_t s) { return rix_ctx::NCLS * blk_of[atomA2[s]] + cls12[ctx->comp[atomA2[s]]]; };
+    std::stable_sort(ordX12.begin(), ordX12.end(), [&](int32_t x, int32_t y) { return of(x) < of(y); });
+    ctx->segX12.assign(rix_ctx::NCLS * nblk + 1, 0);
+    for (auto v : ordX12) ctx->segX12[of(v) + 1]++;
+    for (int b = 0; b < rix_ctx::NCLS * nblk; b++) ctx->segX12[b + 1] += ctx->segX12[b];
   }
   ctx->nblk = nblk;
   TRY(rix_upload(ctx, &ctx->d_itT, itT)); ctx->n_itT = itT.size();

@@ -445,7 +445,7 @@ void launch_pack(const double *X, int64_t sr, int64_t sk, int R, int Kd, int Rpa
 constexpr int GMAX = 4;
 // xmap entries of the terms-3+4 plan: output block index, with this bit set for the blocks of
 // weight 1 (rep3 = 2), half the plan's weight; Src flags of the Z plan: pair index, with this bit
-// set for the pairs of weight 1/2 beside pairs of weight 1 (on-site pairs when Z is halved)
+// set for the pairs (B, G') of weight 1/2 (wZ = 2)
 constexpr int32_t XHALF = 1 << 30;
 
 // One problem of a batched launch: its packed operands, exponents and the
@@ -1000,7 +1000,7 @@ extern "C" rix_status rix_test_stalled_gemm(rix_ctx *ctx, int64_t wait_ns, void 
 //     columns (E', l) over G's neighbours E' != G;
 //   term 4 intermediate (middle atom G, rows of one block):
 //     Z(B,E')[P][j][l] += w sum_{Q on G, k} V(B,G')[P][Q] D(B,G')[j][k] C(G',E')[Q on G][k][l]
-//       (w = 1/2 over all B, or 1 over one pair of each {B, G'}: rix_ctx::z_half);
+//       (w = 1/2 over all B, or 1 over one pair of each {B, G'}: rix_ctx::wZ);
 //     rows (B, P, j), K = (Q, k), columns (E', l) as for term 2.  The row
 //     operand is the Kronecker product of the V and D blocks, formed while
 //     slicing; this costs about nb_B times the FLOPs of the FP64 grouping, so a
@@ -1613,7 +1613,7 @@ rix_status plan_host(rix_ctx *ctx, int kind, const std::vector<int64_t> &ptrZ, P
             if (kind == 2) {  // rows (P, j) of V(B,G')[P][.] x D(B,G')[j][.]
               const int P = y / nbA, j = y - P * nbA;
               sr = Src{ctx->offV[pq] + (int64_t)P * naB, ctx->offD[pq] + (int64_t)j * nbB, 1, 0, nbB, (int32_t)pq};
-              if (ctx->z_half && ctx->wZ[pq] == 2) sr.flag |= XHALF;
+              if (ctx->wZ[pq] == 2) sr.flag |= XHALF;
             } else if (kind == 0) {  // C(A,B)[naA + P][i][j]
               sr = Src{ctx->offC[pq] + ((int64_t)naA * nbA + y) * nbB, -1, nbA * nbB, 1, nbB, (int32_t)pq};
             } else {  // U2(A,G)[Q][i][k]
@@ -1877,14 +1877,14 @@ int32_t rix_launch_count(const rix_ctx *ctx) {
     // per group: exponents and digits of both operands, then the GEMM
     n += 5 * (int32_t)(ctx->mx34->grp.size() - 1) + 5 * (int32_t)(ctx->mx2->grp.size() - 1) +
          5 * (int32_t)(ctx->mxz->grp.size() - 1) + rix_t1_launches(ctx) + rix_tt_launches(ctx);
-    if (ctx->n_t1tc < ctx->nat) n += ctx->nblk;  // k_X12 for the other column atoms
+    if (ctx->n_t1tc < ctx->nat) n += rix_x12_launches(ctx);  // k_X12 for the other column atoms
     if (ctx->n_ztc == ctx->nat) n -= ctx->nblk;   // no k_Z: the Z buffer is zeroed by a memset
     // row-tile K-stage masks: once per Z block, once per terms-3+4 block, once for term 2
     if (ctx->mxz->n_rt > 0) n += ctx->nblk;
     if (ctx->mx34->n_rt > 0) n += ctx->nblk;
     if (ctx->mx2->n_rt > 0) n++;
   } else {
-    n += 2 * ctx->nblk;  // k_X12, k_X34
+    n += rix_x12_launches(ctx) + rix_x34_launches(ctx) * ctx->nblk;
   }
   return n;
 }
@@ -2019,7 +2019,7 @@ rix_status rix_mixed_x34(rix_ctx *ctx, int blk, int64_t zbase, cudaStream_t st) 
   rt_masks(ctx, pl, ctx->d_keepC, nullptr, false, st);
   for (size_t g = 0; g + 1 < pl->grp.size(); g++) {
     if (pl->grp_blk[g] != blk) continue;
-    // weight 2 (1 for the blocks marked XHALF): see rix_ctx::z_half
+    // weight 2 (1 for the blocks marked XHALF): rix_ctx::rep3
     rix_status s = run_group(ctx, pl, g, rows, cols, ctx->d_offK, ctx->d_X, 0, 2.0, st);
     if (s != RIX_OK) return s;
   }
@@ -2050,7 +2050,7 @@ rix_status rix_mixed_z(rix_ctx *ctx, int blk, int64_t zbase, const double *D, cu
   rt_masks(ctx, pl, ctx->d_keepV, ctx->d_keepD, true, st);
   for (size_t g = 0; g + 1 < pl->grp.size(); g++) {
     if (pl->grp_blk[g] != blk) continue;
-    rix_status s = run_group(ctx, pl, g, rows, cols, ctx->d_off2, ctx->d_Z, zbase, ctx->z_half ? 1.0 : 0.5, st);
+    rix_status s = run_group(ctx, pl, g, rows, cols, ctx->d_off2, ctx->d_Z, zbase, 1.0, st);
     if (s != RIX_OK) return s;
   }
   return RIX_OK;
