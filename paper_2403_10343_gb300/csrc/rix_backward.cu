@@ -12,6 +12,10 @@
 // (Sec. "EXX force and stress contributions"); dE/dC and dE/dV are the
 // quantities those chain through.
 //
+// Terms 1 and 4 are halved by their symmetry as in the build (rep1, wZ; wB and c34 where the
+// build takes Z in full): the half that is left out has the transposed partials, which the
+// symmetrisation at the end adds.
+//
 // Every stored entry is an independent variable for the reverse pass; the
 // results are then symmetrised over transpose partners, which yields the
 // partial derivatives of the four-index formula itself (for symmetric inputs
@@ -38,16 +42,17 @@ struct Win {
 __device__ __forceinline__ bool in_win(const Win &w, int64_t i) { return i >= w.lo && i < w.hi; }
 
 // ---------------------------------------------------------------- Cbar(A,B')[P on B']
-// += sum over (pair (A,E'), Z(B,E')) of sum_l Xbar(A,E')[i][l] Z[P][j][l]
+// += sum over (pair (A,E'), Z(B,E')) of c34(A) sum_l Xbar(A,E')[i][l] Z[P][j][l]
 __global__ void __launch_bounds__(NT) kb_C34(const int4 *items, const int64_t *ptr, const int2 *L, const int32_t *pA,
                                              const int32_t *pB, const int32_t *nb, const int32_t *na,
                                              const double *__restrict__ D, const int64_t *offD,
                                              const double *__restrict__ Z, const int64_t *off2, const int64_t *offC,
-                                             const uint8_t *keepC, double sX, Win w, double *dC) {
+                                             const uint8_t *keepC, const uint8_t *c34, double sX, Win w, double *dC) {
   const int4 it = items[blockIdx.x];
   const int p1 = it.x, p0 = it.y;
   if (!keepC[p1]) return;
   const int a = pA[p1], b = pB[p1];
+  sX *= c34[a];
   const int nbA = nb[a], naA = na[a], nbB = nb[b], naB = na[b];
   const int per = nbA * nbB;
   const int pe = min(naB, p0 + tile_rows(per));
@@ -132,13 +137,13 @@ __global__ void __launch_bounds__(NT) kb_Z34(const int4 *items, const int64_t *p
 }
 
 // ---------------------------------------------------------------- Vbar(B,G') from term 4
-// Fbar[P][k][l] = w sum_j D(B,G')[j][k] Zbar(B,E')[P][j][l] (w: wZ of the pair);  Vbar[P][Q] += sum_kl Fbar C(G',E')[Q on G'][k][l]
+// Fbar[P][k][l] = w sum_j D(B,G')[j][k] Zbar(B,E')[P][j][l] (w: wB of the pair);  Vbar[P][Q] += sum_kl Fbar C(G',E')[Q on G'][k][l]
 __global__ void __launch_bounds__(NT) kb_ZV(const int4 *items, const int64_t *ptr, const int2 *L, const int32_t *pA,
                                             const int32_t *pB, const int32_t *nb, const int32_t *na,
                                             const double *__restrict__ C, const int64_t *offC,
                                             const double *__restrict__ D, const int64_t *offD,
                                             const uint8_t *keepC, const uint8_t *keepV, const uint8_t *keepD,
-                                            const uint8_t *wZ, const double *__restrict__ Zbar, const int64_t *off2,
+                                            const uint8_t *wB, const double *__restrict__ Zbar, const int64_t *off2,
                                             const int64_t *offV, Win win, double *dV) {
   extern __shared__ double sm[];
   const int4 it = items[blockIdx.x];
@@ -150,7 +155,7 @@ __global__ void __launch_bounds__(NT) kb_ZV(const int4 *items, const int64_t *pt
   const int pe = min(naB, p0 + tile_rows(per));
   const int nel = (pe - p0) * per;
   const double *Dbg = D + offD[p2];
-  const double w = wZ[p2] == 2 ? 0.5 : 1.0;
+  const double w = wB[p2] == 2 ? 0.5 : 1.0;
   double acc[MAXE];
 #pragma unroll
   for (int r = 0; r < MAXE; r++) acc[r] = 0.0;
@@ -313,7 +318,8 @@ __global__ void __launch_bounds__(NT) kb_U2(const int4 *items, const int64_t *pt
 }
 
 // ---------------------------------------------------------------- Tbar(A,G')
-// term 1: Ubar1[Q][i][k] = 1/2 sum_l Xbar(A,E')[i][l] C(G',E')[Q on E'][k][l], Tbar += V(A,E') Ubar1
+// term 1: Ubar1[Q][i][k] = w sum_l Xbar(A,E')[i][l] C(G',E')[Q on E'][k][l], Tbar += V(A,E') Ubar1
+// (w: rix_ctx::rep1, 1 for the pairs that stand for both orientations, 1/2 on-site)
 // term 2: Tbar += V(A,G') U2bar(A,G')
 __global__ void __launch_bounds__(NT) kb_T(const int4 *items, const int64_t *ptr, const int2 *L,
                                            const int32_t *atomA2, const int32_t *atomB2, const int32_t *map2to1,
@@ -323,7 +329,7 @@ __global__ void __launch_bounds__(NT) kb_T(const int4 *items, const int64_t *ptr
                                            const double *__restrict__ D, const int64_t *offD,
                                            const uint8_t *keepC, const uint8_t *keepV, const int64_t *ptrU2,
                                            const double *__restrict__ U2bar, const int64_t *offU,
-                                           const int64_t *off2, double sX, Win w, double *Tbar) {
+                                           const int64_t *off2, const uint8_t *rep1, double sX, Win w, double *Tbar) {
   extern __shared__ double sm[];
   const int4 it = items[blockIdx.x];
   const int t = it.x, p0 = it.y;
@@ -346,6 +352,7 @@ __global__ void __launch_bounds__(NT) kb_T(const int4 *items, const int64_t *ptr
     const double *Xb = D + offD[pae];
     const double *Ce = C + offC[en.y] + (int64_t)qE0 * nbG * nbE;
     const double *Vae = V + offV[pae];
+    const double s1 = rep1[pae] == 2 ? 0.5 * sX : sX;
     const int qt = max(1, min(naE, SM_BIG / per));
     for (int q0 = 0; q0 < naE; q0 += qt) {
       const int qn = min(qt, naE - q0);
@@ -357,7 +364,7 @@ __global__ void __launch_bounds__(NT) kb_T(const int4 *items, const int64_t *ptr
         const double *cr = Ce + ((int64_t)(q0 + q) * nbG + k) * nbE;
         double u = 0.0;
         for (int l = 0; l < nbE; l++) u = fma(xr[l], cr[l], u);
-        sm[el] = 0.5 * sX * u;
+        sm[el] = s1 * u;
       }
       __syncthreads();
 #pragma unroll
@@ -407,8 +414,8 @@ __global__ void __launch_bounds__(NT) kb_V12(const int4 *items, const int64_t *p
                                              const uint8_t *keepC, const uint8_t *keepV,
                                              const double *__restrict__ T, const int64_t *off2,
                                              const int64_t *ptrU2, const double *__restrict__ U2bar,
-                                             const int64_t *offU, const int64_t *offV, double sX, Win w,
-                                             double *dV) {
+                                             const int64_t *offU, const int64_t *offV, const uint8_t *rep1,
+                                             double sX, Win w, double *dV) {
   extern __shared__ double sm[];
   const int4 it = items[blockIdx.x];
   const int p = it.x, p0 = it.y;
@@ -425,7 +432,9 @@ __global__ void __launch_bounds__(NT) kb_V12(const int4 *items, const int64_t *p
 #pragma unroll
   for (int r = 0; r < MAXE; r++) acc[r] = 0.0;
   const double *Xb = D + offD[p];
-  for (int64_t x = ptrX12[s]; x < ptrX12[s + 1]; x++) {
+  const double s1 = rep1[p] == 2 ? 0.5 * sX : sX;
+  // term 1 where this pair is the representative orientation
+  for (int64_t x = rep1[p] ? ptrX12[s] : ptrX12[s + 1]; x < ptrX12[s + 1]; x++) {
     const X12Entry en = LX12[x];
     if (!en.t1 || !keepC[en.p3]) continue;
     const int g = pA[en.p3];
@@ -445,7 +454,7 @@ __global__ void __launch_bounds__(NT) kb_V12(const int4 *items, const int64_t *p
         const double *cr = Ce + ((int64_t)(q0 + q) * nbG + k) * nbX;
         double u = 0.0;
         for (int l = 0; l < nbX; l++) u = fma(xr[l], cr[l], u);
-        sm[el] = 0.5 * sX * u;
+        sm[el] = s1 * u;
       }
       __syncthreads();
 #pragma unroll
@@ -490,7 +499,7 @@ __global__ void __launch_bounds__(NT) kb_V12(const int4 *items, const int64_t *p
 }
 
 // ---------------------------------------------------------------- Cbar(G',E') from terms 1 and 2
-// term 1: Cbar[Q on E'][k][l] += 1/2 sum_i U1[Q][i][k] Xbar(A,E')[i][l], U1 = V(A,E')^T T(A,G')
+// term 1: Cbar[Q on E'][k][l] += w sum_i U1[Q][i][k] Xbar(A,E')[i][l], U1 = V(A,E')^T T(A,G')
 // term 2: Cbar[Q on G'][k][l] += sum_i U2(A,G')[Q][i][k] Xbar(A,E')[i][l]
 __global__ void __launch_bounds__(NT) kb_C12(const int4 *items, const int64_t *ptr, const BX12Entry *L,
                                              const int32_t *atomA2, const int32_t *map2to1, const int32_t *pA,
@@ -500,7 +509,8 @@ __global__ void __launch_bounds__(NT) kb_C12(const int4 *items, const int64_t *p
                                              const uint8_t *keepC, const uint8_t *keepV,
                                              const double *__restrict__ T, const int64_t *off2,
                                              const double *__restrict__ U, const int64_t *offU,
-                                             const int64_t *offC, double sX, Win w, double *dC) {
+                                             const int64_t *offC, const uint8_t *rep1, double sX, Win w,
+                                             double *dC) {
   extern __shared__ double sm[];
   const int4 it = items[blockIdx.x];
   const int p3 = it.x, r0 = it.y;
@@ -529,6 +539,7 @@ __global__ void __launch_bounds__(NT) kb_C12(const int4 *items, const int64_t *p
       const int uper = nbA * nbG;
       const double *Tt = T + (off2[en.t] - w.base);
       const double *Vae = V + offV[pae];
+      const double s1 = rep1[pae] == 2 ? 0.5 * sX : sX;
       const int qn = q1hi - q1lo;
       __syncthreads();
       for (int el = threadIdx.x; el < qn * uper; el += NT) {
@@ -549,7 +560,7 @@ __global__ void __launch_bounds__(NT) kb_C12(const int4 *items, const int64_t *p
             const double *ur = sm + q * uper + k;
             double v = 0.0;
             for (int i = 0; i < nbA; i++) v = fma(ur[i * nbG], Xb[i * nbE + l], v);
-            acc[r] = fma(0.5 * sX, v, acc[r]);
+            acc[r] = fma(s1, v, acc[r]);
           }
         }
       }
@@ -759,21 +770,22 @@ extern "C" rix_status rix_backward(rix_ctx *ctx, const double *D, double gEx, do
       kb_C12<<<(unsigned)ctx->n_itB[7], NT, SM_BIG * 8, st>>>(
           ctx->d_itB[7], ctx->d_ptrBC12, ctx->d_LBC12, ctx->d_atomA2, ctx->d_map2to1, ctx->d_pA, ctx->d_pB,
           ctx->d_onsite, ctx->d_nb, ctx->d_na, ctx->d_V, ctx->d_offV, D, ctx->d_offD, ctx->d_keepC, ctx->d_keepV,
-          ctx->d_T, ctx->d_off2, ctx->d_U, ctx->d_offU, ctx->d_offC, sX, w, dC);
+          ctx->d_T, ctx->d_off2, ctx->d_U, ctx->d_offU, ctx->d_offC, ctx->d_rep1, sX, w, dC);
       if ((s = last_err(ctx, "kb_C12")) != RIX_OK) return s;
     }
     if (dV && ctx->n_itB[6]) {
       kb_V12<<<(unsigned)ctx->n_itB[6], NT, SM_BIG * 8, st>>>(
           ctx->d_itB[6], ctx->d_ptrX12, ctx->d_LX12, ctx->d_map1to2, ctx->d_pA, ctx->d_pB, ctx->d_onsite, ctx->d_nb,
           ctx->d_na, ctx->d_C, ctx->d_offC, D, ctx->d_offD, ctx->d_keepC, ctx->d_keepV, ctx->d_T, ctx->d_off2,
-          ctx->d_ptrBU2, ctx->d_U2bar, ctx->d_offU, ctx->d_offV, sX, w, dV);
+          ctx->d_ptrBU2, ctx->d_U2bar, ctx->d_offU, ctx->d_offV, ctx->d_rep1, sX, w, dV);
       if ((s = last_err(ctx, "kb_V12")) != RIX_OK) return s;
     }
     if (dC && ctx->n_itB[5]) {
       kb_T<<<(unsigned)ctx->n_itB[5], NT, SM_BIG * 8, st>>>(
           ctx->d_itB[5], ctx->d_ptrBT1, ctx->d_LBT1, ctx->d_atomA2, ctx->d_atomB2, ctx->d_map2to1, ctx->d_pA,
           ctx->d_onsite, ctx->d_nb, ctx->d_na, ctx->d_C, ctx->d_offC, ctx->d_V, ctx->d_offV, D, ctx->d_offD,
-          ctx->d_keepC, ctx->d_keepV, ctx->d_ptrBU2, ctx->d_U2bar, ctx->d_offU, ctx->d_off2, sX, w, ctx->d_T);
+          ctx->d_keepC, ctx->d_keepV, ctx->d_ptrBU2, ctx->d_U2bar, ctx->d_offU, ctx->d_off2, ctx->d_rep1, sX, w,
+          ctx->d_T);
       if ((s = last_err(ctx, "kb_T")) != RIX_OK) return s;
       if (ctx->n_itB[8]) {
         kb_TC<<<(unsigned)ctx->n_itB[8], NT, 0, st>>>(ctx->d_itB[8], ctx->d_ptrBTC, ctx->d_LBTC, ctx->d_pA,
@@ -790,7 +802,7 @@ extern "C" rix_status rix_backward(rix_ctx *ctx, const double *D, double gEx, do
     if (dC && ctx->n_itB[0]) {
       kb_C34<<<(unsigned)ctx->n_itB[0], NT, 0, st>>>(ctx->d_itB[0], ctx->d_ptrBC34, ctx->d_LBC34, ctx->d_pA,
                                                      ctx->d_pB, ctx->d_nb, ctx->d_na, D, ctx->d_offD, ctx->d_Z,
-                                                     ctx->d_off2, ctx->d_offC, ctx->d_keepC, sX, w, dC);
+                                                     ctx->d_off2, ctx->d_offC, ctx->d_keepC, ctx->d_c34, sX, w, dC);
       if ((s = last_err(ctx, "kb_C34")) != RIX_OK) return s;
     }
     if (ctx->n_itB[1]) {
@@ -810,7 +822,7 @@ extern "C" rix_status rix_backward(rix_ctx *ctx, const double *D, double gEx, do
     if (dV && ctx->n_itB[2]) {
       kb_ZV<<<(unsigned)ctx->n_itB[2], NT, SM_BIG * 8, st>>>(
           ctx->d_itB[2], ctx->d_ptrBZV, ctx->d_LBZV, ctx->d_pA, ctx->d_pB, ctx->d_nb, ctx->d_na, ctx->d_C,
-          ctx->d_offC, D, ctx->d_offD, ctx->d_keepC, ctx->d_keepV, ctx->d_keepD, ctx->d_wZ, ctx->d_Z, ctx->d_off2,
+          ctx->d_offC, D, ctx->d_offD, ctx->d_keepC, ctx->d_keepV, ctx->d_keepD, ctx->d_wB, ctx->d_Z, ctx->d_off2,
           ctx->d_offV, w, dV);
       if ((s = last_err(ctx, "kb_ZV")) != RIX_OK) return s;
     }

@@ -237,6 +237,8 @@ struct rix_ctx {
   int4 *d_itB[9] = {nullptr};                              // tiled work items per backward kernel
   int64_t n_itB[9] = {0};
   double *d_U2bar = nullptr, *d_Kbuf = nullptr;   // Tbar and Zbar reuse the T and Z buffers
+  uint8_t *d_wB = nullptr;    // weights of the pairs (B,G') of dV's term 4: 1, 1/2 (2) or not taken (0)
+  uint8_t *d_c34 = nullptr;   // per atom: weight of its C(A,B') partials of term 4 (1 or 2)
   double bwd_flops = 0;
 
   rix_stats_t stats{};
