@@ -151,8 +151,42 @@ __global__ void k_symcheck(int64_t np, const int32_t *pA, const int32_t *pB, con
   if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(flag, 1);
 }
 
+// ------------------------------------------------------------------ live blocks
+// live[t] = 1 when a product of the list of block t is kept: T(A,G') <- (C(A,B'), D(B',G')) with
+// L the T list, Z(B,E') <- (pair (B,G'), pair (G',E')) with the Z list (keepV given).  The other
+// blocks are zero, and the kernels that read T or Z skip them (in the 24-atom ice cell, whose D
+// reaches a quarter of the pairs, half of the terms-3+4 products).  One warp per block.
+__global__ void k_live(int64_t n, const int64_t *ptr, const int2 *L, const uint8_t *keepC, const uint8_t *keepV,
+                       const uint8_t *keepD, PScreen ps, uint8_t *live) {
+  const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (t >= n) return;
+  bool any = false;
+  for (int64_t e = ptr[t]; e < ptr[t + 1] && !any; e += 32) {
+    bool k = false;
+    if (e + lane < ptr[t + 1]) {
+      const int2 en = L[e + lane];
+      k = keepV ? keepD[en.x] && keepV[en.x] && keepC[en.y] && !ps.drop3(en.x, en.x, en.y)
+                : keepC[en.x] && keepD[en.y] && !ps.drop2(en.x, en.y);
+    }
+    any = __any_sync(0xffffffffu, k);
+  }
+  if (lane == 0) live[t] = any;
+}
+
 // ------------------------------------------------------------------ stage T
-// T(A,G')[P][i][k] for P in [p0, p0+pt): sum over (C(A,B'), D(B',G')) entries.
+// T(A,G')[P][i][k] for P in [p0, p0+pt): sum over (C(A,B'), D(B',G')) entries.  The contraction
+// columns (B', j) of the kept entries are taken TCOL at a time: one warp makes a table of their C
+// offsets, all threads stage the D rows, and every element sums over the whole batch between two
+// barriers (an entry alone is 5 or 14 multiply-adds per element, less than its barriers cost).
+// (H2O)64: 110 -> 82 ms (1.16 TFLOP/s of 1.25).
+constexpr int TCOL = 128;   // columns of a batch at most (an entry has up to 64)
+struct TCols {
+  int64_t c[TCOL], d[TCOL];  // offsets of C(A,B')[0][0][j] and D(B',G')[j][0]
+  int nb[TCOL];              // nb of B' (row stride of C)
+  int n, next;               // columns; entries taken
+};
+
 __global__ void __launch_bounds__(NT) k_T(const int2 *items, const int64_t *ptrT, const int2 *LT,
                                           const int32_t *atomA2, const int32_t *atomB2, const int64_t *off2,
                                           const int32_t *pB, const int32_t *nb, const int32_t *na,
@@ -161,6 +195,7 @@ __global__ void __launch_bounds__(NT) k_T(const int2 *items, const int64_t *ptrT
                                           const uint8_t *keepC, const uint8_t *keepD, double *T,
                                           int64_t tbase, const uint8_t *ttc, int cap, PScreen ps) {
   extern __shared__ double sm[];
+  __shared__ TCols tb;
   const int tid = threadIdx.x;
   const int2 it = items[blockIdx.x];
   const int t = it.x, p0 = it.y;
@@ -174,23 +209,49 @@ __global__ void __launch_bounds__(NT) k_T(const int2 *items, const int64_t *ptrT
   double acc[MAXE];
 #pragma unroll
   for (int r = 0; r < MAXE; r++) acc[r] = 0.0;
-  for (int64_t e = ptrT[t]; e < ptrT[t + 1]; e++) {
-    const int2 en = LT[e];
-    if (!keepC[en.x] || !keepD[en.y] || ps.drop2(en.x, en.y)) continue;
-    const int nbB = nb[pB[en.x]];
-    const double *Dg = D + offD[en.y];
+  for (int64_t e = ptrT[t]; e < ptrT[t + 1];) {
     __syncthreads();
-    for (int i = tid; i < nbB * nbG; i += NT) sm[i] = Dg[i];
+    if (tid < 32) {
+      const bool in = e + tid < ptrT[t + 1];
+      const int2 en = LT[in ? e + tid : e];
+      const int w = in && keepC[en.x] && keepD[en.y] && !ps.drop2(en.x, en.y) ? nb[pB[en.x]] : 0;
+      int s = w;  // columns up to and including this entry's
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, s, o);
+        if (tid >= o) s += v;
+      }
+      const int take = __popc(__ballot_sync(0xffffffffu, in && s <= TCOL));
+      if (tid < take) {
+        const int64_t c0 = offC[en.x] + (int64_t)p0 * nbA * w, d0 = offD[en.y];
+        for (int j = 0; j < w; j++) {
+          tb.c[s - w + j] = c0 + j;
+          tb.d[s - w + j] = d0 + j * nbG;
+          tb.nb[s - w + j] = w;
+        }
+      }
+      if (tid == take - 1) {
+        tb.n = s;
+        tb.next = take;
+      }
+    }
     __syncthreads();
-    const double *Cr = C + offC[en.x] + (int64_t)p0 * nbA * nbB;
+    const int n = tb.n;
+    e += tb.next;
+    if (n == 0) continue;
+    for (int i = tid; i < n * nbG; i += NT) {
+      const int c = i / nbG;
+      sm[i] = __ldg(D + tb.d[c] + (i - c * nbG));
+    }
+    __syncthreads();
 #pragma unroll
     for (int r = 0; r < MAXE; r++) {
       const int el = tid + r * NT;
       if (el < nel) {
-        const int row = el / nbG, col = el - row * nbG;
-        const double *cr = Cr + (int64_t)row * nbB;
+        const int row = el / nbG;
+        const double *dc = sm + (el - row * nbG);
         double s = acc[r];
-        for (int j = 0; j < nbB; j++) s = fma(__ldg(cr + j), sm[j * nbG + col], s);
+#pragma unroll 4
+        for (int c = 0; c < n; c++) s = fma(__ldg(C + tb.c[c] + row * tb.nb[c]), dc[c * nbG], s);
         acc[r] = s;
       }
     }
@@ -350,12 +411,12 @@ struct XCols {
 __device__ __forceinline__ void x12_batch(XCols &tb, int64_t it, int64_t end, int maxcol, const X12Entry *L,
                                           const uint8_t *keepC, const int32_t *pA, const int32_t *nb,
                                           const int32_t *na, const uint8_t *onsite, const int64_t *off2,
-                                          int64_t tbase, const int64_t *offC, int nbE) {
+                                          int64_t tbase, const int64_t *offC, int nbE, const uint8_t *liveT) {
   const int lane = threadIdx.x & 31;
   const bool in = it + lane < end;
   const X12Entry en = L[in ? it + lane : it];
   const int g = pA[en.p3];
-  const int w = in && en.t1 && keepC[en.p3] ? nb[g] : 0;
+  const int w = in && en.t1 && keepC[en.p3] && !(liveT && !liveT[en.t]) ? nb[g] : 0;
   int s = w;  // columns up to and including this entry's
   for (int o = 1; o < 32; o <<= 1) {
     const int v = __shfl_up_sync(0xffffffffu, s, o);
@@ -384,7 +445,7 @@ __global__ void __launch_bounds__(NT, R == 1 ? 4 : 1)
           const int32_t *na, const double *__restrict__ C, const int64_t *offC, const double *__restrict__ V,
           const int64_t *offV, const uint8_t *keepC, const uint8_t *keepV, const double *__restrict__ T,
           const int64_t *off2, const double *__restrict__ U, const int64_t *offU, const int64_t *offK, double *X,
-          int64_t tbase, int smb, int t2, const uint8_t *t1tc, const uint8_t *rep1, int ns) {
+          int64_t tbase, int smb, int t2, const uint8_t *t1tc, const uint8_t *rep1, const uint8_t *liveT, int ns) {
   extern __shared__ double sm[];
   __shared__ XCols tb;
   const int tid = threadIdx.x;
@@ -410,7 +471,8 @@ __global__ void __launch_bounds__(NT, R == 1 ? 4 : 1)
     for (int64_t it = ptr[s]; it < ptr[s + 1];) {
       __syncthreads();
       if (tid < 32)
-        x12_batch(tb, it, ptr[s + 1], min(XCOL, smb / nbA), L, keepC, pA, nb, na, onsite, off2, tbase, offC, nbE);
+        x12_batch(tb, it, ptr[s + 1], min(XCOL, smb / nbA), L, keepC, pA, nb, na, onsite, off2, tbase, offC, nbE,
+                  liveT);
       __syncthreads();
       const int n = tb.n;
       it += tb.next;
@@ -469,7 +531,7 @@ __global__ void __launch_bounds__(NT, R == 1 ? 4 : 1)
     // term 2: X += U2(A,G')[Q][i][k] C(G',E')[Q on G'][k][l] (on the tensor cores in mixed precision)
     for (int64_t it = ptr[s]; it < ptr[s + 1]; it++) {
       const X12Entry en = L[it];
-      if (en.u2 < 0 || !keepC[en.p3] || !keepV[en.u2]) continue;
+      if (en.u2 < 0 || !keepC[en.p3] || !keepV[en.u2] || (liveT && !liveT[en.t])) continue;
       const int g = pA[en.p3];
       dot_share<R>(acc, sp, nel, U + offU[en.u2], C + offC[en.p3], na[g], nbA, nb[g], nbE);
     }
@@ -561,7 +623,7 @@ __global__ void __launch_bounds__(NT, R == 1 ? 6 : 1)
     k_X34(const int32_t *ord, const int64_t *ptr, const int2 *L, const int32_t *atomA3, const int32_t *atomB3,
           const int32_t *pB, const int32_t *nb, const int32_t *na, const double *__restrict__ C, const int64_t *offC,
           const uint8_t *keepC, const double *__restrict__ Z, const int64_t *off2, const int64_t *offK, double *X,
-          int64_t zbase, int64_t zlo, int64_t zhi, const uint8_t *rep3, int ns) {
+          int64_t zbase, int64_t zlo, int64_t zhi, const uint8_t *rep3, const uint8_t *liveZ, int ns) {
   __shared__ double red[R == 1 ? NT : NT * R];
   const int x = ord[blockIdx.x / ns];
   const int rank = blockIdx.x % ns;
@@ -581,7 +643,7 @@ __global__ void __launch_bounds__(NT, R == 1 ? 6 : 1)
   for (int r = 0; r < R; r++) acc[r] = 0.0;
   for (int64_t it = ptr[x]; it < ptr[x + 1]; it++) {
     const int2 en = L[it];
-    if (!keepC[en.x] || en.y < zlo || en.y >= zhi) continue;
+    if (!keepC[en.x] || en.y < zlo || en.y >= zhi || (liveZ && !liveZ[en.y])) continue;
     const int b = pB[en.x];
     const int nbB = nb[b];
     dot_share<R>(acc, sp, nel, C + offC[en.x] + (int64_t)naA * nbA * nbB, Z + (off2[en.y] - zbase), na[b], nbA, nbB,
@@ -616,32 +678,39 @@ __global__ void k_sym(int64_t nk, const int32_t *atomA3, const int32_t *atomB3, 
 }
 
 // ------------------------------------------------------------------ energy
-// Pair p contributes sum_il D(B,A,-n)[l][i] K(A,B,n)[i][l]; each thread owns
-// one pair, each CTA reduces its 256 pairs in a fixed tree.
-__global__ void k_energy(int64_t np, const int32_t *pA, const int32_t *pB, const int32_t *partner,
-                         const int32_t *map1to3, const int32_t *nb, const double *__restrict__ D,
-                         const int64_t *offD, const uint8_t *keepD, const double *__restrict__ K,
-                         const int64_t *offK, double *part) {
-  __shared__ double red[256];
-  const int64_t p = blockIdx.x * (int64_t)256 + threadIdx.x;
+// Pair p contributes sum_il D(B,A,-n)[l][i] K(A,B,n)[i][l].  A CTA takes 256 pairs, eight to a warp
+// (lanes along the block's elements), and adds in a fixed tree.  (A thread per pair read both
+// blocks element by element: 33 us for 576 pairs, 15 us now.)
+constexpr int ENERGY_THREADS = 1024;
+__global__ void __launch_bounds__(ENERGY_THREADS)
+    k_energy(int64_t np, const int32_t *pA, const int32_t *pB, const int32_t *partner, const int32_t *map1to3,
+             const int32_t *nb, const double *__restrict__ D, const int64_t *offD, const uint8_t *keepD,
+             const double *__restrict__ K, const int64_t *offK, double *part) {
+  __shared__ double red[ENERGY_THREADS / 32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double s = 0.0;
-  if (p < np) {
+#pragma unroll
+  for (int j = 0; j < 8; j++) {
+    const int64_t p = blockIdx.x * (int64_t)256 + warp + 32 * j;
+    if (p >= np) continue;
     const int64_t q = partner[p];
-    if (keepD[q]) {
-      const int nbA = nb[pA[p]], nbB = nb[pB[p]];
-      const double *dq = D + offD[q];
-      const double *kb = K + offK[map1to3[p]];
-      for (int i = 0; i < nbA; i++)
-        for (int l = 0; l < nbB; l++) s = fma(dq[l * nbA + i], kb[i * nbB + l], s);
+    if (!keepD[q]) continue;
+    const int nbA = nb[pA[p]], nbB = nb[pB[p]];
+    const double *dq = D + offD[q];
+    const double *kb = K + offK[map1to3[p]];
+    for (int el = lane; el < nbA * nbB; el += 32) {
+      const int i = el / nbB, l = el - i * nbB;
+      s = fma(dq[l * nbA + i], kb[el], s);
     }
   }
-  red[threadIdx.x] = s;
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) red[warp] = s;
   __syncthreads();
-  for (int w = 128; w; w >>= 1) {
-    if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
+  if (warp == 0) {
+    s = red[lane];
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) part[blockIdx.x] = s;
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = red[0];
 }
 
 // *Ex = scale * sum(part) (accumulate: *Ex += ...); scale -1/4 for the closed-shell energy
@@ -736,6 +805,7 @@ void set_attrs() {
   if (!g_attr_done) {
     cudaFuncSetAttribute(k_X12<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_MAX * 8);
     cudaFuncSetAttribute(k_X12<XMAXE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_MAX * 8);
+    cudaFuncSetAttribute(k_T, cudaFuncAttributeMaxDynamicSharedMemorySize, TCOL * 64 * 8);
     cudaFuncSetAttribute(k_Z, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_MAX * 8);
     g_attr_done = true;
   }
@@ -772,6 +842,17 @@ cudaError_t launch_split(void (*kernel)(P...), int64_t count, int ns, int smem, 
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// the live flags of the T and Z blocks for the current D flags
+rix_status launch_live(rix_ctx *ctx, cudaStream_t st) {
+  if (!ctx->use_live) return RIX_OK;
+  const unsigned grid = (unsigned)((ctx->n2 * 32 + 255) / 256);
+  k_live<<<grid, 256, 0, st>>>(ctx->n2, ctx->d_ptrT, ctx->d_LT, ctx->d_keepC, nullptr, ctx->d_keepD, rix_pscreen(ctx),
+                               ctx->d_live2);
+  k_live<<<grid, 256, 0, st>>>(ctx->n2, ctx->d_ptrZ, ctx->d_LZ, ctx->d_keepC, ctx->d_keepV, ctx->d_keepD,
+                               rix_pscreen(ctx), ctx->d_live2 + ctx->n2);
+  return last(ctx, "k_live");
+}
+
 // outputs of terms 1+2 in block b
 int64_t n_X12(const rix_ctx *ctx, int b) {
   return ctx->segX12[rix_ctx::NCLS * (b + 1)] - ctx->segX12[rix_ctx::NCLS * b];
@@ -791,7 +872,7 @@ rix_status launch_X12_items(rix_ctx *ctx, int b, int64_t first, int64_t count, i
                           ctx->d_nb, ctx->d_na, ctx->d_C, ctx->d_offC, ctx->d_V, ctx->d_offV, ctx->d_keepC,
                           ctx->d_keepV, ctx->d_T, ctx->d_off2, ctx->d_U, ctx->d_offU, ctx->d_offK, ctx->d_X,
                           ctx->blk_base[b], smb, ctx->have_mx ? 0 : 1, ctx->have_mx ? ctx->d_t1tc : nullptr,
-                          ctx->d_rep1, 1 << c);
+                          ctx->d_rep1, ctx->use_live ? ctx->d_live2 : nullptr, 1 << c);
     };
     cudaError_t e = go(k_X12<1>);
     if (e == cudaSuccess && ctx->max_nel > NT) e = go(k_X12<XMAXE>);
@@ -810,7 +891,7 @@ rix_status launch_X34(rix_ctx *ctx, int b, cudaStream_t st) {
       return launch_split(kernel, n, 1 << c, 0, st, ctx->d_ordX34 + lo, ctx->d_ptrX34, ctx->d_LX34, ctx->d_atomA3,
                           ctx->d_atomB3, ctx->d_pB, ctx->d_nb, ctx->d_na, ctx->d_C, ctx->d_offC, ctx->d_keepC,
                           ctx->d_Z, ctx->d_off2, ctx->d_offK, ctx->d_X, ctx->blk_base[b], zlo, zhi, ctx->d_rep3,
-                          1 << c);
+                          ctx->use_live ? ctx->d_live2 + ctx->n2 : nullptr, 1 << c);
     };
     cudaError_t e = go(k_X34<1>);
     if (e == cudaSuccess && ctx->max_nel > NT) e = go(k_X34<XMAXE>);
@@ -838,6 +919,7 @@ int32_t rix_x34_launches(const rix_ctx *ctx) {
 // precision the buffer is cleared first and the tensor cores add the T blocks
 // of their row atoms; k_T stores the others.
 rix_status rix_launch_T_block(rix_ctx *ctx, const double *D, int b, cudaStream_t st) {
+  set_attrs();
   const int64_t nT = ctx->segT[b + 1] - ctx->segT[b];
   const bool tc = ctx->have_mx && ctx->n_ttc > 0;
   if (tc) {
@@ -845,7 +927,7 @@ rix_status rix_launch_T_block(rix_ctx *ctx, const double *D, int b, cudaStream_t
     RIX_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_T, 0, sizeof(double) * n, st));
   }
   if (nT) {
-    k_T<<<(unsigned)nT, NT, 64 * 64 * 8, st>>>(ctx->d_itT + ctx->segT[b], ctx->d_ptrT, ctx->d_LT, ctx->d_atomA2,
+    k_T<<<(unsigned)nT, NT, TCOL * ctx->max_nb * 8, st>>>(ctx->d_itT + ctx->segT[b], ctx->d_ptrT, ctx->d_LT, ctx->d_atomA2,
                                                ctx->d_atomB2, ctx->d_off2, ctx->d_pB, ctx->d_nb, ctx->d_na,
                                                ctx->d_C, ctx->d_offC, D, ctx->d_offD, ctx->d_keepC, ctx->d_keepD,
                                                ctx->d_T, ctx->blk_base[b], tc ? ctx->d_ttc : nullptr, ctx->cap_T,
@@ -876,6 +958,7 @@ rix_status rix_fp64_build(rix_ctx *ctx, const double *D, double *K, cudaStream_t
   rix_status s;
   if ((s = rix_prof_mark(ctx, 0, st)) != RIX_OK) return s;
   if ((s = rix_launch_flags(ctx, D, ctx->d_offD, ctx->np, ctx->d_keepD, st, ctx->d_normD)) != RIX_OK) return s;
+  if ((s = launch_live(ctx, st)) != RIX_OK) return s;
   if ((s = rix_prof_mark(ctx, 1, st)) != RIX_OK) return s;
   RIX_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_X, 0, sizeof(double) * ctx->offK[ctx->nk], st));
   if (ctx->d_X128)
@@ -1004,6 +1087,7 @@ extern "C" rix_status rix_autotune(rix_ctx *ctx, const double *D, const char *ca
   rix_status s;
   set_attrs();
   if ((s = rix_launch_flags(ctx, D, ctx->d_offD, ctx->np, ctx->d_keepD, st)) != RIX_OK) return s;
+  if ((s = launch_live(ctx, st)) != RIX_OK) return s;
   RIX_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_X, 0, sizeof(double) * ctx->offK[ctx->nk], st));
   const int b = 0;
   const int64_t SAMPLE = 4096;
@@ -1043,7 +1127,7 @@ extern "C" rix_status rix_autotune(rix_ctx *ctx, const double *D, const char *ca
 rix_status rix_launch_energy(rix_ctx *ctx, const double *D, const double *K, double *Ex, cudaStream_t st) {
   rix_status s;
   if ((s = rix_launch_flags(ctx, D, ctx->d_offD, ctx->np, ctx->d_keepD, st)) != RIX_OK) return s;
-  k_energy<<<(unsigned)ctx->n_epart, 256, 0, st>>>(ctx->np, ctx->d_pA, ctx->d_pB, ctx->d_partner1, ctx->d_map1to3,
+  k_energy<<<(unsigned)ctx->n_epart, ENERGY_THREADS, 0, st>>>(ctx->np, ctx->d_pA, ctx->d_pB, ctx->d_partner1, ctx->d_map1to3,
                                                    ctx->d_nb, D, ctx->d_offD, ctx->d_keepD, K, ctx->d_offK,
                                                    ctx->d_epart);
   if ((s = last(ctx, "k_energy")) != RIX_OK) return s;
@@ -1056,7 +1140,7 @@ rix_status rix_launch_energy_scaled(rix_ctx *ctx, const double *D, const double 
                                     int accumulate, cudaStream_t st) {
   rix_status s;
   if ((s = rix_launch_flags(ctx, D, ctx->d_offD, ctx->np, ctx->d_keepD, st)) != RIX_OK) return s;
-  k_energy<<<(unsigned)ctx->n_epart, 256, 0, st>>>(ctx->np, ctx->d_pA, ctx->d_pB, ctx->d_partner1, ctx->d_map1to3,
+  k_energy<<<(unsigned)ctx->n_epart, ENERGY_THREADS, 0, st>>>(ctx->np, ctx->d_pA, ctx->d_pB, ctx->d_partner1, ctx->d_map1to3,
                                                    ctx->d_nb, D, ctx->d_offD, ctx->d_keepD, K, ctx->d_offK,
                                                    ctx->d_epart);
   if ((s = last(ctx, "k_energy")) != RIX_OK) return s;
@@ -1070,7 +1154,7 @@ rix_status rix_launch_energy_partials(rix_ctx *ctx, const double *D, const doubl
                                       cudaStream_t st) {
   rix_status s;
   if ((s = rix_launch_flags(ctx, D, ctx->d_offD, ctx->np, ctx->d_keepD, st)) != RIX_OK) return s;
-  k_energy<<<(unsigned)ctx->n_epart, 256, 0, st>>>(ctx->np, ctx->d_pA, ctx->d_pB, ctx->d_partner1, ctx->d_map1to3,
+  k_energy<<<(unsigned)ctx->n_epart, ENERGY_THREADS, 0, st>>>(ctx->np, ctx->d_pA, ctx->d_pB, ctx->d_partner1, ctx->d_map1to3,
                                                    ctx->d_nb, D, ctx->d_offD, ctx->d_keepD, K, ctx->d_offK,
                                                    partials);
   if ((s = last(ctx, "k_energy")) != RIX_OK) return s;

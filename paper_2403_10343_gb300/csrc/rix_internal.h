@@ -247,10 +247,13 @@ struct rix_ctx {
   // stays as it is: k_X34 stages nothing)
   int32_t tile_X12 = 4096, tile_Z = 12288, tile_X34 = 4096;
   // Launch classes of k_X12 and k_X34: class c holds the outputs shared by a cluster of 2^c CTAs
-  // (segX12[4 b + c] .. of block b, segX34[c] ..); max_nel: the largest K block (elements)
+  // (segX12[4 b + c] .. of block b, segX34[c] ..); max_nel, max_nb: the largest K block (elements) and atom (functions)
   static constexpr int NCLS = 4;
   std::vector<int64_t> segX34;
-  int32_t max_nel = 0;
+  int32_t max_nel = 0, max_nb = 0;
+  // FP64 builds with screening: per build, whether each T and Z block ([n2] each) has a kept product
+  bool use_live = false;
+  uint8_t *d_live2 = nullptr;
   // connected component of the pair list of every atom.  What changes the order of a sum is
   // decided per component, so that systems batched in one context (batch.py) give the bits that
   // each gives alone.

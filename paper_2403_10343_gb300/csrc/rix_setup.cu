@@ -775,7 +775,8 @@ static rix_status build_lists(rix_ctx *ctx) {
     return cls;
   };
   const std::vector<int> cls12 = clusters(ordX12, cX12, [&](int32_t s) { return atomA2[s]; });
-  for (int a = 0; a < nat; a++) ctx->max_nel = std::max(ctx->max_nel, (int32_t)(NB(a) * NB(a)));
+  for (int a = 0; a < nat; a++) ctx->max_nb = std::max(ctx->max_nb, ctx->nb_at[a]);
+  ctx->max_nel = ctx->max_nb * ctx->max_nb;
   {
     std::vector<int64_t> idx(ordX12.size());
     std::iota(idx.begin(), idx.end(), 0);
@@ -863,6 +864,8 @@ static rix_status build_lists(rix_ctx *ctx) {
                          (signed char)key_n(keys3[x], 2), 0);
     TRY(rix_upload(ctx, &ctx->d_n3, n3));
   }
+  ctx->use_live = ctx->opt.precision != RIX_MIXED_BF16 && (ctx->tau > 0 || ctx->opt.product_tau > 0);
+  if (ctx->use_live) TRY(rix_alloc(ctx, &ctx->d_live2, 2 * n2));
   TRY(rix_alloc(ctx, &ctx->d_U, offU[np]));
   TRY(rix_alloc(ctx, &ctx->d_X, ctx->offK[nk]));
   ctx->n_epart = (np + 255) / 256;

@@ -1872,7 +1872,7 @@ rix_status rix_mixed_plan(rix_ctx *ctx, const std::vector<int64_t> &ptrZ) {
 // terms 3+4 (FP64 per block) or per group four slicing kernels and a GEMM
 // (mixed), symmetrise.
 int32_t rix_launch_count(const rix_ctx *ctx) {
-  int32_t n = 2 + 3 * ctx->nblk;
+  int32_t n = 2 + 3 * ctx->nblk + (ctx->use_live ? 2 : 0);
   if (ctx->have_mx) {
     // per group: exponents and digits of both operands, then the GEMM
     n += 5 * (int32_t)(ctx->mx34->grp.size() - 1) + 5 * (int32_t)(ctx->mx2->grp.size() - 1) +
