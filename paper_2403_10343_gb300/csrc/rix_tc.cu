@@ -29,8 +29,8 @@
 // Kernel layout: persistent CTAs over 128 x 80 output tiles; warp 0 issues the
 // bulk copies (cp.async.bulk, mbarrier completion), one thread of warp 1
 // issues tcgen05.mma (A and B from shared memory, accumulators in tensor
-// memory), warps 4-11 drain tensor memory (tcgen05.ld, two warps per 32-lane
-// quadrant, 40 columns each) into the fixed-point sums.  Every wait is
+// memory), warps 4-19 drain tensor memory (tcgen05.ld, four warps per 32-lane
+// quadrant, 20 columns each) into the fixed-point sums.  Every wait is
 // bounded; on a timeout the kernel records an error and returns.
 #include <cuda_bf16.h>
 
@@ -44,12 +44,12 @@ namespace rixtc {
 
 constexpr int TM = 128;         // output rows per tile (one TMEM lane each)
 constexpr int TN = 80;          // output columns per tile
-constexpr int KC = 32;          // K per pipeline stage (two MMA K steps)
-// Accumulation groups of GROUP K stages (512 K values).  Accumulator a < NACC-1
+constexpr int KC = 16;          // K per pipeline stage (one MMA K step)
+// Accumulation groups of GROUP K stages (576 K values, the most that stays exact).  Accumulator a < NACC-1
 // holds diagonal a: pairs (0, a) and (a, 0) with a leading digit (<= 128)
 // and a balanced one (<= 64), and a - 1 pairs of balanced digits (a = 0: the
 // one pair of leading digits), so its sum stays an integer below 2^24.
-constexpr int GROUP = 16;
+constexpr int GROUP = 36;
 constexpr int64_t diag_bound(int a) {  // largest |sum over one K value| of diagonal a
   return a == 0 ? 128 * 128 : 2 * 128 * 64 + (int64_t)(a - 1) * 64 * 64;
 }
@@ -57,30 +57,39 @@ constexpr bool exact_group(int a) { return diag_bound(a) * GROUP * KC < ((int64_
 static_assert(exact_group(0) && exact_group(1) && exact_group(2) && exact_group(3) && exact_group(4),
               "accumulation groups must stay exact");
 constexpr int NACC = 6;         // accumulators: s+t = 2 .. 6 and s+t >= 7 (480 TMEM columns)
-constexpr int NTHR = 384;       // warps 0-3: copies, MMA, TMEM allocation; warps 4-11: drain
+// Sixteen drain warps (4-19, four to a 32-lane quadrant of tensor memory, 20 columns each): with
+// eight of 40 columns both the fold (11.5k against 8.9k clocks, during which the MMAs wait) and the
+// scatter epilogue were bound by the latency of two warps per scheduler ((H2O)64 build, GEMM
+// launches 88 and 64 ms).
+constexpr int DRAIN_WARPS = 16;
+constexpr int NTHR = 128 + 32 * DRAIN_WARPS;  // warps 0-3: copies, MMA, TMEM allocation
 constexpr int MAXS = 8;         // slices supported
 constexpr uint64_t WAIT_NS = 2000000000ull;  // a wait gives up after 2 s
 
 // bytes of one packed tile (no-swizzle K-major core matrices, 8 rows x 16 B)
-constexpr int A_TILE = TM * KC * 2;  // 8 KB
-constexpr int B_TILE = TN * KC * 2;  // 5 KB
+constexpr int A_TILE = TM * KC * 2;  // 4 KB
+constexpr int B_TILE = TN * KC * 2;  // 2.5 KB
 
-constexpr int NSTAGE = 3;            // pipeline stages when they fit in shared memory
+// Pipeline stages, as many as shared memory holds (five at six slices, six at five).  The tiles of
+// all slices of a K stage lie back to back in memory and in shared memory, so a stage is two bulk
+// copies.  (32-wide stages, two of which fit at six slices, left the MMAs 450 of 3,280 clocks per
+// stage waiting for copies.)
+constexpr int NSTAGE = 6;
 constexpr int SMEM_LIMIT = 227 * 1024;
 // Scatter epilogue staging: per drain warp 32 rows x EPI_CW values plus each row's
 // output-block base and in-block row offset
-constexpr int EPI_CW = 4;
+constexpr int EPI_CW = 2;
 constexpr int EPI_WARP_BYTES = 32 * EPI_CW * 8 + 32 * 8 + 32 * 4;
-constexpr int EPI_BYTES = 8 * EPI_WARP_BYTES;
+constexpr int EPI_BYTES = DRAIN_WARPS * EPI_WARP_BYTES;
 
 // stages that fit for S slices, and the dynamic shared memory they need
 __host__ __device__ inline int n_stages(int S) {
   const int st = S * (A_TILE + B_TILE);
   const int fit = (SMEM_LIMIT - 256 - EPI_BYTES) / st;
-  return fit >= NSTAGE ? NSTAGE : (fit >= 2 ? fit : 1);
+  return fit >= NSTAGE ? NSTAGE : fit;
 }
 __host__ __device__ inline int smem_bytes(int S) {
-  return n_stages(S) * S * (A_TILE + B_TILE) + EPI_BYTES + 8 * (2 * NSTAGE + 4) + 16;
+  return n_stages(S) * S * (A_TILE + B_TILE) + EPI_BYTES + 8 * (2 * NSTAGE + 4) + 4 * NSTAGE + 16;
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -106,11 +115,13 @@ __device__ __forceinline__ uint64_t now_ns() {
   return t;
 }
 
-// bounded wait for the phase with the given parity; returns false after WAIT_NS.
+// bounded wait for the phase with the given parity; returns false after WAIT_NS, or once *stop
+// (another role gave up) is set.
 // try_wait may suspend the thread for up to SUSPEND_NS until the phase completes,
 // so waiting warps leave the issue slots to the copy and MMA threads.
 constexpr uint32_t SUSPEND_NS = 20000;
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint64_t limit_ns = WAIT_NS) {
+__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint64_t limit_ns = WAIT_NS,
+                                          const volatile int *stop = nullptr) {
   const uint32_t a = smem_u32(bar);
   uint64_t t0 = 0;
   while (true) {
@@ -121,6 +132,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint64
         : "r"(a), "r"(parity), "r"(SUSPEND_NS)
         : "memory");
     if (ok) return true;
+    if (stop && *stop) return false;
     const uint64_t t = now_ns();
     if (!t0) t0 = t;
     else if (t - t0 > limit_ns) return false;
@@ -164,7 +176,7 @@ __host__ __device__ constexpr int run_width(int left) {  // next run of `left` s
 }
 
 // The MMAs of one K stage: slice pairs (s, u) with s + u < S, each into
-// accumulator min(s + u, NACC - 1), two K steps of 16.  The B tiles of
+// accumulator min(s + u, NACC - 1).  The B tiles of
 // consecutive slices lie back to back in shared memory (one K-major matrix of
 // 80 rows per slice) and their accumulators s + u, s + u + 1, ... back to back
 // in tensor memory, so one MMA with N = 80 w columns multiplies A slice s by w
@@ -176,10 +188,11 @@ __host__ __device__ constexpr int run_width(int left) {  // next run of `left` s
 // ad0 / bd0 are the descriptors of slice 0 of the stage; the others follow at
 // fixed offsets (the start-address field counts 16-byte units and stays below
 // 2^14 in shared memory).  With open set (a group of accumulations starts at
-// this stage) the MMAs of A slice 0 and the first K step overwrite their
-// accumulators; they come first and cover all of them.
+// this stage) the MMAs of A slice 0 overwrite their accumulators; they come
+// first and cover all of them.
 template <int S>
 __device__ __forceinline__ void issue_stage(uint32_t tmem, uint64_t ad0, uint64_t bd0, uint32_t open) {
+  static_assert(KC == 16, "one MMA K step per stage");
 #pragma unroll
   for (int s = 0; s < S; s++) {
     const int top = S < NACC ? S : NACC;  // accumulators in use
@@ -187,51 +200,103 @@ __device__ __forceinline__ void issue_stage(uint32_t tmem, uint64_t ad0, uint64_
 #pragma unroll
     for (int u = 0; u < nu; u += run_width(nu - u)) {
       const int w = run_width(nu - u);
-#pragma unroll
-      for (int kk = 0; kk < KC / 16; kk++)
-        mma_bf16(tmem + (uint32_t)((s + u) * TN), ad0 + (uint64_t)((s * A_TILE + kk * 256) >> 4),
-                 bd0 + (uint64_t)((u * B_TILE + kk * 256) >> 4), idesc_bf16(TM, w * TN),
-                 s == 0 && kk == 0 ? 1u - open : 1u);
+      mma_bf16(tmem + (uint32_t)((s + u) * TN), ad0 + (uint64_t)((s * A_TILE) >> 4),
+               bd0 + (uint64_t)((u * B_TILE) >> 4), idesc_bf16(TM, w * TN), s == 0 ? 1u - open : 1u);
     }
 #pragma unroll
     for (int u = nu > 0 ? nu : 0; u < S - s; u++)
-#pragma unroll
-      for (int kk = 0; kk < KC / 16; kk++)
-        mma_bf16(tmem + (uint32_t)((NACC - 1) * TN), ad0 + (uint64_t)((s * A_TILE + kk * 256) >> 4),
-                 bd0 + (uint64_t)((u * B_TILE + kk * 256) >> 4), idesc_bf16(TM, TN), 1u);
+      mma_bf16(tmem + (uint32_t)((NACC - 1) * TN), ad0 + (uint64_t)((s * A_TILE) >> 4),
+               bd0 + (uint64_t)((u * B_TILE) >> 4), idesc_bf16(TM, TN), 1u);
   }
 }
 
-__device__ __forceinline__ void issue_stage_s(int S, uint32_t tmem, uint64_t ad0, uint64_t bd0, uint32_t open) {
-  switch (S) {
-    case 1: issue_stage<1>(tmem, ad0, bd0, open); break;
-    case 2: issue_stage<2>(tmem, ad0, bd0, open); break;
-    case 3: issue_stage<3>(tmem, ad0, bd0, open); break;
-    case 4: issue_stage<4>(tmem, ad0, bd0, open); break;
-    case 5: issue_stage<5>(tmem, ad0, bd0, open); break;
-    case 6: issue_stage<6>(tmem, ad0, bd0, open); break;
-    case 7: issue_stage<7>(tmem, ad0, bd0, open); break;
-    default: issue_stage<8>(tmem, ad0, bd0, open); break;
-  }
-}
+__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 __device__ __forceinline__ void mma_commit(uint64_t *bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+// 20 columns of one accumulator (this warp's 32 lanes), asynchronously: the registers hold the
+// values after tmem_wait(r)
+__device__ __forceinline__ void tmem_ld20(uint32_t taddr, uint32_t (&r)[20]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19])
+               : "r"(taddr + 16));
 }
 
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr));
+// waits for the tensor-memory loads of this warp; r is an operand so that its uses stay behind
+__device__ __forceinline__ void tmem_wait(uint32_t (&r)[20]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
+                 "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19])
+               :
+               : "memory");
+}
+
+// What the producer says of a stage beside its data.
+constexpr uint32_t ST_OPEN = 1, ST_LAST = 2, ST_END = 4;  // opens / closes an accumulation group; no more stages
+
+struct MmaRing {
+  uint64_t *full, *empty, *accfull, *accempty;
+  const volatile uint32_t *flags;
+  const volatile int *stop;
+  uint64_t wait_ns;
+  int nst;
+};
+
+// The MMA issuer's loop over the stages of all its CTA's tiles; false if a wait gave up.  What
+// bounds it is the time between a stage's last MMA and the next stage's first one: the tensor
+// pipe has little more than one MMA queued.  So the stage's flags come from the producer
+// through shared memory (no tile records or K-stage masks are read here), the ring position is
+// counted and not divided, and the slice count is a template parameter of the whole loop.
+// (Six slices, dense 19456 x 640 x 1600, clocks per K stage of 16 with 849 of MMAs in it: 1,650 with
+// tile records, divisions and 12 copies per stage, 1,335 now: 582 issuing, 267 waiting for folds,
+// 186 for copies; 1,189 and 1,444 TFLOP/s issued at 1.93 GHz.)
+template <int S>
+__device__ __forceinline__ bool mma_loop(const MmaRing &r, uint32_t tmem, uint32_t sbase, bool &issued) {
+  constexpr uint32_t STAGE = S * (A_TILE + B_TILE);
+  const uint64_t ad = sdesc(sbase, 128, (KC / 8) * 128), bd = sdesc(sbase + S * A_TILE, 128, (KC / 8) * 128);
+  uint32_t gg = 0, ph = 0;  // accumulation groups issued, parity of the ring's round
+  for (int st = 0;;) {
+    if (!mbar_wait(&r.full[st], ph, r.wait_ns, r.stop)) return false;
+    const uint32_t fl = r.flags[st];
+    if (fl & ST_END) return true;
+    if ((fl & ST_OPEN) && gg > 0 && !mbar_wait(r.accempty, (gg - 1) & 1, r.wait_ns, r.stop)) return false;
+    tc_fence_after();
+    const uint64_t so = (uint64_t)(st * (STAGE >> 4));
+    issue_stage<S>(tmem, ad + so, bd + so, fl & ST_OPEN);
+    issued = true;
+    mma_commit(&r.empty[st]);
+    if (fl & ST_LAST) {
+      mma_commit(r.accfull);
+      gg++;
+    }
+    if (++st == r.nst) {
+      st = 0;
+      ph ^= 1;
+    }
+  }
+}
+
+__device__ __forceinline__ bool mma_loop_s(int S, const MmaRing &r, uint32_t tmem, uint32_t sbase, bool &issued) {
+  switch (S) {
+    case 1: return mma_loop<1>(r, tmem, sbase, issued);
+    case 2: return mma_loop<2>(r, tmem, sbase, issued);
+    case 3: return mma_loop<3>(r, tmem, sbase, issued);
+    case 4: return mma_loop<4>(r, tmem, sbase, issued);
+    case 5: return mma_loop<5>(r, tmem, sbase, issued);
+    case 6: return mma_loop<6>(r, tmem, sbase, issued);
+    case 7: return mma_loop<7>(r, tmem, sbase, issued);
+    default: return mma_loop<8>(r, tmem, sbase, issued);
+  }
 }
 
 // An FP32 accumulator value times 2^sh as a 64-bit integer, truncated toward
@@ -250,11 +315,13 @@ __device__ __forceinline__ int64_t f32_fixed(uint32_t b, int sh) {
 }
 
 // Drain of one exactly accumulated diagonal a into the fixed-point sums: the
-// FP32 value is an integer I times 2^-7a with |I| < 2^24, so I = trunc(v 2^7a)
-// is exact in a 32-bit conversion, and I 2^L (L = 7(S-1) - drop - 7a, the same
-// for the whole tile) is added with one 32 x 32 -> 64-bit multiply-add: for
-// 0 <= L <= 37 as (I 2^pre) 2^(L-pre) with pre = max(0, L - 30), both factors
-// within 32 bits (|I 2^pre| < 2^31); other L by a 64-bit shift.
+// FP32 value is an integer I times 2^-7a with |I| < 2^24, and I 2^L (L = 7(S-1)
+// - drop - 7a, the same for the whole tile) is added with one 32 x 32 -> 64-bit
+// multiply-add: for 0 <= L <= 37 as (I 2^pre) 2^(L-pre) with pre = max(0, L - 30),
+// both factors within 32 bits (|I 2^pre| < 2^31); other L by a 64-bit shift.  (The
+// conversion unit takes 16 values per clock and SM, 3,840 clocks for the 61,440
+// values of a fold; splitting part of them exactly on the FP32 pipe instead measured
+// slower.)
 template <int N>
 __device__ __forceinline__ void drain_exact(int64_t *acc, const uint32_t (&r)[N], int a, int L) {
   const float up = __int_as_float((127 + 7 * a) << 23);
@@ -321,10 +388,6 @@ __device__ __forceinline__ double fixed_to_double(int64_t x, int sc) {
   const uint64_t mant = ((ax << lz) >> 11) & ((1ull << 52) - 1);
   return __longlong_as_double((long long)(sgn | ((uint64_t)E << 52) | mant));
 }
-
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 // ------------------------------------------------------------------ packing
 // Byte offset of element (row r, k) inside a packed tile of `rows` rows x KC
@@ -403,7 +466,7 @@ __global__ void k_col_exp(const double *X, int64_t ld, int Kd, int Cn, int Cpad,
 }
 
 // Pack "rows" of an operand into slice tiles.  Element (r, k) is X[r*sr + k*sk].
-// Output: planes[s][rt][kt] tiles of `rows_per_tile` x KC BF16 digits.
+// Output: planes[rt][kt][s] tiles of `rows_per_tile` x KC BF16 digits.
 template <int S>
 __global__ void k_pack(const double *X, int64_t sr, int64_t sk, int R, int Kd, int Rpad, int Kpad, const int *e,
                        int rows_per_tile, __nv_bfloat16 *planes) {
@@ -416,12 +479,11 @@ __global__ void k_pack(const double *X, int64_t sr, int64_t sk, int R, int Kd, i
   digits_of<S>(x, e[r], d);
   const int rt = r / rows_per_tile, kt = k / KC;
   const int64_t tile_bytes = (int64_t)rows_per_tile * KC * 2;
-  const int64_t ntile = (int64_t)(Rpad / rows_per_tile) * (Kpad / KC);
-  const int64_t tbase = ((int64_t)rt * (Kpad / KC) + kt) * tile_bytes + tile_off(r % rows_per_tile, k % KC);
+  const int64_t tbase = ((int64_t)rt * (Kpad / KC) + kt) * S * tile_bytes + tile_off(r % rows_per_tile, k % KC);
   char *base = (char *)planes;
 #pragma unroll
   for (int t = 0; t < S; t++)
-    *(__nv_bfloat16 *)(base + (int64_t)t * ntile * tile_bytes + tbase) = __float2bfloat16_rn(d[t] * slice_scale(t));
+    *(__nv_bfloat16 *)(base + t * tile_bytes + tbase) = __float2bfloat16_rn(d[t] * slice_scale(t));
 }
 
 void launch_pack(const double *X, int64_t sr, int64_t sk, int R, int Kd, int Rpad, int Kpad, const int *e, int S,
@@ -472,8 +534,8 @@ struct QInfo {
 };
 
 struct GemmArgs {
-  const __nv_bfloat16 *A;  // planes [S][Mpad/128][Kpad/32] tiles
-  const __nv_bfloat16 *B;  // planes [S][Npad/64][Kpad/32] tiles
+  const __nv_bfloat16 *A;  // [Mpad/128][Kpad/16][S] tiles
+  const __nv_bfloat16 *B;  // [Npad/80][Kpad/16][S] tiles
   const int *eA, *eB;      // row / column exponents
   double *C;               // output, row-major with ldc
   int64_t ldc;
@@ -540,10 +602,6 @@ struct TileInfo {
   int nlive;                      // number of live K stages
 };
 
-__device__ __forceinline__ bool stage_live(const TileInfo &ti, int c) {
-  return !ti.km || ((ti.km[c >> 6] >> (c & 63)) & 1ull);
-}
-
 __device__ __forceinline__ TileInfo tile_info(const GemmArgs &g, int t) {
   TileInfo ti;
   if (g.tiles) {
@@ -599,7 +657,8 @@ __global__ void __launch_bounds__(NTHR, 1) k_gemm_sliced(GemmArgs g) {
   uint64_t *accempty = accfull + 1;
   uint64_t *mmadone = accempty + 1;  // the MMA issuer's last commit (no MMA in flight at exit)
   uint64_t *never = mmadone + 1;     // completed by nothing: the stall of the timeout test
-  uint32_t *tmem_slot = (uint32_t *)(never + 1);
+  uint32_t *st_flags = (uint32_t *)(never + 1);  // per stage: ST_* for the MMA issuer
+  uint32_t *tmem_slot = st_flags + NSTAGE;
   int *abort_flag = (int *)(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -629,85 +688,63 @@ __global__ void __launch_bounds__(NTHR, 1) k_gemm_sliced(GemmArgs g) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  uint32_t issued_chunks = 0;  // producer thread: chunks whose copies it issued
+  uint32_t issued_chunks = 0;  // producer thread: stages whose copies it issued
+  uint32_t end_posted = 0;     // and whether it posted the stage without data after them
 
   if (warp == 0 && lane == 0) {
     // ------------------------------------------------------------ producer
-    uint32_t cg = 0;  // chunks issued by this CTA
+    uint32_t cg = 0;  // stages issued by this CTA
+    int st = 0;
+    uint32_t ph = 1;  // parity of the ring's previous round (the first one passes at once)
     bool aborted = false;
+    const volatile int *stop = abort_flag;
     for (int t = blockIdx.x; t < ntiles && !aborted; t += gridDim.x) {
       const TileInfo ti = tile_info(g, t);
-      if (!ti.live) continue;  // all-zero rows: no copies (the other roles skip it too)
+      if (!ti.live) continue;  // all-zero rows: no copies (the other roles never see the tile)
       const int nk = ti.Kpad / KC;
-      const int64_t a_tiles = (int64_t)(ti.Mpad / TM) * nk;  // tiles per A plane
-      const int64_t b_tiles = (int64_t)(ti.Npad / TN) * nk;
-      for (int c = 0; c < nk; c++) {
-        if (!stage_live(ti, c)) continue;  // an all-zero B tile: neither copied nor multiplied
-        const int st = cg % nst;
-        if (cg >= (uint32_t)nst && !mbar_wait(&empty[st], ((cg / nst) - 1) & 1, g.wait_ns)) {
-          atomicExch(abort_flag, 1);
-          aborted = true;
-          break;
+      const char *ga = (const char *)ti.gA + (int64_t)ti.mt * nk * (S * A_TILE);
+      const char *gb = (const char *)ti.gB + (int64_t)ti.nt * nk * (S * B_TILE);
+      int lc = 0, gl = 0;  // live stages of the tile so far, and of the open group
+      for (int w = 0; w < (nk + 63) / 64 && !aborted; w++) {
+        unsigned long long m = nk - 64 * w < 64 ? (1ull << (nk - 64 * w)) - 1 : ~0ull;
+        if (ti.km) m &= ti.km[w];  // an all-zero B tile or row block: neither copied nor multiplied
+        for (; m; m &= m - 1) {
+          const int c = 64 * w + __ffsll((long long)m) - 1;
+          if (!mbar_wait(&empty[st], ph, g.wait_ns, stop)) {
+            atomicExch(abort_flag, 1);
+            aborted = true;
+            break;
+          }
+          lc++;
+          st_flags[st] = (gl == 0 ? ST_OPEN : 0u) | (gl == GROUP - 1 || lc == ti.nlive ? ST_LAST : 0u);
+          if (++gl == GROUP) gl = 0;
+          uint8_t *sa = smem + st * stage_bytes;
+          mbar_expect_tx(&full[st], (uint32_t)stage_bytes);
+          bulk_g2s(sa, ga + (int64_t)c * (S * A_TILE), (uint32_t)(S * A_TILE), &full[st]);
+          bulk_g2s(sa + S * A_TILE, gb + (int64_t)c * (S * B_TILE), (uint32_t)(S * B_TILE), &full[st]);
+          cg++;
+          if (++st == nst) {
+            st = 0;
+            ph ^= 1;
+          }
         }
-        if (*(volatile int *)abort_flag) {
-          aborted = true;
-          break;
-        }
-        uint8_t *sa = smem + st * stage_bytes;
-        uint8_t *sb = sa + S * A_TILE;
-        mbar_expect_tx(&full[st], (uint32_t)stage_bytes);
-        for (int s = 0; s < S; s++) {
-          const char *ga = (const char *)ti.gA + ((int64_t)s * a_tiles + (int64_t)ti.mt * nk + c) * A_TILE;
-          bulk_g2s(sa + s * A_TILE, ga, A_TILE, &full[st]);
-          const char *gb = (const char *)ti.gB + ((int64_t)s * b_tiles + (int64_t)ti.nt * nk + c) * B_TILE;
-          bulk_g2s(sb + s * B_TILE, gb, B_TILE, &full[st]);
-        }
-        cg++;
       }
-      if (*(volatile int *)abort_flag) aborted = true;
+    }
+    // one more stage without data: nothing follows
+    if (!aborted && mbar_wait(&empty[st], ph, g.wait_ns, stop)) {
+      st_flags[st] = ST_END;
+      mbar_arrive(&full[st]);
+      end_posted = 1;
     }
     issued_chunks = cg;
     if (g.chunks && cg)
       atomicAdd(g.chunks, (unsigned long long)cg * (unsigned long long)(S * (S + 1) / 2) * (KC / 16));
   } else if (warp == 1 && lane == 0) {
     // ------------------------------------------------------------ MMA issuer
-    uint32_t cg = 0, gg = 0;  // chunks consumed, accumulation groups completed
     bool issued = false;
     if (g.stall && !mbar_wait(never, 0, g.wait_ns)) atomicExch(abort_flag, 1);
-    for (int t = blockIdx.x; t < ntiles && !*(volatile int *)abort_flag; t += gridDim.x) {
-      const TileInfo ti = tile_info(g, t);
-      if (!ti.live) continue;
-      const int nk = ti.Kpad / KC;
-      int lc = 0;  // live K stages issued for this tile
-      for (int c = 0; c < nk; c++) {
-        if (!stage_live(ti, c)) continue;
-        const int st = cg % nst;
-        if (lc % GROUP == 0 && gg > 0 && !mbar_wait(accempty, (gg - 1) & 1, g.wait_ns)) {
-          atomicExch(abort_flag, 1);
-          break;
-        }
-        if (!mbar_wait(&full[st], (cg / nst) & 1, g.wait_ns)) {
-          atomicExch(abort_flag, 1);
-          break;
-        }
-        if (*(volatile int *)abort_flag) break;
-        tc_fence_after();
-        const uint32_t sa = smem_u32(smem + st * stage_bytes);
-        const uint32_t sb = sa + S * A_TILE;
-        // K step kk covers core-matrix columns 2kk, 2kk+1 (LBO = 128 B apart)
-        const uint32_t open = lc % GROUP == 0 ? 1u : 0u;  // every accumulator starts a group
-        issue_stage_s(S, tmem, sdesc(sa, 128, (KC / 8) * 128), sdesc(sb, 128, (KC / 8) * 128), open);
-        issued = true;
-        mma_commit(&empty[st]);
-        if (lc % GROUP == GROUP - 1 || lc == ti.nlive - 1) {
-          mma_commit(accfull);
-          gg++;
-        }
-        lc++;
-        cg++;
-      }
-      if (*(volatile int *)abort_flag) break;
-    }
+    const MmaRing ring{full, empty, accfull, accempty, st_flags, abort_flag, g.wait_ns, nst};
+    if (!*(volatile int *)abort_flag && !mma_loop_s(S, ring, tmem, smem_u32(smem), issued)) atomicExch(abort_flag, 1);
     if (issued) {
       // every MMA this thread issued has completed before tensor memory is freed
       mma_commit(mmadone);
@@ -715,9 +752,9 @@ __global__ void __launch_bounds__(NTHR, 1) k_gemm_sliced(GemmArgs g) {
     }
   } else if (warp >= 4) {
     // ------------------------------------------------------------ drain, fold, epilogue
-    constexpr int HN = TN / 2;           // columns per drain warp
+    constexpr int HN = 4 * TN / DRAIN_WARPS;  // columns per drain warp
     const int q = warp & 3;              // TMEM lane quadrant (a warp reaches lanes 32 (warp % 4) ..)
-    const int h = (warp - 4) >> 2;       // column half
+    const int h = (warp - 4) >> 2;       // its columns [h HN, h HN + HN)
     const int row = q * 32 + lane;       // output row inside the tile
     uint32_t gg = 0;
     bool ok = true;
@@ -736,33 +773,25 @@ __global__ void __launch_bounds__(NTHR, 1) k_gemm_sliced(GemmArgs g) {
       for (int n = 0; n < HN; n++) acc[n] = 0;
       for (int grp = 0; grp < ngroups; grp++, gg++) {
         // warp-uniform outcome: the tensor-memory loads and the scatter below are warp-collective
-        if (!__all_sync(0xffffffffu, mbar_wait(accfull, gg & 1, g.wait_ns))) {
+        if (!__all_sync(0xffffffffu, mbar_wait(accfull, gg & 1, g.wait_ns, abort_flag))) {
           atomicExch(abort_flag, 1);
           ok = false;
           break;
         }
         tc_fence_after();
-        static_assert(HN == 40, "drain loads: 16 + 16 + 8 columns");
+        static_assert(HN == 20, "drain loads: 20 columns");
+        const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * HN);
         for (int a = 0; a < nacc; a++) {
-          // all loads of the accumulator in flight before one wait
-          const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * TN + h * HN);
-          uint32_t r0[16], r1[16], r2[8];
-          tmem_ld16(ta, r0);
-          tmem_ld16(ta + 16, r1);
-          tmem_ld8(ta + 32, r2);
-          tmem_wait_ld();
-          if (a < nexact) {
-            drain_exact(acc, r0, a, fsh - 7 * a);
-            drain_exact(acc + 16, r1, a, fsh - 7 * a);
-            drain_exact(acc + 32, r2, a, fsh - 7 * a);
-          } else {
-            drain_any(acc, r0, fsh);
-            drain_any(acc + 16, r1, fsh);
-            drain_any(acc + 32, r2, fsh);
+          uint32_t r[20];
+          tmem_ld20(ta + a * TN, r);
+          tmem_wait(r);
+          if (a + 1 == nacc) {  // all in registers: tensor memory is free for the next group (or tile)
+            tc_fence_before();
+            mbar_arrive(accempty);
           }
+          if (a < nexact) drain_exact(acc, r, a, fsh - 7 * a);
+          else drain_any(acc, r, fsh);
         }
-        tc_fence_before();
-        mbar_arrive(accempty);  // tensor memory free for the next group (or tile)
       }
       if (!ok) break;
       const int gr = mt * TM + row;
@@ -871,12 +900,12 @@ __global__ void __launch_bounds__(NTHR, 1) k_gemm_sliced(GemmArgs g) {
   __syncthreads();
   if (*(volatile int *)abort_flag) {
     if (warp == 0 && lane == 0) {
-      // after an abort the MMAs may not have consumed every chunk: no bulk copy may
+      // after an abort the MMAs may not have consumed every stage: no bulk copy may
       // still be writing shared memory when the CTA exits, so wait (bounded) for the
-      // last chunk issued on every stage (earlier ones completed before their stage
-      // was reused)
-      const uint32_t cg = issued_chunks;
-      const uint32_t first = cg > (uint32_t)nst ? cg - (uint32_t)nst : 0u;
+      // last copies issued on every stage (earlier ones completed before their stage
+      // was reused, also by the stage without data)
+      const uint32_t cg = issued_chunks, ring = (uint32_t)nst - end_posted;
+      const uint32_t first = cg > ring ? cg - ring : 0u;
       for (uint32_t c2 = first; c2 < cg; c2++) mbar_wait(&full[c2 % nst], (c2 / nst) & 1);
       *(volatile int *)g.err = 1;  // may be mapped host memory
     }
@@ -1091,10 +1120,8 @@ __global__ void k_slice_dig(int64_t n0, int64_t n, Acc acc, __nv_bfloat16 *plane
   const typename Acc::Row R = acc.row(w);
   const int m = e[(acc.is_b ? R.pr.eboff : R.pr.eaoff) + R.r];
   const int trows = acc.is_b ? TN : TM, tbytes = acc.is_b ? B_TILE : A_TILE;
-  const int rows_pad = acc.is_b ? R.pr.Npad : R.pr.Mpad;
   const int nkt = R.pr.Kpad / KC;
   char *base = (char *)planes + (acc.is_b ? R.pr.boff : R.pr.aoff);
-  const int64_t plane = (int64_t)(rows_pad / trows) * nkt * tbytes;
   const int rt = R.r / trows, rr = R.r % trows;
   for (int k0 = (lane >> 3) * 8; k0 < R.pr.Kpad; k0 += 32) {
     if (!dig_live(acc, R, k0)) continue;  // a stage the GEMM skips: its tile is never read
@@ -1104,10 +1131,10 @@ __global__ void k_slice_dig(int64_t n0, int64_t n, Acc acc, __nv_bfloat16 *plane
     uint32_t pk[4][S];
 #pragma unroll
     for (int j = 0; j < 4; j++) digit_pairs<S>(v[2 * j], v[2 * j + 1], m, pk[j]);
-    const int64_t off = ((int64_t)rt * nkt + k0 / KC) * tbytes + tile_off(rr, k0 % KC);
+    const int64_t off = ((int64_t)rt * nkt + k0 / KC) * S * tbytes + tile_off(rr, k0 % KC);
 #pragma unroll
     for (int t = 0; t < S; t++)
-      *reinterpret_cast<uint4 *>(base + t * plane + off) = make_uint4(pk[0][t], pk[1][t], pk[2][t], pk[3][t]);
+      *reinterpret_cast<uint4 *>(base + t * tbytes + off) = make_uint4(pk[0][t], pk[1][t], pk[2][t], pk[3][t]);
   }
 }
 
