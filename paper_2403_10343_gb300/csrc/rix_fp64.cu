@@ -101,20 +101,32 @@ __global__ void k_pairs(int nat, const double *xyz, const double *cell, int peri
 }
 
 // ------------------------------------------------------------------ screening flags
-// keep[b] = max |block b| >= tau (always 1 when tau <= 0); one warp per block.
-// norm (optional): the block's max |x| rounded up to a float (product screening).
-__global__ void k_flags(const double *arr, const int64_t *off, int64_t n, double tau, uint8_t *keep, float *norm) {
-  int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  int lane = threadIdx.x & 31;
+// keep[b] = max |block b| >= tau (always 1 when tau <= 0); one CTA of W warps per block.
+// norm (optional): the block's max |x| rounded up to a float (product screening).  C and V blocks
+// (up to 176 KB) take eight warps, D blocks (at most 1.5 KB in the water systems) one.
+template <int W>
+__global__ void __launch_bounds__(256)
+    k_flags(const double *arr, const int64_t *off, int64_t n, double tau, uint8_t *keep, float *norm) {
+  // W == 1: eight blocks to a CTA
+  const int64_t w = W == 1 ? (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5 : blockIdx.x;
+  const int t = W == 1 ? threadIdx.x & 31 : threadIdx.x;
   if (w >= n) return;
   if (!(tau > 0) && !norm) {
-    if (lane == 0) keep[w] = 1;
+    if (t == 0) keep[w] = 1;
     return;
   }
   double m = 0;
-  for (int64_t i = off[w] + lane; i < off[w + 1]; i += 32) m = fmax(m, fabs(arr[i]));
+#pragma unroll 4
+  for (int64_t i = off[w] + t; i < off[w + 1]; i += 32 * W) m = fmax(m, fabs(arr[i]));
   for (int s = 16; s; s >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, s));
-  if (lane == 0) {
+  if (W > 1) {
+    __shared__ double red[W];
+    if ((t & 31) == 0) red[t >> 5] = m;
+    __syncthreads();
+    if (t == 0)
+      for (int i = 1; i < W; i++) m = fmax(m, red[i]);
+  }
+  if (t == 0) {
     keep[w] = !(tau > 0) || m >= tau;
     if (norm) norm[w] = __double2float_ru(m);
   }
@@ -122,33 +134,35 @@ __global__ void k_flags(const double *arr, const int64_t *off, int64_t n, double
 
 // ------------------------------------------------------------------ symmetry check of C and V
 // C(B,A,-n)[P'][j][i] == C(A,B,n)[P][i][j] with P' the same aux function, and
-// V(B,A,-n) == V(A,B,n)^T, bit for bit.  One warp per pair; sets *flag on a mismatch.
-__global__ void k_symcheck(int64_t np, const int32_t *pA, const int32_t *pB, const int32_t *partner,
-                           const uint8_t *onsite, const int32_t *nb, const int32_t *na, const double *C,
-                           const int64_t *offC, const double *V, const int64_t *offV, int32_t *flag) {
-  int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  int lane = threadIdx.x & 31;
-  if (p >= np) return;
-  int a = pA[p], b = pB[p];
-  int64_t q = partner[p];
-  int nbA = nb[a], nbB = nb[b], naA = na[a], naB = na[b];
+// V(B,A,-n) == V(A,B,n)^T, bit for bit.  One CTA per pair, which compares both of the two partners
+// (each comparison is its own mirror); sets *flag on a mismatch.  ((H2O)27: 325 us with a warp
+// per pair, both partners comparing; 78 us now.)
+__global__ void __launch_bounds__(256)
+    k_symcheck(const int32_t *pA, const int32_t *pB, const int32_t *partner, const uint8_t *onsite, const int32_t *nb,
+               const int32_t *na, const double *C, const int64_t *offC, const double *V, const int64_t *offV,
+               int32_t *flag) {
+  const int64_t p = blockIdx.x;
+  const int64_t q = partner[p];
+  if (q < p) return;
+  const int a = pA[p], b = pB[p];
+  const int nbA = nb[a], nbB = nb[b], naA = na[a], naB = na[b];
+  const bool ons = onsite[p];
   bool bad = false;
   const double *c = C + offC[p], *cq = C + offC[q];
-  int rows = naA + (onsite[p] ? 0 : naB);
-  int64_t n = (int64_t)rows * nbA * nbB;
-  for (int64_t e = lane; e < n; e += 32) {
-    int P = (int)(e / (nbA * nbB));
-    int r = (int)(e % (nbA * nbB));
-    int i = r / nbB, j = r % nbB;
-    int Pq = onsite[p] ? P : (P < naA ? P + naB : P - naA);
-    if (c[e] != cq[((int64_t)Pq * nbB + j) * nbA + i]) bad = true;
+  const int n = (naA + (ons ? 0 : naB)) * nbA * nbB;
+#pragma unroll 4
+  for (int e = threadIdx.x; e < n; e += 256) {
+    const int P = e / (nbA * nbB), r = e - P * (nbA * nbB);
+    const int i = r / nbB, j = r - i * nbB;
+    const int Pq = ons ? P : (P < naA ? P + naB : P - naA);
+    bad |= c[e] != cq[(Pq * nbB + j) * nbA + i];
   }
   const double *v = V + offV[p], *vq = V + offV[q];
-  for (int e = lane; e < naA * naB; e += 32) {
-    int P = e / naB, Q = e % naB;
-    if (v[e] != vq[Q * naA + P]) bad = true;
+  for (int e = threadIdx.x; e < naA * naB; e += 256) {
+    const int P = e / naB, Q = e - P * naB;
+    bad |= v[e] != vq[Q * naA + P];
   }
-  if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(flag, 1);
+  if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(flag, 1);
 }
 
 // ------------------------------------------------------------------ live blocks
@@ -771,8 +785,9 @@ rix_status rix_launch_pairs(rix_ctx *ctx, const double *d_xyz, const double *d_c
 rix_status rix_launch_flags(rix_ctx *ctx, const double *arr, const int64_t *off, int64_t n, uint8_t *keep,
                             cudaStream_t st, float *norm) {
   if (n == 0) return RIX_OK;
-  const int64_t blocks = (n * 32 + 255) / 256;
-  k_flags<<<(unsigned)blocks, 256, 0, st>>>(arr, off, n, ctx->tau, keep, ctx->opt.product_tau > 0 ? norm : nullptr);
+  float *nm = ctx->opt.product_tau > 0 ? norm : nullptr;
+  if (off == ctx->d_offD) k_flags<1><<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>(arr, off, n, ctx->tau, keep, nm);
+  else k_flags<8><<<(unsigned)n, 256, 0, st>>>(arr, off, n, ctx->tau, keep, nm);
   return last(ctx, "k_flags");
 }
 
@@ -792,10 +807,8 @@ rix_status rix_launch_atom_max(rix_ctx *ctx, const float *norm, float *out, cuda
 
 rix_status rix_launch_symcheck(rix_ctx *ctx, cudaStream_t st) {
   RIX_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_flag, 0, sizeof(int32_t), st));
-  const int64_t blocks = (ctx->np * 32 + 255) / 256;
-  k_symcheck<<<(unsigned)blocks, 256, 0, st>>>(ctx->np, ctx->d_pA, ctx->d_pB, ctx->d_partner1, ctx->d_onsite,
-                                               ctx->d_nb, ctx->d_na, ctx->d_C, ctx->d_offC, ctx->d_V,
-                                               ctx->d_offV, ctx->d_flag);
+  k_symcheck<<<(unsigned)ctx->np, 256, 0, st>>>(ctx->d_pA, ctx->d_pB, ctx->d_partner1, ctx->d_onsite, ctx->d_nb,
+                                                ctx->d_na, ctx->d_C, ctx->d_offC, ctx->d_V, ctx->d_offV, ctx->d_flag);
   return last(ctx, "k_symcheck");
 }
 
