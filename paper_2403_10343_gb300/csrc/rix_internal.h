@@ -90,6 +90,13 @@ struct BX12Entry {
 
 // Output elements of a row-tiled work item: 32 or 4 per thread of a 256-thread CTA.
 constexpr int CAP_MAX = 8192, CAP_MIN = 1024;
+// Shared-memory tile of the adjoint kernels (doubles: three CTAs per SM), and the rows of a
+// kb_C12 item with it (U1 of every row for up to 64 functions i, nbG k each).
+constexpr int BWD_TILE = 9216;
+__host__ __device__ inline int bwd_c12_rows(int per, int nbG) {
+  const int a = CAP_MAX / per, b = BWD_TILE / (64 * nbG), r = a < b ? a : b;
+  return r > 1 ? r : 1;
+}
 
 // Device allocation tracked for the workspace statistics.
 struct DevBuf {

@@ -113,11 +113,26 @@ static void csr_group(int64_t nkeys, const std::vector<int64_t> &key, const std:
   for (size_t e = 0; e < key.size(); e++) out[pos[key[e]]++] = pay[e];
 }
 
-// Work items (output, first row) over `rows` rows of `per` elements each, rows per item
-// chosen by the same rule as the kernels.
-static void add_items(std::vector<int4> &it, int64_t out, int64_t rows, int64_t rt) {
-  for (int64_t r0 = 0; r0 < rows; r0 += rt) it.push_back(make_int4((int)out, (int)r0, 0, 0));
-}
+// Work items (output, first row) over `rows` rows, rt per item (the kernels' rule), with a cost per
+// row; sort_items puts the long ones first (longest processing time first).
+struct BwdItems {
+  std::vector<int4> it;
+  std::vector<double> cost;
+  void add(int64_t out, int64_t rows, int64_t rt, double row_cost) {
+    for (int64_t r0 = 0; r0 < rows; r0 += rt) {
+      it.push_back(make_int4((int)out, (int)r0, 0, 0));
+      cost.push_back((double)std::min(rt, rows - r0) * row_cost);
+    }
+  }
+  void sort() {
+    std::vector<int64_t> idx(it.size());
+    std::iota(idx.begin(), idx.end(), 0);
+    std::stable_sort(idx.begin(), idx.end(), [&](int64_t x, int64_t y) { return cost[x] > cost[y]; });
+    std::vector<int4> o(it.size());
+    for (size_t i = 0; i < idx.size(); i++) o[i] = it[idx[i]];
+    it.swap(o);
+  }
+};
 
 // Product lists of the adjoint (reverse order of the stages of rix_build_K).  Only
 // output blocks (A,E') on the pair list carry a nonzero adjoint, so every list is
@@ -125,8 +140,9 @@ static void add_items(std::vector<int4> &it, int64_t out, int64_t rows, int64_t 
 static rix_status build_backward_lists(rix_ctx *ctx, const std::vector<int2> &LT, const std::vector<int64_t> &ptrT,
                                        const std::vector<X12Entry> &LX12, const std::vector<int64_t> &ptrX12,
                                        const std::vector<int2> &LZ, const std::vector<int64_t> &ptrZ,
-                                       const std::vector<int32_t> &map2to1, const std::vector<int32_t> &atomA2,
-                                       const std::vector<int32_t> &atomB2, const std::vector<uint8_t> &z_half) {
+                                       const std::vector<int32_t> &map1to2, const std::vector<int32_t> &map2to1,
+                                       const std::vector<int32_t> &atomA2, const std::vector<int32_t> &atomB2,
+                                       const std::vector<uint8_t> &z_half) {
   const int nat = ctx->nat;
   const int64_t np = ctx->np, n2 = ctx->n2;
   auto &pA = ctx->pA, &pB = ctx->pB;
@@ -136,7 +152,7 @@ static rix_status build_backward_lists(rix_ctx *ctx, const std::vector<int2> &LT
   auto NB = [&](int a) { return (int64_t)ctx->nb_at[a]; };
   auto NA = [&](int a) { return (int64_t)ctx->na_at[a]; };
   auto find2 = [&](int64_t key) { int a = key_a(key); return find_in(keys2, row2[a], row2[a + 1], key); };
-  const int64_t CAP = 8192, SMB = 12288;
+  const int64_t CAP = CAP_MAX;
   double fl = 0;
 
   // (pair (A,B') not on-site, pair (A,E')) -> Z(B, E'-n1)
@@ -262,26 +278,33 @@ static rix_status build_backward_lists(rix_ctx *ctx, const std::vector<int2> &LT
   std::vector<int64_t>().swap(kTC); std::vector<int2>().swap(vTC);
 
   // ------------------------------------------------------------ tiled work items
-  std::vector<int4> it[9];
+  // cost of an item: list entries x rows x multiply-adds per row and entry (of an average partner)
+  BwdItems it[9];
+  auto len = [](const std::vector<int64_t> &ptr, int64_t i) { return (double)(ptr[i + 1] - ptr[i]); };
   for (int64_t p = 0; p < np; p++) {
-    int a = pA[p], x = pB[p];
-    if (ptrBC[p + 1] > ptrBC[p]) add_items(it[0], p, NA(x), std::max<int64_t>(1, CAP / (NB(a) * NB(x))));
-    if (ptrZV[p + 1] > ptrZV[p]) add_items(it[2], p, NA(a), std::max<int64_t>(1, CAP / NA(x)));
-    if (ptrZC[p + 1] > ptrZC[p]) add_items(it[3], p, NA(a), std::max<int64_t>(1, CAP / (NB(a) * NB(x))));
-    if (ptrU2[p + 1] > ptrU2[p]) add_items(it[4], p, NA(x), std::max<int64_t>(1, CAP / (NB(a) * NB(x))));
-    if (hasT1[p] || ptrU2[p + 1] > ptrU2[p]) add_items(it[6], p, NA(a), std::max<int64_t>(1, CAP / NA(x)));
-    if (ptrC12[p + 1] > ptrC12[p]) {
-      int64_t rows = NA(a) + (ctx->onsite[p] ? 0 : NA(x));
-      int64_t per = NB(a) * NB(x);
-      add_items(it[7], p, rows, std::max<int64_t>(1, std::min(CAP / per, SMB / (64 * NB(a)))));
+    const int a = pA[p], x = pB[p];
+    const int64_t per = NB(a) * NB(x), rt = std::max<int64_t>(1, CAP / per);
+    const double dper = (double)per;
+    if (len(ptrBC, p) > 0) it[0].add(p, NA(x), rt, len(ptrBC, p) * dper);
+    if (len(ptrZV, p) > 0) it[2].add(p, NA(a), std::max<int64_t>(1, CAP / NA(x)), len(ptrZV, p) * NA(x) * NB(x));
+    if (len(ptrZC, p) > 0) it[3].add(p, NA(a), rt, len(ptrZC, p) * dper);
+    if (len(ptrU2, p) > 0) it[4].add(p, NA(x), rt, len(ptrU2, p) * dper);
+    if (hasT1[p] || len(ptrU2, p) > 0)
+      it[6].add(p, NA(a), std::max<int64_t>(1, CAP / NA(x)),
+                (hasT1[p] ? len(ptrX12, map1to2[p]) : 1.0) * NA(x) * NB(a));
+    if (len(ptrC12, p) > 0) {
+      const int64_t rows = NA(a) + (ctx->onsite[p] ? 0 : NA(x));
+      it[7].add(p, rows, bwd_c12_rows((int)per, (int)NB(a)), len(ptrC12, p) * dper);
     }
-    if (ptrTC[p + 1] > ptrTC[p]) add_items(it[8], p, NA(a), std::max<int64_t>(1, CAP / (NB(a) * NB(x))));
+    if (len(ptrTC, p) > 0) it[8].add(p, NA(a), rt, len(ptrTC, p) * dper);
   }
   for (int64_t z = 0; z < n2; z++) {
-    int b = atomA2[z], e = atomB2[z];
-    if (ptrBZ[z + 1] > ptrBZ[z]) add_items(it[1], z, NA(b), std::max<int64_t>(1, CAP / (NB(b) * NB(e))));
-    if (needT[z]) add_items(it[5], z, NA(b), std::max<int64_t>(1, CAP / (NB(b) * NB(e))));
+    const int b = atomA2[z], e = atomB2[z];
+    const int64_t per = NB(b) * NB(e), rt = std::max<int64_t>(1, CAP / per);
+    if (len(ptrBZ, z) > 0) it[1].add(z, NA(b), rt, len(ptrBZ, z) * (double)per);
+    if (needT[z]) it[5].add(z, NA(b), rt, (1.0 + len(ptrT1, z)) * (double)per);
   }
+  for (BwdItems &k : it) k.sort();
   ctx->bwd_flops = fl;
 
   TRY(rix_upload(ctx, &ctx->d_wB, wB)); TRY(rix_upload(ctx, &ctx->d_c34, c34));
@@ -294,8 +317,8 @@ static rix_status build_backward_lists(rix_ctx *ctx, const std::vector<int2> &LT
   TRY(rix_upload(ctx, &ctx->d_ptrBC12, ptrC12)); TRY(rix_upload(ctx, &ctx->d_LBC12, LC12));
   TRY(rix_upload(ctx, &ctx->d_ptrBTC, ptrTC)); TRY(rix_upload(ctx, &ctx->d_LBTC, LTC));
   for (int k = 0; k < 9; k++) {
-    TRY(rix_upload(ctx, &ctx->d_itB[k], it[k]));
-    ctx->n_itB[k] = it[k].size();
+    TRY(rix_upload(ctx, &ctx->d_itB[k], it[k].it));
+    ctx->n_itB[k] = it[k].it.size();
   }
   int64_t nU = 0;
   for (int64_t p = 0; p < np; p++) nU += NA(pB[p]) * NB(pA[p]) * NB(pB[p]);
@@ -699,8 +722,8 @@ static rix_status build_lists(rix_ctx *ctx) {
 
   // ---------------------------------------------------------------- backward plan
   if (ctx->opt.backward) {
-    rix_status sb = build_backward_lists(ctx, LT, ptrT, LX12, ptrX12, LZ, ptrZ, map2to1, atomA2, atomB2,
-                                         z_half);
+    rix_status sb = build_backward_lists(ctx, LT, ptrT, LX12, ptrX12, LZ, ptrZ, map1to2, map2to1, atomA2,
+                                         atomB2, z_half);
     if (sb != RIX_OK) return sb;
   }
 
