@@ -45,7 +45,9 @@ namespace rixtc {
 constexpr int TM = 128;         // output rows per tile (one TMEM lane each)
 constexpr int TN = 80;          // output columns per tile
 constexpr int KC = 16;          // K per pipeline stage (one MMA K step)
-// Accumulation groups of GROUP K stages (576 K values, the most that stays exact).  Accumulator a < NACC-1
+// Accumulation groups of GROUP K stages (576 K values, the most that stays exact whatever the
+// digits are; a tile whose digits are known to be small enough is one group, see
+// TileInfo::group).  Accumulator a < NACC-1
 // holds diagonal a: pairs (0, a) and (a, 0) with a leading digit (<= 128)
 // and a balanced one (<= 64), and a - 1 pairs of balanced digits (a = 0: the
 // one pair of leading digits), so its sum stays an integer below 2^24.
@@ -574,6 +576,8 @@ struct GemmArgs {
   const int64_t *kmask_off = nullptr;
   unsigned long long *chunks = nullptr;  // profiling: 128 x 80 x 16 MMAs issued (K stages x K steps x slice pairs)
   unsigned long long *X128 = nullptr;  // deterministic mode: X additions as 128-bit fixed point (2 words each)
+  // batched mode: the largest digit sum of squares of every row and column tile (wsq)
+  const float *tA = nullptr, *tB = nullptr;
   uint64_t wait_ns = WAIT_NS;  // limit of every bounded wait
   int stall = 0;           // 1: the MMA issuer waits on a barrier nothing completes (timeout test)
 };
@@ -605,6 +609,13 @@ struct TileInfo {
   bool live;  // false: the tile's A rows are all zero (screened), every role skips it
   const unsigned long long *km;  // live K stages (nullptr: all)
   int nlive;                      // number of live K stages
+  // Stages per accumulation group.  A diagonal's partial sums are at most sum |a_s||b_u| <= sqrt(W_row
+  // W_col) (Cauchy-Schwarz over all slices and K values), so where the digits' sums of squares
+  // keep that below 2^24 every sum of the whole tile stays exact in FP32 and it is one group, up to six
+  // slices (each accumulator one diagonal).  Digits of dense data average 37, so that is K up to about
+  // 2,000; a fold stops the MMAs for ~8.9k clocks, ten stages' worth.  ((H2O)64 build: GEMM launches
+  // 63.4 -> 59.4 ms.)
+  int group;
 };
 
 __device__ __forceinline__ TileInfo tile_info(const GemmArgs &g, int t) {
@@ -621,6 +632,10 @@ __device__ __forceinline__ TileInfo tile_info(const GemmArgs &g, int t) {
     ti.geB = g.eB + pr->eboff;
     ti.Mpad = pr->Mpad; ti.Npad = pr->Npad; ti.Kpad = pr->Kpad; ti.M = pr->M; ti.N = pr->N; ti.drop = pr->drop;
     ti.live = !g.row_live || g.row_live[tt.w];
+    ti.group = GROUP;
+    if (g.tA && g.S <= NACC &&
+        g.tA[pr->eaoff / TM + tt.y] * g.tB[pr->eboff / TN + tt.z] < 281474976710656.f)  // 2^48
+      ti.group = 1 << 30;
     ti.km = nullptr;
     ti.nlive = ti.Kpad / KC;
     if (g.kmask) {
@@ -638,6 +653,7 @@ __device__ __forceinline__ TileInfo tile_info(const GemmArgs &g, int t) {
     ti.gA = g.A; ti.gB = g.B; ti.geA = g.eA; ti.geB = g.eB;
     ti.Mpad = g.Mpad; ti.Npad = g.Npad; ti.Kpad = g.Kpad; ti.M = g.M; ti.N = g.N; ti.drop = g.drop;
     ti.live = true;
+    ti.group = GROUP;
     ti.km = nullptr;
     ti.nlive = ti.Kpad / KC;
   }
@@ -721,8 +737,8 @@ __global__ void __launch_bounds__(NTHR, 1) k_gemm_sliced(GemmArgs g) {
             break;
           }
           lc++;
-          st_flags[st] = (gl == 0 ? ST_OPEN : 0u) | (gl == GROUP - 1 || lc == ti.nlive ? ST_LAST : 0u);
-          if (++gl == GROUP) gl = 0;
+          st_flags[st] = (gl == 0 ? ST_OPEN : 0u) | (gl == ti.group - 1 || lc == ti.nlive ? ST_LAST : 0u);
+          if (++gl == ti.group) gl = 0;
           uint8_t *sa = smem + st * stage_bytes;
           mbar_expect_tx(&full[st], (uint32_t)stage_bytes);
           bulk_g2s(sa, ga + (int64_t)c * (S * A_TILE), (uint32_t)(S * A_TILE), &full[st]);
@@ -766,7 +782,7 @@ __global__ void __launch_bounds__(NTHR, 1) k_gemm_sliced(GemmArgs g) {
     for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
       const TileInfo ti = tile_info(g, t);
       if (!ti.live) continue;  // its output is zero: nothing to drain or add
-      const int ngroups = (ti.nlive + GROUP - 1) / GROUP;  // accumulation groups of live K stages
+      const int ngroups = (ti.nlive - 1) / ti.group + 1;  // accumulation groups of live K stages
       const int mt = ti.mt, nt = ti.nt, drop = ti.drop, Ncols = ti.N;
       const Prob *pr = ti.pr;
       const int *geA = ti.geA, *geB = ti.geB;
@@ -1060,24 +1076,26 @@ struct Src {
 // K values, so each warp writes whole core-matrix rows (16 B per slice, 256 B
 // contiguous per warp and slice).  The accessor gives element k of packed row w.
 // Digit t of two values as a packed BF16 pair (low half: x0), with integer
-// and FMA-pipe operations only (the conversion unit is the scarce one): the
-// plain digit u of digit_sum is made the FP32 number 1.5 2^23 + u by its bits, and one FMA
-// takes off the 1.5 2^23 (and the 64 of the bias) and scales by 2^-7t (exact: the
+// and FP32 operations only (the conversion unit is the scarce one): the
+// plain digit u of digit_sum is made the FP32 number 1.5 2^23 + u by its bits, 1.5 2^23 (and
+// the 64 of the bias) is taken off and the digit scaled by 2^-7t (both exact: the
 // digit has at most 8 significant bits, 128 being a power of two), so its top 16 bits
 // are its BF16 encoding; the signs of the values are applied to the pair at the end.
+// sq += the squares of the digits.
 template <int S>
-__device__ __forceinline__ void digit_pairs(double x0, double x1, int e, uint32_t (&w)[S]) {
+__device__ __forceinline__ void digit_pairs(double x0, double x1, int e, uint32_t (&w)[S], float &sq) {
   const uint64_t b0 = (uint64_t)__double_as_longlong(x0), b1 = (uint64_t)__double_as_longlong(x1);
   const uint64_t f0 = digit_sum<S>(frac_of(b0, e)), f1 = digit_sum<S>(frac_of(b1, e));
   const uint32_t sg = ((uint32_t)(b0 >> 63) << 15) | ((uint32_t)(b1 >> 32) & 0x80000000u);
 #pragma unroll
   for (int t = 0; t < S; t++) {
     const float sc = __int_as_float((127 - 7 * t) << 23);  // 2^-7t
-    const float off = -(12582912.f + (t ? 64.f : 0.f)) * sc;
+    const float off = 12582912.f + (t ? 64.f : 0.f);
     const uint32_t mask = t ? 127u : 255u;
-    const float d0 = __fmaf_rn(__uint_as_float(0x4B400000u | ((uint32_t)(f0 >> (56 - 7 * t)) & mask)), sc, off);
-    const float d1 = __fmaf_rn(__uint_as_float(0x4B400000u | ((uint32_t)(f1 >> (56 - 7 * t)) & mask)), sc, off);
-    w[t] = __byte_perm(__float_as_uint(d0), __float_as_uint(d1), 0x7632) ^ sg;
+    const float d0 = __uint_as_float(0x4B400000u | ((uint32_t)(f0 >> (56 - 7 * t)) & mask)) - off;
+    const float d1 = __uint_as_float(0x4B400000u | ((uint32_t)(f1 >> (56 - 7 * t)) & mask)) - off;
+    sq = fmaf(d0, d0, fmaf(d1, d1, sq));
+    w[t] = __byte_perm(__float_as_uint(d0 * sc), __float_as_uint(d1 * sc), 0x7632) ^ sg;
   }
 }
 
@@ -1095,16 +1113,18 @@ __device__ __forceinline__ bool dig_live(const Acc &, const typename Acc::Row &,
   return true;
 }
 
-template <class Acc>
-__global__ void k_slice_exp(int64_t n0, int64_t n, Acc acc, int *e) {
-  const int64_t w = n0 + ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (w >= n0 + n) return;
-  const typename Acc::Row R = acc.row(w);
+// W warps per row (eight warps to a CTA): four where the plan has few rows.
+template <class Acc, int W>
+__global__ void __launch_bounds__(256) k_slice_exp(int64_t n0, int64_t n, Acc acc, int *e, float *wsq) {
+  __shared__ int red[8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t w = n0 + blockIdx.x * (int64_t)(8 / W) + warp / W;
+  const bool in = w < n0 + n;
+  const typename Acc::Row R = acc.row(in ? w : n0);
   int m = -2000;
   // eight elements per lane in flight (their gathers are independent; lanes along K, which eight
   // consecutive values per lane would spread over eight times the sectors)
-  for (int k = lane; k < R.pr.Kpad; k += 256) {
+  for (int k = 256 * (warp % W) + lane; k < R.pr.Kpad; k += 256 * W) {
     double v[8];
 #pragma unroll
     for (int j = 0; j < 8; j++) v[j] = k + 32 * j < R.pr.Kpad ? acc.at(R, k + 32 * j) : 0.0;
@@ -1112,13 +1132,25 @@ __global__ void k_slice_exp(int64_t n0, int64_t n, Acc acc, int *e) {
     for (int j = 0; j < 8; j++) m = max(m, exp_of(fabs(v[j])));
   }
   for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0) e[(acc.is_b ? R.pr.eboff : R.pr.eaoff) + R.r] = m;
+  if (W > 1) {
+    if (lane == 0) red[warp] = m;
+    __syncthreads();
+    if (warp % W == 0)
+      for (int i = 1; i < W; i++) m = max(m, red[warp + i]);
+  }
+  if (in && warp % W == 0 && lane == 0) {
+    e[(acc.is_b ? R.pr.eboff : R.pr.eaoff) + R.r] = m;
+    wsq[(acc.is_b ? R.pr.eboff : R.pr.eaoff) + R.r] = 0.f;
+  }
 }
 
 // K values [kper blockIdx.y, + kper) of the rows (kper a multiple of 32): a plan with few rows
-// spreads its K over the grid's y.
+// spreads its K over the grid's y.  wsq: the sum of the squares of a row's digits, all slices (an
+// upper bound: 2^-6 covers the FP32 rounding of up to 2^18 additions per thread, K = 131,072), which
+// decides how long the GEMM may accumulate; the exponent pass has set it to 0.
 template <class Acc, int S>
-__global__ void k_slice_dig(int64_t n0, int64_t n, Acc acc, __nv_bfloat16 *planes, const int *e, int kper) {
+__global__ void __launch_bounds__(256, 4)
+    k_slice_dig(int64_t n0, int64_t n, Acc acc, __nv_bfloat16 *planes, const int *e, float *wsq, int kper) {
   const int64_t g8 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (g8 * 8 >= n) return;  // n is a multiple of 8 (problems pad to whole tiles)
@@ -1130,6 +1162,7 @@ __global__ void k_slice_dig(int64_t n0, int64_t n, Acc acc, __nv_bfloat16 *plane
   const int nkt = R.pr.Kpad / KC;
   char *base = (char *)planes + (acc.is_b ? R.pr.boff : R.pr.aoff);
   const int rt = R.r / trows, rr = R.r % trows;
+  float W = 0.f;
   for (int k0 = blockIdx.y * kper + (lane >> 3) * 8; k0 < kend; k0 += 32) {
     if (!dig_live(acc, R, k0)) continue;  // a stage the GEMM skips: its tile is never read
     // the eight loads first (independent, so their latencies overlap), then the digits
@@ -1137,18 +1170,42 @@ __global__ void k_slice_dig(int64_t n0, int64_t n, Acc acc, __nv_bfloat16 *plane
     load8(acc, R, k0, v);
     uint32_t pk[4][S];
 #pragma unroll
-    for (int j = 0; j < 4; j++) digit_pairs<S>(v[2 * j], v[2 * j + 1], m, pk[j]);
+    for (int j = 0; j < 4; j++) digit_pairs<S>(v[2 * j], v[2 * j + 1], m, pk[j], W);
     const int64_t off = ((int64_t)rt * nkt + k0 / KC) * S * tbytes + tile_off(rr, k0 % KC);
 #pragma unroll
     for (int t = 0; t < S; t++)
       *reinterpret_cast<uint4 *>(base + t * tbytes + off) = make_uint4(pk[0][t], pk[1][t], pk[2][t], pk[3][t]);
   }
+  W += __shfl_xor_sync(0xffffffffu, W, 8);
+  W += __shfl_xor_sync(0xffffffffu, W, 16);
+  if (lane < 8) {
+    float *d = wsq + (acc.is_b ? R.pr.eboff : R.pr.eaoff) + R.r;
+    W *= 1.f + 1.f / 64.f;
+    if (gridDim.y > 1) atomicAdd(d, W);
+    else *d = W;
+  }
+}
+
+// Largest wsq of every row tile in [a0, a1) and column tile in [b0, b1), one warp per tile.
+__global__ void k_tile_wsq(int64_t a0, int64_t a1, int64_t b0, int64_t b1, const float *wA, const float *wB, float *tA,
+                           float *tB) {
+  const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  const bool is_b = w >= a1 - a0;
+  const int64_t tile = is_b ? b0 + (w - (a1 - a0)) : a0 + w;
+  if (is_b && tile >= b1) return;
+  const int n = is_b ? TN : TM;
+  const float *src = (is_b ? wB : wA) + tile * n;
+  float m = 0.f;
+  for (int i = lane; i < n; i += 32) m = fmaxf(m, src[i]);
+  for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) (is_b ? tB : tA)[tile] = m;
 }
 
 // exponents and digit planes of rows [n0, n0 + n) (n a multiple of 8): the exponent pass,
 // then the digit pass
 template <class Acc>
-void slice_rows(int64_t n0, int64_t n, const Acc &acc, int S, __nv_bfloat16 *planes, int *e, int kmax,
+void slice_rows(int64_t n0, int64_t n, const Acc &acc, int S, __nv_bfloat16 *planes, int *e, float *wsq, int kmax,
                 cudaStream_t st);
 
 // k_slice_dig over rows [n0, n0 + n) (n a multiple of 8, K at most kmax) for S slices.  A warp
@@ -1156,30 +1213,31 @@ void slice_rows(int64_t n0, int64_t n, const Acc &acc, int S, __nv_bfloat16 *pla
 // are split, down to 32 per warp ((H2O)8: the digits of terms 2 and 3+4 were 130 us per launch on
 // 130 warps, 13 us now).
 template <class Acc>
-void launch_slice_dig(int64_t n0, int64_t n, const Acc &acc, int S, __nv_bfloat16 *planes, const int *e, int kmax,
-                      cudaStream_t st) {
+void launch_slice_dig(int64_t n0, int64_t n, const Acc &acc, int S, __nv_bfloat16 *planes, const int *e, float *wsq,
+                      int kmax, cudaStream_t st) {
   const int64_t warps = n / 8, k32 = (kmax + 31) / 32;
   const int64_t ny = std::min<int64_t>(k32, (152 * 32 + warps - 1) / warps);
   const int kper = (int)((k32 + ny - 1) / ny) * 32;
   const dim3 grid((unsigned)((warps * 32 + 255) / 256), (unsigned)((kmax + kper - 1) / kper));
   switch (S) {
-    case 1: k_slice_dig<Acc, 1><<<grid, 256, 0, st>>>(n0, n, acc, planes, e, kper); break;
-    case 2: k_slice_dig<Acc, 2><<<grid, 256, 0, st>>>(n0, n, acc, planes, e, kper); break;
-    case 3: k_slice_dig<Acc, 3><<<grid, 256, 0, st>>>(n0, n, acc, planes, e, kper); break;
-    case 4: k_slice_dig<Acc, 4><<<grid, 256, 0, st>>>(n0, n, acc, planes, e, kper); break;
-    case 5: k_slice_dig<Acc, 5><<<grid, 256, 0, st>>>(n0, n, acc, planes, e, kper); break;
-    case 6: k_slice_dig<Acc, 6><<<grid, 256, 0, st>>>(n0, n, acc, planes, e, kper); break;
-    case 7: k_slice_dig<Acc, 7><<<grid, 256, 0, st>>>(n0, n, acc, planes, e, kper); break;
-    default: k_slice_dig<Acc, 8><<<grid, 256, 0, st>>>(n0, n, acc, planes, e, kper); break;
+    case 1: k_slice_dig<Acc, 1><<<grid, 256, 0, st>>>(n0, n, acc, planes, e, wsq, kper); break;
+    case 2: k_slice_dig<Acc, 2><<<grid, 256, 0, st>>>(n0, n, acc, planes, e, wsq, kper); break;
+    case 3: k_slice_dig<Acc, 3><<<grid, 256, 0, st>>>(n0, n, acc, planes, e, wsq, kper); break;
+    case 4: k_slice_dig<Acc, 4><<<grid, 256, 0, st>>>(n0, n, acc, planes, e, wsq, kper); break;
+    case 5: k_slice_dig<Acc, 5><<<grid, 256, 0, st>>>(n0, n, acc, planes, e, wsq, kper); break;
+    case 6: k_slice_dig<Acc, 6><<<grid, 256, 0, st>>>(n0, n, acc, planes, e, wsq, kper); break;
+    case 7: k_slice_dig<Acc, 7><<<grid, 256, 0, st>>>(n0, n, acc, planes, e, wsq, kper); break;
+    default: k_slice_dig<Acc, 8><<<grid, 256, 0, st>>>(n0, n, acc, planes, e, wsq, kper); break;
   }
 }
 
 template <class Acc>
-void slice_rows(int64_t n0, int64_t n, const Acc &acc, int S, __nv_bfloat16 *planes, int *e, int kmax,
+void slice_rows(int64_t n0, int64_t n, const Acc &acc, int S, __nv_bfloat16 *planes, int *e, float *wsq, int kmax,
                 cudaStream_t st) {
   if (n <= 0) return;
-  k_slice_exp<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>(n0, n, acc, e);
-  launch_slice_dig(n0, n, acc, S, planes, e, kmax, st);
+  if (n < 152 * 32) k_slice_exp<Acc, 4><<<(unsigned)((n + 1) / 2), 256, 0, st>>>(n0, n, acc, e, wsq);
+  else k_slice_exp<Acc, 1><<<(unsigned)((n + 7) / 8), 256, 0, st>>>(n0, n, acc, e, wsq);
+  launch_slice_dig(n0, n, acc, S, planes, e, wsq, kmax, st);
 }
 
 // element access of the plans of terms 2, 3+4 and Z: packed row (or column) w
@@ -1263,7 +1321,7 @@ __device__ __forceinline__ void load8(const SrcAcc &acc, SrcAcc::Row &R, int k0,
 // the product of the two maximising entries: the same FP64 product, hence the same
 // exponent, as the element-wise pass, from na + nb loads per member instead of
 // na nb products.
-__global__ void k_kron_exp(int64_t n0, int64_t n, SrcAcc acc, int *e) {
+__global__ void k_kron_exp(int64_t n0, int64_t n, SrcAcc acc, int *e, float *wsq) {
   const int64_t w = n0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (w >= n0 + n) return;
   const SrcAcc::Row R = acc.row(w);
@@ -1281,6 +1339,7 @@ __global__ void k_kron_exp(int64_t n0, int64_t n, SrcAcc acc, int *e) {
     m = max(m, exp_of(sr.flag & XHALF ? 0.5 * (mv * md) : mv * md));
   }
   e[R.pr.eaoff + R.r] = m;
+  wsq[R.pr.eaoff + R.r] = 0.f;
 }
 
 // Per row tile r of a grouped plan, for this build: bit c of its K-stage mask is set
@@ -1333,6 +1392,29 @@ __global__ void k_flag_set(int n, const int32_t *idx, uint8_t *flags) {
 #include <map>
 #include <vector>
 
+// Sums of the squares of the digits of every packed row and column, and the largest per tile.
+struct rix_digit_sums {
+  float *a = nullptr, *b = nullptr, *ta = nullptr, *tb = nullptr;
+  rix_status alloc(rix_ctx *ctx, int64_t rows, int64_t cols) {
+    rix_status s;
+    if ((s = rix_alloc(ctx, &a, std::max<int64_t>(rows, 1))) != RIX_OK) return s;
+    if ((s = rix_alloc(ctx, &b, std::max<int64_t>(cols, 1))) != RIX_OK) return s;
+    if ((s = rix_alloc(ctx, &ta, std::max<int64_t>(rows / rixtc::TM, 1))) != RIX_OK) return s;
+    return rix_alloc(ctx, &tb, std::max<int64_t>(cols / rixtc::TN, 1));
+  }
+  // device bytes of `rows` packed rows and `cols` columns (whole tiles)
+  static int64_t bytes(int64_t rows, int64_t cols) { return 4 * (rows + cols + rows / rixtc::TM + cols / rixtc::TN); }
+  // the tiles of packed rows [r0, r1) and columns [c0, c1), into the GEMM's arguments
+  void tiles(int64_t r0, int64_t r1, int64_t c0, int64_t c1, int kmax, cudaStream_t st, rixtc::GemmArgs &ga) const {
+    const int64_t a0 = r0 / rixtc::TM, a1 = r1 / rixtc::TM, b0 = c0 / rixtc::TN, b1 = c1 / rixtc::TN;
+    const int64_t n = (a1 - a0) + (b1 - b0);
+    if (n <= 0 || kmax <= rixtc::GROUP * rixtc::KC) return;  // no tile is longer than a group
+    rixtc::k_tile_wsq<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>(a0, a1, b0, b1, a, b, ta, tb);
+    ga.tA = ta;
+    ga.tB = tb;
+  }
+};
+
 // Host and device state of one batched plan.
 struct rix_mx_plan {
   int kind = 0;                          // 0: terms 3+4, 1: term 2, 2: term-4 intermediate Z
@@ -1351,6 +1433,7 @@ struct rix_mx_plan {
   rixtc::Src *d_rowsrc = nullptr, *d_colsrc = nullptr;
   int32_t *d_xmap = nullptr;
   int *d_eA = nullptr, *d_eB = nullptr;
+  rix_digit_sums wsq;
   // row tiles: per build, the K stages that meet a kept block of their rows (a member
   // of the problem whose blocks with these rows are all screened or absent is skipped)
   int64_t n_rt = 0;
@@ -1652,7 +1735,8 @@ rix_status plan_host(rix_ctx *ctx, int kind, const std::vector<int64_t> &ptrZ, P
       // xmap, rowinfo + rowprob + rowsrc + exponent, colinfo + colprob + colsrc + exponent, tiles
       maps += (int64_t)rt_here.size() * (8 + 8 + 1 + 8 * nkw) + (int64_t)rtq_here.size() * 8 +
               (int64_t)rm.size() * cm.size() * 4 + (int64_t)Mpad * (8 + 8 + 32 * G + 4) +
-              (int64_t)Npad * (16 + 8 + 32 * G + 4) + (int64_t)(Mpad / TM) * (Npad / TN) * 16 + (int64_t)sizeof(Prob);
+              (int64_t)Npad * (16 + 8 + 32 * G + 4) + (int64_t)(Mpad / TM) * (Npad / TN) * 16 + (int64_t)sizeof(Prob) +
+              rix_digit_sums::bytes(Mpad, Npad);
       h.tflops += 2.0 * Mpad * Npad * Kpad * npairs;
       if (count_only) continue;
       const int pidx = (int)h.probs.size();
@@ -1891,6 +1975,7 @@ rix_status rix_mixed_plan(rix_ctx *ctx, const std::vector<int64_t> &ptrZ) {
     if ((s = rix_upload(ctx, &pl->d_xmap, h.xmap)) != RIX_OK) return s;
     if ((s = rix_alloc(ctx, &pl->d_eA, std::max<int64_t>(h.eaoff, 1))) != RIX_OK) return s;
     if ((s = rix_alloc(ctx, &pl->d_eB, std::max<int64_t>(h.eboff, 1))) != RIX_OK) return s;
+    if ((s = pl->wsq.alloc(ctx, h.eaoff, h.eboff)) != RIX_OK) return s;
     if (!h.rt.empty()) {
       pl->n_rt = (int64_t)h.rt.size();
       if ((s = rix_upload(ctx, &pl->d_rt, h.rt)) != RIX_OK) return s;
@@ -1945,14 +2030,14 @@ rix_status rix_mixed_plan(rix_ctx *ctx, const std::vector<int64_t> &ptrZ) {
 }
 
 // Kernel launches of one rix_build_K: flags, per block T, U2 and Z, terms 1+2 and
-// terms 3+4 (FP64 per block) or per group four slicing kernels and a GEMM
+// terms 3+4 (FP64 per block) or per group five slicing kernels and a GEMM
 // (mixed), symmetrise.
 int32_t rix_launch_count(const rix_ctx *ctx) {
   int32_t n = 2 + 3 * ctx->nblk + (ctx->use_live ? 2 : 0);
   if (ctx->have_mx) {
-    // per group: exponents and digits of both operands, then the GEMM
-    n += 5 * (int32_t)(ctx->mx34->grp.size() - 1) + 5 * (int32_t)(ctx->mx2->grp.size() - 1) +
-         5 * (int32_t)(ctx->mxz->grp.size() - 1) + rix_t1_launches(ctx) + rix_tt_launches(ctx);
+    // per group: exponents and digits of both operands, the tiles' digit sums, the GEMM
+    n += 6 * (int32_t)(ctx->mx34->grp.size() - 1) + 6 * (int32_t)(ctx->mx2->grp.size() - 1) +
+         6 * (int32_t)(ctx->mxz->grp.size() - 1) + rix_t1_launches(ctx) + rix_tt_launches(ctx);
     if (ctx->n_t1tc < ctx->nat) n += rix_x12_launches(ctx);  // k_X12 for the other column atoms
     if (ctx->n_ztc == ctx->nat) n -= ctx->nblk;   // no k_Z: the Z buffer is zeroed by a memset
     // row-tile K-stage masks: once per Z block, once per terms-3+4 block, once for term 2
@@ -1998,15 +2083,15 @@ rix_status run_group(rix_ctx *ctx, const rix_mx_plan *pl, size_t g, const Operan
   if (r1 > r0) {
     const SrcAcc a{pl->d_rowprob, pl->d_probs, pl->d_rowsrc, pl->G, ra.x, ra.shift, ra.x2, ra.keep, ra.keep2, 0};
     if (pl->kind == 2) {  // Kronecker rows: exponents from the factors' maxima
-      k_kron_exp<<<(unsigned)((r1 - r0 + 127) / 128), 128, 0, st>>>(r0, r1 - r0, a, pl->d_eA);
-      launch_slice_dig(r0, r1 - r0, a, S, buf, pl->d_eA, pl->kmax, st);
+      k_kron_exp<<<(unsigned)((r1 - r0 + 127) / 128), 128, 0, st>>>(r0, r1 - r0, a, pl->d_eA, pl->wsq.a);
+      launch_slice_dig(r0, r1 - r0, a, S, buf, pl->d_eA, pl->wsq.a, pl->kmax, st);
     } else {
-      slice_rows(r0, r1 - r0, a, S, buf, pl->d_eA, pl->kmax, st);
+      slice_rows(r0, r1 - r0, a, S, buf, pl->d_eA, pl->wsq.a, pl->kmax, st);
     }
   }
   if (c1 > c0) {
     const SrcAcc b{pl->d_colprob, pl->d_probs, pl->d_colsrc, pl->G, cb.x, cb.shift, cb.x2, cb.keep, cb.keep2, 1};
-    slice_rows(c0, c1 - c0, b, S, buf, pl->d_eB, pl->kmax, st);
+    slice_rows(c0, c1 - c0, b, S, buf, pl->d_eB, pl->wsq.b, pl->kmax, st);
   }
   if (t1 > t0) {
     GemmArgs ga{buf, buf, pl->d_eA, pl->d_eB, nullptr, 0, 0, 0, 0, 0, 0, S, 1, 0, ctx->d_mx_err,
@@ -2019,6 +2104,7 @@ rix_status run_group(rix_ctx *ctx, const rix_mx_plan *pl, size_t g, const Operan
     ga.kmask = pl->d_kmask;
     ga.kmask_off = pl->d_rtkw;
     if (out == ctx->d_X && ctx->d_X128) ga.X128 = ctx->d_X128;  // deterministic: X as 128-bit fixed point
+    pl->wsq.tiles(r0, r1, c0, c1, pl->kmax, st, ga);
     rix_status ls = launch_gemm(ctx, ga, t1 - t0, S, st);
     if (ls != RIX_OK) return ls;
   }
@@ -2267,7 +2353,7 @@ __global__ void k_rowexp(int64_t t0, const int64_t *off2, const int64_t *roff2, 
 // row: the rows of a warp are neighbours in every block, so its loads are contiguous (a warp per
 // row, lanes over g, took 4.0 ms per build of the 192-atom ice cell, 1.1 ms now).
 __global__ void k_t1_exp(int64_t n0, int64_t n, T1RowAcc acc, const int64_t *segR, const int *rexp,
-                         int64_t rbase, int *e) {
+                         int64_t rbase, int *e, float *wsq) {
   const int64_t w = n0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (w >= n0 + n) return;
   const T1RowAcc::Row R = acc.row(w);
@@ -2283,6 +2369,7 @@ __global__ void k_t1_exp(int64_t n0, int64_t n, T1RowAcc acc, const int64_t *seg
     }
   }
   e[R.pr.eaoff + R.r] = m;
+  wsq[R.pr.eaoff + R.r] = 0.f;
 }
 
 }  // namespace rixtc
@@ -2305,6 +2392,7 @@ struct rix_t1_plan {
   int32_t *d_gpair = nullptr;
   QInfo *d_qinfo = nullptr;
   int *d_eA = nullptr, *d_eB = nullptr;
+  rix_digit_sums wsq;
 };
 
 // Term-1 plan: decide per column atom, build problems (E, block) for the tensor ones.
@@ -2389,7 +2477,8 @@ rix_status rix_t1_plan_build(rix_ctx *ctx, bool count_only, int64_t *bytes_out) 
       maxp = std::max(maxp, bytes);
       maps += (int64_t)Mpad * (8 + 8 + 4) + (int64_t)Npad * (16 + 8 + 4) + (int64_t)Kpad * 16 +
               (int64_t)qs.size() * ng * 16 + (int64_t)ng * 12 + (int64_t)qs.size() * 24 +
-              (int64_t)(Mpad / TM) * (Npad / TN) * 16 + (int64_t)(sizeof(Prob) + sizeof(T1Ext));
+              (int64_t)(Mpad / TM) * (Npad / TN) * 16 + (int64_t)(sizeof(Prob) + sizeof(T1Ext)) +
+              rix_digit_sums::bytes(Mpad, Npad);
       tflops += 2.0 * Mpad * Npad * Kpad * npairs;
       if (count_only) continue;
       const int pidx = (int)probs.size();
@@ -2522,6 +2611,7 @@ rix_status rix_t1_plan_build(rix_ctx *ctx, bool count_only, int64_t *bytes_out) 
   if ((s = rix_upload(ctx, &pl->d_qinfo, qinfo)) != RIX_OK) return s;
   if ((s = rix_alloc(ctx, &pl->d_eA, std::max<int64_t>(eaoff, 1))) != RIX_OK) return s;
   if ((s = rix_alloc(ctx, &pl->d_eB, std::max<int64_t>(eboff, 1))) != RIX_OK) return s;
+  if ((s = pl->wsq.alloc(ctx, eaoff, eboff)) != RIX_OK) return s;
   // column atoms whose term 1 runs here: k_X12 skips them
   std::vector<int32_t> on;
   for (int e = 0; e < nat; e++)
@@ -2577,13 +2667,13 @@ rix_status rix_mixed_t1(rix_ctx *ctx, int b, int64_t tbase, cudaStream_t st) {
       const T1RowAcc a{pl->d_rowprob, pl->d_probs, pl->d_ext, pl->d_rowinfo, pl->d_qinfo, pl->d_kmap, pl->d_segT,
                        ctx->d_T, tbase};
       k_t1_exp<<<(unsigned)((r1 - r0 + 127) / 128), 128, 0, st>>>(r0, r1 - r0, a, pl->d_segR, rexp, rbase,
-                                                                          pl->d_eA);
-      launch_slice_dig(r0, r1 - r0, a, S, buf, pl->d_eA, pl->kmax, st);
+                                                                  pl->d_eA, pl->wsq.a);
+      launch_slice_dig(r0, r1 - r0, a, S, buf, pl->d_eA, pl->wsq.a, pl->kmax, st);
     }
     if (c1 > c0) {
       const T1ColAcc b{pl->d_colprob, pl->d_probs, pl->d_ext, pl->d_colinfo, pl->d_kmap, pl->d_segC, pl->d_gpair,
                        ctx->d_keepC, ctx->d_C};
-      slice_rows(c0, c1 - c0, b, S, buf, pl->d_eB, pl->kmax, st);
+      slice_rows(c0, c1 - c0, b, S, buf, pl->d_eB, pl->wsq.b, pl->kmax, st);
     }
     if (t1 > t0) {
       GemmArgs ga{buf, buf, pl->d_eA, pl->d_eB, nullptr, 0, 0, 0, 0, 0, 0, S, 1, 0, ctx->d_mx_err,
@@ -2591,6 +2681,7 @@ rix_status rix_mixed_t1(rix_ctx *ctx, int b, int64_t tbase, cudaStream_t st) {
                   1, pl->d_qinfo, ctx->d_V, ctx->d_keepV, 1.0};
       ga.ntiles = (int)(t1 - t0);
       ga.X128 = ctx->d_X128;  // deterministic builds: 128-bit fixed-point additions
+      pl->wsq.tiles(r0, r1, c0, c1, pl->kmax, st, ga);
       rix_status ls = launch_gemm(ctx, ga, t1 - t0, S, st);
       if (ls != RIX_OK) return ls;
     }
@@ -2609,7 +2700,7 @@ int32_t rix_t1_launches(const rix_ctx *ctx) {
   int32_t n = 0, last_blk = -1;
   for (size_t g = 0; g + 1 < pl->grp_prob.size(); g++) {
     if (pl->grp_prob[g + 1] == pl->grp_prob[g]) continue;
-    n += 5;  // row exponents and digits, column exponents and digits, the GEMM
+    n += 6;  // row exponents and digits, column exponents and digits, digit sums, the GEMM
     if (pl->grp_blk[g] != last_blk) n++;  // k_rowexp, once per block (groups are in block order)
     last_blk = pl->grp_blk[g];
   }
@@ -2780,7 +2871,7 @@ __global__ void k_dcolexp(int64_t np, const int32_t *pA, const int32_t *pB, cons
 // D(B', G'_t) of the column's T block (its product list) of their column-k maxima,
 // which is the largest exponent over the column's K values (the rest are zero).
 __global__ void k_tt_colexp(int64_t n0, int64_t n, TTColAcc acc, const int64_t *dcoff, const int *dcolexp,
-                            int *e) {
+                            int *e, float *wsq) {
   const int64_t w = n0 + ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (w >= n0 + n) return;
@@ -2793,7 +2884,10 @@ __global__ void k_tt_colexp(int64_t n0, int64_t n, TTColAcc acc, const int64_t *
     }
   }
   for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0) e[R.pr.eboff + R.r] = m;
+  if (lane == 0) {
+    e[R.pr.eboff + R.r] = m;
+    wsq[R.pr.eboff + R.r] = 0.f;
+  }
 }
 
 // K-stage masks of the T plan: for every product (C(A,B'), D(B',G')) of a T block with kept
@@ -2840,6 +2934,7 @@ struct rix_tt_plan {
   int64_t *d_rowprob = nullptr, *d_colprob = nullptr;
   int32_t *d_xmap = nullptr;
   int *d_eA = nullptr, *d_eB = nullptr;
+  rix_digit_sums wsq;
   // K-stage masks: per (problem, column tile) the stages whose D tile is not all zero,
   // set per build from the D screening flags (most (B', G') are not D pairs or are screened)
   int64_t n_mask = 0;
@@ -2915,6 +3010,7 @@ rix_status rix_tt_plan_build(rix_ctx *ctx, bool count_only, int64_t *bytes_out) 
     const int mwords = (Kpad / KC + 63) / 64;
     maps += (int64_t)Mpad * (8 + 8 + 4) + (int64_t)Npad * (16 + 8 + 4) + (int64_t)Kpad * 16 + (int64_t)nz * 4 +
             (int64_t)(Mpad / TM) * (Npad / TN) * 16 + (int64_t)(sizeof(Prob) + sizeof(TTExt)) +
+            rix_digit_sums::bytes(Mpad, Npad) +
             (int64_t)(Npad / TN) * mwords * 8 + (int64_t)(row1[a + 1] - row1[a]) * 4 + (int64_t)nz * 12;
     tflops += 2.0 * Mpad * Npad * Kpad * npairs;
     if (count_only) continue;
@@ -3037,6 +3133,7 @@ rix_status rix_tt_plan_build(rix_ctx *ctx, bool count_only, int64_t *bytes_out) 
   }
   if ((s = rix_alloc(ctx, &pl->d_eA, std::max<int64_t>(eaoff, 1))) != RIX_OK) return s;
   if ((s = rix_alloc(ctx, &pl->d_eB, std::max<int64_t>(eboff, 1))) != RIX_OK) return s;
+  if ((s = pl->wsq.alloc(ctx, eaoff, eboff)) != RIX_OK) return s;
   {
     std::vector<int64_t> dcoff(ctx->np + 1, 0);
     for (int64_t p = 0; p < ctx->np; p++) dcoff[p + 1] = dcoff[p] + ctx->nb_at[ctx->pB[p]];
@@ -3095,14 +3192,14 @@ rix_status rix_mixed_T(rix_ctx *ctx, int b, int64_t tbase, const double *D, cuda
     if (r1 > r0) {
       const TTRowAcc a{pl->d_rowprob, pl->d_probs, pl->d_ext, pl->d_rowinfo, pl->d_kmap, ctx->d_offC, ctx->d_keepC,
                        ctx->d_C};
-      slice_rows(r0, r1 - r0, a, S, buf, pl->d_eA, pl->kmax, st);
+      slice_rows(r0, r1 - r0, a, S, buf, pl->d_eA, pl->wsq.a, pl->kmax, st);
     }
     if (c1 > c0) {
       const TTColAcc bb{pl->d_colprob, pl->d_probs, pl->d_ext, pl->d_colinfo, pl->d_kmap, ctx->d_ptrT, ctx->d_LT,
                         ctx->d_offD, ctx->d_keepD, D, pl->n_mask > 0 ? pl->d_mask : nullptr};
       k_tt_colexp<<<(unsigned)(((c1 - c0) * 32 + 255) / 256), 256, 0, st>>>(c0, c1 - c0, bb, pl->d_dcoff,
-                                                                             pl->d_dcolexp, pl->d_eB);
-      launch_slice_dig(c0, c1 - c0, bb, S, buf, pl->d_eB, pl->kmax, st);
+                                                                             pl->d_dcolexp, pl->d_eB, pl->wsq.b);
+      launch_slice_dig(c0, c1 - c0, bb, S, buf, pl->d_eB, pl->wsq.b, pl->kmax, st);
     }
     if (t1 > t0) {
       GemmArgs ga{buf, buf, pl->d_eA, pl->d_eB, nullptr, 0, 0, 0, 0, 0, 0, S, 1, 0, ctx->d_mx_err,
@@ -3112,6 +3209,7 @@ rix_status rix_mixed_T(rix_ctx *ctx, int b, int64_t tbase, const double *D, cuda
       ga.xshift = tbase;
       ga.ntiles = (int)(t1 - t0);
       ga.kmask = pl->d_mask;  // skip the K stages whose D tile is all zero
+      pl->wsq.tiles(r0, r1, c0, c1, pl->kmax, st, ga);
       rix_status ls = launch_gemm(ctx, ga, t1 - t0, S, st);
       if (ls != RIX_OK) return ls;
     }
@@ -3127,7 +3225,7 @@ rix_status rix_mixed_T(rix_ctx *ctx, int b, int64_t tbase, const double *D, cuda
 int32_t rix_tt_launches(const rix_ctx *ctx) {
   if (!ctx->mxt) return 0;
   const int32_t ng = (int32_t)(ctx->mxt->grp_prob.size() - 1);
-  return 5 * ng + (ctx->mxt->n_mask > 0 ? 1 : 0) + (ng > 0 ? 1 : 0);  // + k_tt_mask, k_dcolexp
+  return 6 * ng + (ctx->mxt->n_mask > 0 ? 1 : 0) + (ng > 0 ? 1 : 0);  // + k_tt_mask, k_dcolexp
 }
 
 extern "C" rix_status rix_gemm_profile(rix_ctx *ctx, double *ms, int64_t *launches, int64_t *chunks) {
