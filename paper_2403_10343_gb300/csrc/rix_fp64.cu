@@ -414,7 +414,6 @@ __device__ __forceinline__ void gather_shares(double (&acc)[R], const Split &s, 
 // few Q over all of them in shared memory (full warps whatever the species), then the split product.
 // Term 2 is a split product per entry.
 constexpr int XCOL = 192;    // columns of a batch at most
-constexpr int XENT = 32;     // entries of a batch at most (one warp builds the table)
 struct XCols {
   int64_t t[XCOL], c[XCOL];  // offsets of T(A,G')[0][0][k] and C(G',E')[Q = 0 on E'][k][0]
   int nb[XCOL];              // nb of G'

@@ -531,7 +531,8 @@ struct Prob {
   int32_t kb[GMAX + 1];    // their K ranges; kb[ng] = K
 };
 
-// Output row block of a term-1 problem: the K block X(A',E'), the pair (A',E')
+// Output row block of a term-1 problem and one of its column atoms: the K block X(A',E')
+// (x < 0: none, the pair is absent or left to its transpose partner), the pair (A',E')
 // carrying V(A',E') (offset voff), nb of A', and whether the block takes term 1
 // with weight 1/2 (the on-site pair; every other pair takes it with weight 1 in
 // one orientation).
@@ -558,10 +559,10 @@ struct GemmArgs {
   const int32_t *xmap;     // output block index per (q, z)
   const int64_t *offK;
   double *X;               // X[offK[x] + i * nbE + l] += value (atomic)
-  // mode 1 (term 1): rows (q, P nbA + i), columns (l, Q, nbE, naE) l-major;
+  // mode 1 (term 1): rows (q, P nbA + i), columns (l + member 2^16, Q, nbE, naE) l-major;
   // X(A',E')[i][l] += oscale w sum_Q V(A',E')[P][Q] R[row][col], one atomic per l (w: QInfo)
   int mode;
-  const QInfo *qinfo;      // per row block, indexed from Prob::xoff
+  const QInfo *qinfo;      // per row block and member ([nq][ng]), indexed from Prob::xoff
   const double *V;
   const uint8_t *keepV;
   double oscale;           // scale of the added values (modes 0 and 1)
@@ -887,31 +888,39 @@ __global__ void __launch_bounds__(NTHR, 1) k_gemm_sliced(GemmArgs g) {
         } else if (g.mode == 1) {
           const int2 ri = g.rowinfo[pr->rowoff + gr];
           if (ri.x >= 0) {
-            const QInfo qi = g.qinfo[pr->xoff + ri.x];
-            if (g.keepV[qi.vpair]) {
-              const double osc = qi.half ? 0.5 * g.oscale : g.oscale;
-              const int P = ri.y / qi.nbA, i = ri.y - P * qi.nbA;
-              int lcur = -1, nbE = 0;
-              double part = 0.0;
+            const QInfo *qb = g.qinfo + pr->xoff + (int64_t)ri.x * pr->ng;
+            const int nbA = qb->nbA;
+            const int P = ri.y / nbA, i = ri.y - P * nbA;
+            int cur = -1, mem = -1, nbE = 0, xb = -1;  // column (member, l), member, its nb, output block
+            int64_t vb = 0;
+            double osc = 0.0, part = 0.0;
 #pragma unroll
-              for (int n = 0; n < HN; n++) {
-                const int gc = nt * TN + h * HN + n;
-                if (gc < Ncols) {
-                  const int4 ci = g.colinfo[pr->coloff + gc];  // (l, Q, nbE, naE)
-                  if (ci.x >= 0) {
-                    if (ci.x != lcur) {
-                      if (lcur >= 0) x_add(g, qi.x, (int64_t)i * nbE + lcur, osc * part);
-                      lcur = ci.x;
+            for (int n = 0; n < HN; n++) {
+              const int gc = nt * TN + h * HN + n;
+              if (gc < Ncols) {
+                const int4 ci = g.colinfo[pr->coloff + gc];  // (l + member 2^16, Q, nbE, naE)
+                if (ci.x >= 0) {
+                  if (ci.x != cur) {
+                    if (xb >= 0) x_add(g, xb, (int64_t)i * nbE + (cur & 0xFFFF), osc * part);
+                    cur = ci.x;
+                    part = 0.0;
+                    if (ci.x >> 16 != mem) {
+                      mem = ci.x >> 16;
                       nbE = ci.z;
-                      part = 0.0;
+                      const QInfo qi = qb[mem];
+                      xb = qi.x >= 0 && g.keepV[qi.vpair] ? qi.x : -1;
+                      vb = qi.voff + (int64_t)P * ci.w;
+                      osc = qi.half ? 0.5 * g.oscale : g.oscale;
                     }
+                  }
+                  if (xb >= 0) {
                     const int sc = er + geB[gc] - 7 * (S + 1) + drop;
-                    part = fma(g.V[qi.voff + (int64_t)P * ci.w + ci.y], fixed_to_double(acc[n], sc), part);
+                    part = fma(g.V[vb + ci.y], fixed_to_double(acc[n], sc), part);
                   }
                 }
               }
-              if (lcur >= 0) x_add(g, qi.x, (int64_t)i * nbE + lcur, osc * part);
             }
+            if (xb >= 0) x_add(g, xb, (int64_t)i * nbE + (cur & 0xFFFF), osc * part);
           }
         }
       }
@@ -1530,6 +1539,58 @@ constexpr double FP64_RATE_T1 = 0.7e12, FP64_RATE_Z = 1.2e12, FP64_RATE_T = 1.0e
 // Middle atoms within this distance of a group's first atom join its problem (2.5 A).
 constexpr double GROUP_R = 2.5 / 0.529177210903;
 
+// An atom of a group and its image relative to the group's first atom.
+struct MolMember {
+  int b;
+  int o[3];
+};
+
+// Atoms that share most of their neighbours, grouped: atoms consecutive in index order (of those
+// in use) within GROUP_R of the first, GMAX at most, in one memory-plan block (blk, if given): the
+// atoms of a molecule.  Member k sits at image o_k from the first (its shortest pair).
+std::vector<std::vector<MolMember>> molecule_groups(const rix_ctx *ctx, const std::vector<uint8_t> &use,
+                                                    const std::vector<int32_t> *blk) {
+  const int nat = ctx->nat;
+  std::vector<std::vector<MolMember>> groups;
+  for (int b = 0; b < nat;) {
+    if (!use[b]) {
+      b++;
+      continue;
+    }
+    std::vector<MolMember> gm(1, MolMember{b, {0, 0, 0}});
+    int c = b + 1;
+    for (; c < nat && (int)gm.size() < rixtc::GMAX && use[c] && !(blk && (*blk)[c] != (*blk)[b]); c++) {
+      double best = GROUP_R;
+      int64_t qb = -1;
+      for (int64_t q = ctx->row1[b]; q < ctx->row1[b + 1]; q++) {
+        if (ctx->pB[q] != c) continue;
+        double d2 = 0.0;
+        for (int x = 0; x < 3; x++) {
+          double sh = 0.0;
+          if (ctx->periodic)
+            for (int d = 0; d < 3; d++) sh += (double)ctx->pn[3 * q + d] * ctx->cell[3 * d + x];
+          const double r = (ctx->xyz[3 * c + x] + sh) - ctx->xyz[3 * b + x];
+          d2 += r * r;
+        }
+        if (std::sqrt(d2) < best) {
+          best = std::sqrt(d2);
+          qb = q;
+        }
+      }
+      if (qb < 0) break;
+      // the member's image relative to the first atom: a neighbour within GROUP_R, so at
+      // most one cell away unless a cell edge is shorter than GROUP_R
+      bool near = true;
+      for (int x = 0; x < 3; x++) near &= ctx->pn[3 * qb + x] >= -1 && ctx->pn[3 * qb + x] <= 1;
+      if (!near) break;
+      gm.push_back(MolMember{c, {ctx->pn[3 * qb], ctx->pn[3 * qb + 1], ctx->pn[3 * qb + 2]}});
+    }
+    groups.push_back(std::move(gm));
+    b = c;
+  }
+  return groups;
+}
+
 // Build the problems of one plan (see the section comment for the three kinds).
 // count_only: no host arrays, just the map bytes, the largest problem's slices
 // and the total slice bytes (the memory plan is not known yet: one block).
@@ -1580,56 +1641,14 @@ rix_status plan_host(rix_ctx *ctx, int kind, const std::vector<int64_t> &ptrZ, P
   if (have_blocks)
     for (int b = 0; b < ctx->nblk; b++)
       for (int a = ctx->blk_atom[b]; a < ctx->blk_atom[b + 1]; a++) mblk[a] = b;
-  // Problems: groups of middle atoms that share most of their neighbours (atoms
-  // consecutive in index order within GROUP_R of the first, in one memory-plan
-  // block: the atoms of a molecule).  A group's contraction ranges are
+  // Problems: groups of middle atoms that share most of their neighbours (molecule_groups).  A
+  // group's contraction ranges are
   // concatenated on the K axis, its rows and columns are the union of its
   // members', so the output of the group is added once instead of once per atom.
-  // Member k sits at image o_k from the first (its shortest pair); row (A', M)
-  // means A' at image M from the first member, i.e. at M - o_k from member k,
+  // Row (A', M) means A' at image M from the first member, i.e. at M - o_k from member k,
   // and the output block of (row (A', M), column (E', N)) is (A', E', N - M).
-  struct Member {
-    int b;
-    int o[3];
-  };
-  std::vector<std::vector<Member>> groups;
-  for (int b = 0; b < nat;) {
-    if (!h.use[b]) {
-      b++;
-      continue;
-    }
-    std::vector<Member> gm(1, Member{b, {0, 0, 0}});
-    int c = b + 1;
-    for (; c < nat && (int)gm.size() < GMAX && h.use[c] && mblk[c] == mblk[b]; c++) {
-      double best = GROUP_R;
-      int64_t qb = -1;
-      for (int64_t q = row1[b]; q < row1[b + 1]; q++) {
-        if (ctx->pB[q] != c) continue;
-        double d2 = 0.0;
-        for (int x = 0; x < 3; x++) {
-          double sh = 0.0;
-          if (ctx->periodic)
-            for (int d = 0; d < 3; d++) sh += (double)ctx->pn[3 * q + d] * ctx->cell[3 * d + x];
-          const double r = (ctx->xyz[3 * c + x] + sh) - ctx->xyz[3 * b + x];
-          d2 += r * r;
-        }
-        if (std::sqrt(d2) < best) {
-          best = std::sqrt(d2);
-          qb = q;
-        }
-      }
-      if (qb < 0) break;
-      // the member's image relative to the first atom: a neighbour within GROUP_R, so at
-      // most one cell away unless a cell edge is shorter than GROUP_R
-      bool near = true;
-      for (int x = 0; x < 3; x++) near &= ctx->pn[3 * qb + x] >= -1 && ctx->pn[3 * qb + x] <= 1;
-      if (!near) break;
-      gm.push_back(Member{c, {ctx->pn[3 * qb], ctx->pn[3 * qb + 1], ctx->pn[3 * qb + 2]}});
-    }
-    h.G = std::max(h.G, (int)gm.size());
-    groups.push_back(std::move(gm));
-    b = c;
-  }
+  const std::vector<std::vector<MolMember>> groups = molecule_groups(ctx, h.use, &mblk);
+  for (const auto &gm : groups) h.G = std::max(h.G, (int)gm.size());
   const int G = h.G;
   const Src absent{-1, -1, 1, 1, 1, -1};
   // (atom, image) as a sortable key; member images are within one cell, so a pair's image
@@ -2219,7 +2238,7 @@ rix_status rix_mixed_z(rix_ctx *ctx, int blk, int64_t zbase, const double *D, cu
 }
 
 // ==========================================================================
-// Term 1 on the tensor cores, one problem per column atom E (and memory-plan
+// Term 1 on the tensor cores, one problem per molecule {E} of column atoms (and memory-plan
 // block of row atoms):
 //
 //   R(A',E')[(P,i)][(l,Q)] = sum_{G' near E'} sum_k T(A',G')[P][i][k] C(G',E')[Q on E'][k][l]
@@ -2228,8 +2247,12 @@ rix_status rix_mixed_z(rix_ctx *ctx, int blk, int64_t zbase, const double *D, cu
 // with w = 1 for the pairs (A', E') in their representative orientation, w = 1/2
 // for the on-site pair and no row for the others (term 1 is symmetric under the
 // transposition of its pair, and K = X + X^T restores the other orientation).
-// Rows (A', P, i) over those row atoms A' near E', K = (G', k) over E's
-// neighbours G', columns (l, Q).  The V contraction (a few FLOPs per R
+// Rows (A', P, i) over those row atoms A' near a member E', K = (G', k) over the members'
+// neighbours G', columns (E', l, Q).  The members share most rows and K values, so the digits of
+// T, which only depend on those, are written once per molecule and not once per atom (two thirds of
+// them served a hydrogen's single column tile); rows and K values are ordered by the members
+// that they belong to, and the tiles and K stages of other members are left out.  ((H2O)64 build, GEMM and
+// T digits: 59.3 + 12.4 -> 60.1 + 4.8 ms; 192-atom ice: 152 + 34.8 -> 156 + 16.0 ms.)  The V contraction (a few FLOPs per R
 // element) runs in the GEMM epilogue in FP64.  This costs about nb_E times
 // the FLOPs of the FP64 grouping (which applies V per (A', G', E') triple),
 // so a column atom runs here only when its tensor time is estimated lower.
@@ -2240,7 +2263,7 @@ namespace rixtc {
 struct T1Ext {
   int64_t koff;    // kmap offset (Kpad entries: (g, k, nbG, -), g < 0 past K)
   int64_t segoff;  // segT offset ([nq][ng]: off2 of T(A'_q, G'_g), -1 if absent)
-  int64_t goff;    // segC / gpair offset ([ng])
+  int64_t goff;    // segC / gpair offset ([ng][members])
   int32_t nq, ng;
 };
 
@@ -2274,7 +2297,7 @@ struct T1RowAcc {
     R.P = R.i = 0;
     R.nbA = 1;
     if (ri.x >= 0) {
-      R.nbA = qinfo[R.pr.xoff + ri.x].nbA;
+      R.nbA = qinfo[R.pr.xoff + (int64_t)ri.x * R.pr.ng].nbA;
       R.P = ri.y / R.nbA;
       R.i = ri.y - R.P * R.nbA;
       R.seg = segT + ex.segoff + (int64_t)ri.x * ex.ng;
@@ -2291,7 +2314,7 @@ struct T1RowAcc {
   }
 };
 
-// columns: element (l, Q ; g, k) = C(G'_g, E')[Q on E'][k][l]
+// columns: element (E', l, Q ; g, k) = C(G'_g, E')[Q on E'][k][l]
 struct T1ColAcc {
   const int64_t *prob_of;
   const Prob *probs;
@@ -2323,8 +2346,11 @@ struct T1ColAcc {
   __device__ double at(const Row &R, int kk) const {
     if (R.ci.x < 0) return 0.0;
     const int4 km = kmap[R.koff + kk];
-    if (km.x < 0 || !keepC[gpair[R.goff + km.x]]) return 0.0;
-    return C[segC[R.goff + km.x] + ((int64_t)R.ci.y * km.z + km.y) * R.ci.z + R.ci.x];
+    if (km.x < 0) return 0.0;
+    const int64_t s = R.goff + (int64_t)km.x * R.pr.ng + (R.ci.x >> 16);
+    const int p = gpair[s];
+    if (p < 0 || !keepC[p]) return 0.0;
+    return C[segC[s] + ((int64_t)R.ci.y * km.z + km.y) * R.ci.z + (R.ci.x & 0xFFFF)];
   }
 };
 
@@ -2391,6 +2417,7 @@ struct rix_t1_plan {
   std::vector<int64_t> roff2;
   int32_t *d_gpair = nullptr;
   QInfo *d_qinfo = nullptr;
+  unsigned long long *d_kmask = nullptr;  // per (problem, column tile): the K stages of its members
   int *d_eA = nullptr, *d_eB = nullptr;
   rix_digit_sums wsq;
 };
@@ -2456,35 +2483,74 @@ rix_status rix_t1_plan_build(rix_ctx *ctx, bool count_only, int64_t *bytes_out) 
   std::vector<QInfo> qinfo;
   int64_t eaoff = 0, eboff = 0, maps = 0, maxp = 0, total = 0;
   double tflops = 0;
-  std::vector<int64_t> qs;
+  std::vector<unsigned long long> kmask;  // per (problem, column tile): the K stages of its members
+  const std::vector<std::vector<MolMember>> groups = molecule_groups(ctx, use, nullptr);
+  // a row or K node: (atom, image from the group's first member) and its pair with every member
+  struct Node {
+    int64_t key;
+    std::array<int64_t, GMAX> q;
+    int mask;
+  };
+  bool img_ok = true;
   for (int b = 0; b < nblk; b++)
-    for (int e = 0; e < nat; e++) {
-      if (!use[e]) continue;
-      qs.clear();
-      for (int64_t q = row1[e]; q < row1[e + 1]; q++)
-        if (blk_of[ctx->pB[q]] == b && ctx->rep1[ctx->partner1[q]]) qs.push_back(q);
+    for (const auto &gm : groups) {
+      const int nm = (int)gm.size();
+      // nodes (A', M) of the members' pairs (E_k, A', m), M = m + o_k; ordered by the members
+      // they belong to (all of them first), then by atom
+      auto nodes = [&](auto take) {
+        std::map<int64_t, Node> m;
+        for (int k = 0; k < nm; k++)
+          for (int64_t q = row1[gm[k].b]; q < row1[gm[k].b + 1]; q++) {
+            if (!take(q)) continue;
+            int M[3];
+            for (int c = 0; c < 3; c++) {
+              M[c] = ctx->pn[3 * q + c] + gm[k].o[c];
+              img_ok &= M[c] > -128 && M[c] < 128;
+            }
+            const int64_t key = pair_key(0, ctx->pB[q], M[0], M[1], M[2]);
+            auto it = m.find(key);
+            if (it == m.end()) {
+              Node nd{key, {}, 0};
+              nd.q.fill(-1);
+              it = m.emplace(key, nd).first;
+            }
+            it->second.q[k] = q;
+            it->second.mask |= 1 << k;
+          }
+        std::vector<Node> v;
+        for (const auto &x : m) v.push_back(x.second);
+        std::stable_sort(v.begin(), v.end(), [](const Node &x, const Node &y) { return x.mask > y.mask; });
+        return v;
+      };
+      const std::vector<Node> qs =
+          nodes([&](int64_t q) { return blk_of[ctx->pB[q]] == b && ctx->rep1[ctx->partner1[q]] != 0; });
       if (qs.empty()) continue;
-      const int nbE = ctx->nb_at[e], naE = ctx->na_at[e];
-      const int ng = (int)(row1[e + 1] - row1[e]);
-      int M = 0, K = 0;
-      for (auto q : qs) M += ctx->na_at[ctx->pB[q]] * ctx->nb_at[ctx->pB[q]];
-      for (int64_t g = row1[e]; g < row1[e + 1]; g++) K += ctx->nb_at[ctx->pB[g]];
-      const int N = naE * nbE;
+      const std::vector<Node> gs = nodes([](int64_t) { return true; });
+      if (!img_ok) {
+        ctx->last_error = "term-1 plan: an image index outside the pair key's range";
+        return RIX_EINVAL;
+      }
+      const int ng = (int)gs.size();
+      int M = 0, K = 0, N = 0;
+      for (const Node &q : qs) M += ctx->na_at[key_b(q.key)] * ctx->nb_at[key_b(q.key)];
+      for (const Node &g : gs) K += ctx->nb_at[key_b(g.key)];
+      for (const MolMember &e : gm) N += ctx->na_at[e.b] * ctx->nb_at[e.b];
       const int Mpad = std::max(TM, (M + TM - 1) / TM * TM), Npad = std::max(TN, (N + TN - 1) / TN * TN);
       const int Kpad = std::max(KC, (K + KC - 1) / KC * KC);
+      const int mwords = (Kpad / KC + 63) / 64;
       const int64_t bytes = (int64_t)S * (Mpad + Npad) * Kpad * 2;
       total += bytes;
       maxp = std::max(maxp, bytes);
       maps += (int64_t)Mpad * (8 + 8 + 4) + (int64_t)Npad * (16 + 8 + 4) + (int64_t)Kpad * 16 +
-              (int64_t)qs.size() * ng * 16 + (int64_t)ng * 12 + (int64_t)qs.size() * 24 +
-              (int64_t)(Mpad / TM) * (Npad / TN) * 16 + (int64_t)(sizeof(Prob) + sizeof(T1Ext)) +
-              rix_digit_sums::bytes(Mpad, Npad);
-      tflops += 2.0 * Mpad * Npad * Kpad * npairs;
+              (int64_t)qs.size() * ng * 16 + (int64_t)ng * nm * 12 + (int64_t)qs.size() * nm * 24 +
+              (int64_t)(Mpad / TM) * (Npad / TN) * 16 + (int64_t)(Npad / TN) * mwords * 8 +
+              (int64_t)(sizeof(Prob) + sizeof(T1Ext)) + rix_digit_sums::bytes(Mpad, Npad);
       if (count_only) continue;
       const int pidx = (int)probs.size();
       Prob pr{};
       pr.M = M; pr.N = N; pr.Mpad = Mpad; pr.Npad = Npad; pr.Kpad = Kpad; pr.pad_ = K;
       pr.nz = ng;
+      pr.ng = nm;
       pr.drop = fixed_point_drop(Kpad, S);
       pr.eaoff = eaoff; pr.eboff = eboff;
       pr.rowoff = (int64_t)rowinfo.size();
@@ -2493,57 +2559,94 @@ rix_status rix_t1_plan_build(rix_ctx *ctx, bool count_only, int64_t *bytes_out) 
       eaoff += Mpad;
       eboff += Npad;
       T1Ext ex{(int64_t)kmap.size(), (int64_t)segT.size(), (int64_t)segC.size(), (int32_t)qs.size(), ng};
-      // K map and the C segments (G' at image n from E'; C(G',E') is the partner of (E',G',n))
-      for (int64_t g = row1[e]; g < row1[e + 1]; g++) {
-        const int gg = ctx->pB[g];
-        const int64_t p3 = ctx->partner1[g];
-        const int nbG = ctx->nb_at[gg];
-        const int qE0 = ctx->onsite[p3] ? 0 : ctx->na_at[gg];
-        for (int k = 0; k < nbG; k++) kmap.push_back(make_int4((int)(g - row1[e]), k, nbG, 0));
-        segC.push_back(ctx->offC[p3] + (int64_t)qE0 * nbG * nbE);
-        gpair.push_back((int32_t)p3);
+      // K map, the members of every K stage, and the C segments (G' at image n from E'; C(G',E') is the
+      // partner of (E',G',n))
+      std::vector<int> stage_mem(Kpad / KC, 0);
+      for (int gi = 0, kpos = 0; gi < ng; gi++) {
+        const Node &g = gs[gi];
+        const int gg = key_b(g.key), nbG = ctx->nb_at[gg];
+        for (int k = 0; k < nbG; k++, kpos++) {
+          kmap.push_back(make_int4(gi, k, nbG, 0));
+          stage_mem[kpos / KC] |= g.mask;
+        }
+        for (int k = 0; k < nm; k++) {
+          if (g.q[k] < 0) {
+            segC.push_back(-1);
+            gpair.push_back(-1);
+            continue;
+          }
+          const int64_t p3 = ctx->partner1[g.q[k]];
+          const int qE0 = ctx->onsite[p3] ? 0 : ctx->na_at[gg];
+          segC.push_back(ctx->offC[p3] + (int64_t)qE0 * nbG * ctx->nb_at[gm[k].b]);
+          gpair.push_back((int32_t)p3);
+        }
       }
       for (int k = K; k < Kpad; k++) kmap.push_back(make_int4(-1, 0, 1, 0));
-      for (int qi = 0; qi < (int)qs.size(); qi++) {
-        const int64_t q = qs[qi];
-        const int a = ctx->pB[q];
+      std::vector<int> rt_mem(Mpad / TM, 0), ct_mem(Npad / TN, 0);  // members of every row and column tile
+      for (int qi = 0, rpos = 0; qi < (int)qs.size(); qi++) {
+        const Node &q = qs[qi];
+        const int a = key_b(q.key);
         const int nbA = ctx->nb_at[a], naA = ctx->na_at[a];
-        const int64_t vp = ctx->partner1[q];  // pair (A', E', -m)
-        int nm[3];
-        for (int c = 0; c < 3; c++) nm[c] = -(int)ctx->pn[3 * q + c];
-        const int64_t x = find_sorted(ctx->keys3, row3[a], row3[a + 1], pair_key(a, e, nm[0], nm[1], nm[2]));
-        if (x < 0) {
-          ctx->last_error = "term-1 plan: output block outside the K pattern";
-          return RIX_EINVAL;
+        for (int k = 0; k < nm; k++) {
+          if (q.q[k] < 0) {
+            qinfo.push_back(QInfo{0, -1, 0, nbA, 0});
+            continue;
+          }
+          const int64_t vp = ctx->partner1[q.q[k]];  // pair (A', E', -m)
+          int n3[3];
+          for (int c = 0; c < 3; c++) n3[c] = -(int)ctx->pn[3 * q.q[k] + c];
+          const int64_t x =
+              find_sorted(ctx->keys3, row3[a], row3[a + 1], pair_key(a, gm[k].b, n3[0], n3[1], n3[2]));
+          if (x < 0) {
+            ctx->last_error = "term-1 plan: output block outside the K pattern";
+            return RIX_EINVAL;
+          }
+          qinfo.push_back(QInfo{ctx->offV[vp], (int32_t)x, (int32_t)vp, nbA, ctx->rep1[vp] == 2 ? 1 : 0});
         }
-        qinfo.push_back(QInfo{ctx->offV[vp], (int32_t)x, (int32_t)vp, nbA, ctx->rep1[vp] == 2 ? 1 : 0});
-        for (int64_t g = row1[e]; g < row1[e + 1]; g++) {
+        for (const Node &g : gs) {
           int d[3];
-          for (int c = 0; c < 3; c++) d[c] = (int)ctx->pn[3 * g + c] - (int)ctx->pn[3 * q + c];
-          const int64_t t =
-              find_sorted(ctx->keys2, row2[a], row2[a + 1], pair_key(a, ctx->pB[g], d[0], d[1], d[2]));
+          for (int c = 0; c < 3; c++) d[c] = key_n(g.key, c) - key_n(q.key, c);
+          const int64_t t = find_sorted(ctx->keys2, row2[a], row2[a + 1], pair_key(a, key_b(g.key), d[0], d[1], d[2]));
           segT.push_back(t < 0 ? -1 : ctx->off2[t]);
           segR.push_back(t < 0 ? -1 : roff2[t]);
         }
-        for (int r = 0; r < naA * nbA; r++) {
+        for (int r = 0; r < naA * nbA; r++, rpos++) {
           rowinfo.push_back(make_int2(qi, r));
           rowprob.push_back(pidx);
+          rt_mem[rpos / TM] |= q.mask;
         }
       }
       for (int r = M; r < Mpad; r++) {
         rowinfo.push_back(make_int2(-1, 0));
         rowprob.push_back(pidx);
       }
-      for (int l = 0; l < nbE; l++)
-        for (int Q = 0; Q < naE; Q++) {
-          colinfo.push_back(make_int4(l, Q, nbE, naE));
-          colprob.push_back(pidx);
-        }
+      int cpos = 0;
+      for (int k = 0; k < nm; k++) {
+        const int nbE = ctx->nb_at[gm[k].b], naE = ctx->na_at[gm[k].b];
+        for (int l = 0; l < nbE; l++)
+          for (int Q = 0; Q < naE; Q++, cpos++) {
+            colinfo.push_back(make_int4(l | k << 16, Q, nbE, naE));
+            colprob.push_back(pidx);
+            ct_mem[cpos / TN] |= 1 << k;
+          }
+      }
       for (int c = N; c < Npad; c++) {
         colinfo.push_back(make_int4(-1, 0, 1, 1));
         colprob.push_back(pidx);
       }
-      push_tiles(tiles, pidx, Mpad / TM, Npad / TN, [](int, int) { return 0; });
+      const int64_t mbase = (int64_t)kmask.size();
+      kmask.resize(mbase + (int64_t)(Npad / TN) * mwords, 0ull);
+      std::vector<int> ct_stages(Npad / TN, 0);
+      for (int nt = 0; nt < Npad / TN; nt++)
+        for (int c = 0; c < Kpad / KC; c++)
+          if (stage_mem[c] & ct_mem[nt]) {
+            kmask[mbase + (int64_t)nt * mwords + (c >> 6)] |= 1ull << (c & 63);
+            ct_stages[nt]++;
+          }
+      const size_t tiles0 = tiles.size();
+      push_tiles_if(tiles, pidx, Mpad / TM, Npad / TN, [&](int, int nt) { return (int)(mbase + (int64_t)nt * mwords); },
+                    [&](int mt, int nt) { return (rt_mem[mt] & ct_mem[nt]) != 0; });
+      for (size_t i = tiles0; i < tiles.size(); i++) tflops += 2.0 * TM * TN * KC * ct_stages[tiles[i].z] * npairs;
       probs.push_back(pr);
       ext.push_back(ex);
       pbytes.push_back(bytes);
@@ -2609,6 +2712,7 @@ rix_status rix_t1_plan_build(rix_ctx *ctx, bool count_only, int64_t *bytes_out) 
   if ((s = rix_upload(ctx, &pl->d_segC, segC)) != RIX_OK) return s;
   if ((s = rix_upload(ctx, &pl->d_gpair, gpair)) != RIX_OK) return s;
   if ((s = rix_upload(ctx, &pl->d_qinfo, qinfo)) != RIX_OK) return s;
+  if ((s = rix_upload(ctx, &pl->d_kmask, kmask)) != RIX_OK) return s;
   if ((s = rix_alloc(ctx, &pl->d_eA, std::max<int64_t>(eaoff, 1))) != RIX_OK) return s;
   if ((s = rix_alloc(ctx, &pl->d_eB, std::max<int64_t>(eboff, 1))) != RIX_OK) return s;
   if ((s = pl->wsq.alloc(ctx, eaoff, eboff)) != RIX_OK) return s;
@@ -2681,6 +2785,7 @@ rix_status rix_mixed_t1(rix_ctx *ctx, int b, int64_t tbase, cudaStream_t st) {
                   1, pl->d_qinfo, ctx->d_V, ctx->d_keepV, 1.0};
       ga.ntiles = (int)(t1 - t0);
       ga.X128 = ctx->d_X128;  // deterministic builds: 128-bit fixed-point additions
+      ga.kmask = pl->d_kmask;
       pl->wsq.tiles(r0, r1, c0, c1, pl->kmax, st, ga);
       rix_status ls = launch_gemm(ctx, ga, t1 - t0, S, st);
       if (ls != RIX_OK) return ls;
