@@ -284,14 +284,14 @@ __global__ void __launch_bounds__(NT) k_U2(const int2 *items, const int32_t *pA,
                                            const int32_t *nb, const int32_t *na, const double *__restrict__ V,
                                            const int64_t *offV, const uint8_t *keepV, const int32_t *map1to2,
                                            const double *__restrict__ T, const int64_t *off2,
-                                           const int64_t *offU, double *U, int64_t tbase) {
+                                           const int64_t *offU, double *U, int64_t tbase, int cap) {
   const int2 it = items[blockIdx.x];
   const int p = it.x, q0 = it.y;
   if (!keepV[p]) return;
   const int a = pA[p], g = pB[p];
   const int nbA = nb[a], naA = na[a], nbG = nb[g], naG = na[g];
   const int per = nbA * nbG;
-  const int qt = max(1, CAP_MIN / per);
+  const int qt = max(1, cap / per);
   const int qe = min(naG, q0 + qt);
   const int nel = (qe - q0) * per;
   const double *Vb = V + offV[p];
@@ -815,6 +815,11 @@ namespace {
 
 void set_attrs() {
   if (!g_attr_done) {
+    // clusters of 16 CTAs are beyond the portable size
+    cudaFuncSetAttribute(k_X12<1>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaFuncSetAttribute(k_X12<XMAXE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaFuncSetAttribute(k_X34<1>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaFuncSetAttribute(k_X34<XMAXE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cudaFuncSetAttribute(k_X12<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_MAX * 8);
     cudaFuncSetAttribute(k_X12<XMAXE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_MAX * 8);
     cudaFuncSetAttribute(k_T, cudaFuncAttributeMaxDynamicSharedMemorySize, TCOL * 64 * 8);
@@ -984,7 +989,7 @@ rix_status rix_fp64_build(rix_ctx *ctx, const double *D, double *K, cudaStream_t
     if (nU) {
       k_U2<<<(unsigned)nU, NT, 0, st>>>(ctx->d_itU + ctx->segU[b], ctx->d_pA, ctx->d_pB, ctx->d_nb, ctx->d_na,
                                         ctx->d_V, ctx->d_offV, ctx->d_keepV, ctx->d_map1to2, ctx->d_T, ctx->d_off2,
-                                        ctx->d_offU, ctx->d_U, tbase);
+                                        ctx->d_offU, ctx->d_U, tbase, ctx->cap_U);
       if ((s = last(ctx, "k_U2")) != RIX_OK) return s;
     }
     if (b == 0 && (s = rix_prof_mark(ctx, 3, st)) != RIX_OK) return s;
@@ -1109,7 +1114,7 @@ extern "C" rix_status rix_autotune(rix_ctx *ctx, const double *D, const char *ca
   if (nU) {
     k_U2<<<(unsigned)nU, NT, 0, st>>>(ctx->d_itU + ctx->segU[b], ctx->d_pA, ctx->d_pB, ctx->d_nb, ctx->d_na,
                                       ctx->d_V, ctx->d_offV, ctx->d_keepV, ctx->d_map1to2, ctx->d_T, ctx->d_off2,
-                                      ctx->d_offU, ctx->d_U, ctx->blk_base[b]);
+                                      ctx->d_offU, ctx->d_U, ctx->blk_base[b], ctx->cap_U);
     if ((s = last(ctx, "k_U2")) != RIX_OK) return s;
   }
   float ms = 0.f;

@@ -88,8 +88,8 @@ struct BX12Entry {
   int32_t t1;    // 1 if term 1
 };
 
-// Output elements of a row-tiled work item: 32 or 4 per thread of a 256-thread CTA.
-constexpr int CAP_MAX = 8192, CAP_MIN = 1024;
+// Output elements of a row-tiled work item: 32, 4 or 1 per thread of a 256-thread CTA.
+constexpr int CAP_MAX = 8192, CAP_MID = 1024, CAP_MIN = 256;
 // Shared-memory tile of the adjoint kernels (doubles: three CTAs per SM), and the rows of a
 // kb_C12 item with it (U1 of every row for up to 64 functions i, nbG k each).
 constexpr int BWD_TILE = 9216;
@@ -229,7 +229,7 @@ struct rix_ctx {
   std::vector<int64_t> blk_base;                  // off2 of the block's first 2-hop block
   std::vector<int64_t> segT, segU, segZ;          // [nblk+1] ranges in the item arrays
   std::vector<int64_t> segX12;                    // [NCLS nblk + 1], see NCLS
-  int32_t cap_T = 0, cap_Z = 0;                   // output elements per T and Z item (CAP_MAX or CAP_MIN)
+  int32_t cap_T = 0, cap_Z = 0, cap_U = 0;        // output elements per T, Z and U2 item (CAP_*)
 
   // ------------------------------------------------------------ backward plan (opt.backward)
   bool have_bwd = false;
@@ -254,8 +254,8 @@ struct rix_ctx {
   // stays as it is: k_X34 stages nothing)
   int32_t tile_X12 = 4096, tile_Z = 12288, tile_X34 = 4096;
   // Launch classes of k_X12 and k_X34: class c holds the outputs shared by a cluster of 2^c CTAs
-  // (segX12[4 b + c] .. of block b, segX34[c] ..); max_nel, max_nb: the largest K block (elements) and atom (functions)
-  static constexpr int NCLS = 4;
+  // (segX12[NCLS b + c] .. of block b, segX34[c] ..); max_nel, max_nb: the largest K block (elements) and atom (functions)
+  static constexpr int NCLS = 5;
   std::vector<int64_t> segX34;
   int32_t max_nel = 0, max_nb = 0;
   // FP64 builds with screening: per build, whether each T and Z block ([n2] each) has a kept product

@@ -730,13 +730,15 @@ static rix_status build_lists(rix_ctx *ctx) {
   // ---------------------------------------------------------------- work items and launch orders
   // Row tiles of T and Z (a block's P rows, CAP output elements per item at most) and of U2.
   // 8192 elements (32 per thread) re-read the operands least; a system whose stage would have
-  // fewer than 32 items per SM takes 1024, so that its longest item does not run on alone (the
-  // sums do not depend on the tile).  U2 has one product per output and always takes 1024.
+  // fewer than 32 items per SM takes 1024, and 256 with fewer than 4 of those, so that its longest
+  // item does not run on alone (the sums do not depend on the tile).  U2 has one product per
+  // output and takes 1024 at most.  (Two waters, 1024 -> 256
+  // elements: Z 66 -> 48 us, U2 28 -> 12 us; (H2O)8 keeps 1024, where U2 and Z have items enough.)
   std::vector<int2> itT, itZ, itU;
   std::vector<double> cT, cZ;
   auto tile2 = [&](const std::vector<int64_t> &ptr, std::vector<int2> &it, std::vector<double> &c, bool empty) {
     int64_t cap = CAP_MAX;
-    for (;; cap = CAP_MIN) {
+    for (;; cap = cap == CAP_MAX ? CAP_MID : CAP_MIN) {
       for (int64_t t = 0; t < n2; t++) {
         const int a = atomA2[t];
         const int64_t per = NB(a) * NB(atomB2[t]), pt = std::max<int64_t>(1, cap / per);
@@ -747,18 +749,21 @@ static rix_status build_lists(rix_ctx *ctx) {
           c.push_back(len * std::min(pt, NA(a) - p0) * per);
         }
       }
-      if (cap == CAP_MIN || it.size() >= 32 * 152) return (int32_t)cap;
+      if (cap == CAP_MIN || it.size() >= (cap == CAP_MAX ? 32 : 4) * 152) return (int32_t)cap;
       it.clear();
       c.clear();
     }
   };
   ctx->cap_T = tile2(ptrT, itT, cT, true);
   ctx->cap_Z = tile2(ptrZ, itZ, cZ, false);
-  for (int64_t p = 0; p < np; p++) {
-    int a = pA[p], g = pB[p];
-    int64_t per = NB(a) * NB(g);
-    int64_t qt = std::max<int64_t>(1, CAP_MIN / per);
-    for (int64_t q0 = 0; q0 < NA(g); q0 += qt) itU.push_back(make_int2((int)p, (int)q0));
+  for (ctx->cap_U = CAP_MID;; ctx->cap_U = CAP_MIN) {
+    itU.clear();
+    for (int64_t p = 0; p < np; p++) {
+      const int a = pA[p], g = pB[p];
+      const int64_t qt = std::max<int64_t>(1, ctx->cap_U / (NB(a) * NB(g)));
+      for (int64_t q0 = 0; q0 < NA(g); q0 += qt) itU.push_back(make_int2((int)p, (int)q0));
+    }
+    if (ctx->cap_U == CAP_MIN || itU.size() >= 4 * 152) break;
   }
   // launch order: most expensive first (longest processing time first)
   auto order_by = [](std::vector<int2> &it, const std::vector<double> &cost) {
@@ -782,9 +787,10 @@ static rix_status build_lists(rix_ctx *ctx) {
       const double t1 = pae >= 0 && ctx->rep1[pae] ? (double)NA(e) * NB(a) * (NA(a) + NB(e)) : 0.0;
       cX12.push_back((double)(ptrX12[s + 1] - ptrX12[s]) * (t1 + (double)NA(a) * NB(a) * NB(e)));
     }
-  // A cluster of 2^c CTAs per output (1, 2, 4 or 8) where the longest output of its component
+  // A cluster of 2^c CTAs per output (1 to 16) where the longest output of its component
   // would otherwise take more than half of an even share of the stage on the 152 SMs: its CTA
-  // would run on alone at the end.
+  // would run on alone at the end.  (Two waters, at most 8 -> 16 CTAs: terms 1+2 168 -> 107 us,
+  // terms 3+4 27 -> 20 us.)
   auto clusters = [&](const std::vector<int32_t> &ord, const std::vector<double> &c, auto atom) {
     std::vector<double> tot(ctx->ncomp, 0.0), top(ctx->ncomp, 0.0);
     for (size_t i = 0; i < ord.size(); i++) {
