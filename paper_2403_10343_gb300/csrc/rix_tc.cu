@@ -1411,13 +1411,15 @@ struct rix_digit_sums {
     if ((s = rix_alloc(ctx, &ta, std::max<int64_t>(rows / rixtc::TM, 1))) != RIX_OK) return s;
     return rix_alloc(ctx, &tb, std::max<int64_t>(cols / rixtc::TN, 1));
   }
+  // whether a plan's tiles can be longer than a group
+  static bool needed(int kmax) { return kmax > rixtc::GROUP * rixtc::KC; }
   // device bytes of `rows` packed rows and `cols` columns (whole tiles)
   static int64_t bytes(int64_t rows, int64_t cols) { return 4 * (rows + cols + rows / rixtc::TM + cols / rixtc::TN); }
   // the tiles of packed rows [r0, r1) and columns [c0, c1), into the GEMM's arguments
   void tiles(int64_t r0, int64_t r1, int64_t c0, int64_t c1, int kmax, cudaStream_t st, rixtc::GemmArgs &ga) const {
     const int64_t a0 = r0 / rixtc::TM, a1 = r1 / rixtc::TM, b0 = c0 / rixtc::TN, b1 = c1 / rixtc::TN;
     const int64_t n = (a1 - a0) + (b1 - b0);
-    if (n <= 0 || kmax <= rixtc::GROUP * rixtc::KC) return;  // no tile is longer than a group
+    if (n <= 0 || !needed(kmax)) return;
     rixtc::k_tile_wsq<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>(a0, a1, b0, b1, a, b, ta, tb);
     ga.tA = ta;
     ga.tB = tb;
@@ -2049,14 +2051,15 @@ rix_status rix_mixed_plan(rix_ctx *ctx, const std::vector<int64_t> &ptrZ) {
 }
 
 // Kernel launches of one rix_build_K: flags, per block T, U2 and Z, terms 1+2 and
-// terms 3+4 (FP64 per block) or per group five slicing kernels and a GEMM
-// (mixed), symmetrise.
+// terms 3+4 (FP64 per block) or per group four slicing kernels, the tiles' digit
+// sums where a tile can be longer than an accumulation group, and a GEMM (mixed),
+// symmetrise.
 int32_t rix_launch_count(const rix_ctx *ctx) {
   int32_t n = 2 + 3 * ctx->nblk + (ctx->use_live ? 2 : 0);
   if (ctx->have_mx) {
-    // per group: exponents and digits of both operands, the tiles' digit sums, the GEMM
-    n += 6 * (int32_t)(ctx->mx34->grp.size() - 1) + 6 * (int32_t)(ctx->mx2->grp.size() - 1) +
-         6 * (int32_t)(ctx->mxz->grp.size() - 1) + rix_t1_launches(ctx) + rix_tt_launches(ctx);
+    for (const rix_mx_plan *pl : {ctx->mx34, ctx->mx2, ctx->mxz})
+      n += (5 + rix_digit_sums::needed(pl->kmax)) * (int32_t)(pl->grp.size() - 1);
+    n += rix_t1_launches(ctx) + rix_tt_launches(ctx);
     if (ctx->n_t1tc < ctx->nat) n += rix_x12_launches(ctx);  // k_X12 for the other column atoms
     if (ctx->n_ztc == ctx->nat) n -= ctx->nblk;   // no k_Z: the Z buffer is zeroed by a memset
     // row-tile K-stage masks: once per Z block, once per terms-3+4 block, once for term 2
@@ -2805,7 +2808,8 @@ int32_t rix_t1_launches(const rix_ctx *ctx) {
   int32_t n = 0, last_blk = -1;
   for (size_t g = 0; g + 1 < pl->grp_prob.size(); g++) {
     if (pl->grp_prob[g + 1] == pl->grp_prob[g]) continue;
-    n += 6;  // row exponents and digits, column exponents and digits, digit sums, the GEMM
+    // row exponents and digits, column exponents and digits, digit sums, the GEMM
+    n += 5 + rix_digit_sums::needed(pl->kmax);
     if (pl->grp_blk[g] != last_blk) n++;  // k_rowexp, once per block (groups are in block order)
     last_blk = pl->grp_blk[g];
   }
@@ -3330,7 +3334,8 @@ rix_status rix_mixed_T(rix_ctx *ctx, int b, int64_t tbase, const double *D, cuda
 int32_t rix_tt_launches(const rix_ctx *ctx) {
   if (!ctx->mxt) return 0;
   const int32_t ng = (int32_t)(ctx->mxt->grp_prob.size() - 1);
-  return 6 * ng + (ctx->mxt->n_mask > 0 ? 1 : 0) + (ng > 0 ? 1 : 0);  // + k_tt_mask, k_dcolexp
+  return (5 + rix_digit_sums::needed(ctx->mxt->kmax)) * ng + (ctx->mxt->n_mask > 0 ? 1 : 0) +
+         (ng > 0 ? 1 : 0);  // + k_tt_mask, k_dcolexp
 }
 
 extern "C" rix_status rix_gemm_profile(rix_ctx *ctx, double *ms, int64_t *launches, int64_t *chunks) {
