@@ -133,6 +133,8 @@ struct rix_ctx {
 
   // ------------------------------------------------------------ device
   std::vector<rix::DevBuf> bufs;
+  char *chunk = nullptr;   // the free end of the chunk that small arrays share (one of bufs)
+  size_t chunk_left = 0;
   size_t dev_bytes = 0;
   // atoms
   int32_t *d_nb = nullptr, *d_na = nullptr;
