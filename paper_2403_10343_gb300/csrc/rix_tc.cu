@@ -16,8 +16,8 @@
 // Slice s is stored pre-scaled by 2^-7(s-1) (exact in BF16), so a product
 // carries its own power of two.  Six FP32 accumulators in tensor memory take
 // the products with s+t = 2, 3, 4, 5, 6 and s+t >= 7: by those bounds the
-// first five hold integers (times 2^-7(s+t-2)) below 2^24 over a group of 512
-// K values, so the tensor cores accumulate them exactly; the sixth holds
+// first five hold integers (times 2^-7(s+t-2)) below 2^24 over a group of 576
+// K values (longer where the operands' digits are known to be small), so the tensor cores accumulate them exactly; the sixth holds
 // terms at least 2^-35 below the leading one, where the tensor cores' FP32
 // accumulation costs about 2^-53 of the row x column x K scale.  After each
 // group the accumulators are folded into a 64-bit fixed-point sum per output
@@ -2062,6 +2062,7 @@ int32_t rix_launch_count(const rix_ctx *ctx) {
     n += rix_t1_launches(ctx) + rix_tt_launches(ctx);
     if (ctx->n_t1tc < ctx->nat) n += rix_x12_launches(ctx);  // k_X12 for the other column atoms
     if (ctx->n_ztc == ctx->nat) n -= ctx->nblk;   // no k_Z: the Z buffer is zeroed by a memset
+    if (ctx->n_ttc == ctx->nat) n -= ctx->nblk;   // nor k_T
     // row-tile K-stage masks: once per Z block, once per terms-3+4 block, once for term 2
     if (ctx->mxz->n_rt > 0) n += ctx->nblk;
     if (ctx->mx34->n_rt > 0) n += ctx->nblk;
