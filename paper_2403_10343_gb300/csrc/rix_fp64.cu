@@ -335,7 +335,9 @@ __device__ __forceinline__ Split split_of(int nel, int rank, int ns) {
 }
 
 // acc[r] += sum over this share of the rows (P, j) of a[P][i][j] b[P][j][l] (a: nP x nbA x nbJ,
-// b: nP x nbJ x nbE); element el = i nbE + l.
+// b: nP x nbJ x nbE); element el = i nbE + l.  The share is summed by itself before it is added:
+// sums of sums round less than one long chain ((H2O)64, terms 1-4 together: relative error of K
+// 9.5e-15 -> 1.1e-15 for 657 -> 660 ms).
 template <int R>
 __device__ __forceinline__ void dot_share(double (&acc)[R], const Split &s, int nel, const double *__restrict__ a,
                                           const double *__restrict__ b, int nP, int nbA, int nbJ, int nbE) {
@@ -350,7 +352,7 @@ __device__ __forceinline__ void dot_share(double (&acc)[R], const Split &s, int 
       const int i = el / nbE, l = el - i * nbE;
       const double *ap = a + ((int64_t)P0 * nbA + i) * nbJ + j0;
       const double *bp = b + (int64_t)k0 * nbE + l;
-      double v = acc[r];
+      double v = 0.0;
       int j = j0;
 #pragma unroll 4
       for (int k = k0; k < k1; k++) {
@@ -362,7 +364,7 @@ __device__ __forceinline__ void dot_share(double (&acc)[R], const Split &s, int 
           ap += (nbA - 1) * nbJ;
         }
       }
-      acc[r] = v;
+      acc[r] += v;
     }
   }
 }
@@ -522,7 +524,7 @@ __global__ void __launch_bounds__(NT, R == 1 ? 4 : 1)
               const int i = el / nbE, l = el - i * nbE;
               int q = k0 / n, c = k0 - q * n;
               const double *up = sm + ((int64_t)q * nbA + i) * n + c;
-              double v = acc[r];
+              double v = 0.0;
 #pragma unroll 4
               for (int k = k0; k < k1; k++) {
                 v = fma(*up, __ldg(C + tb.c[c] + (int64_t)(q0 + q) * (tb.nb[c] * nbE) + l), v);
@@ -533,7 +535,7 @@ __global__ void __launch_bounds__(NT, R == 1 ? 4 : 1)
                   up += (nbA - 1) * n;
                 }
               }
-              acc[r] = v;
+              acc[r] += v;
             }
           }
         }
