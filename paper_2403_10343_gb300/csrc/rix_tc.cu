@@ -1532,11 +1532,12 @@ namespace {
 
 int plan_slices(const rix_ctx *ctx, int kind) { return rix_plan_slices(ctx, kind); }
 
-// Rates measured on GB300 (the (H2O)64 and 768-atom ice builds) for the
-// choice between an FP64 kernel and a tensor-core regrouping: the FP64 kernels
-// of term 1 (k_X12, ~0.7 TFLOP/s), of Z (k_Z, ~1.2) and of T (k_T, ~1.0), and
-// the sliced GEMM with its slicing kernels (~0.75 PFLOP/s issued).
-constexpr double FP64_RATE_T1 = 0.7e12, FP64_RATE_Z = 1.2e12, FP64_RATE_T = 1.0e12, TC_RATE = 7.5e14;
+// Rates measured on GB300 (the (H2O)64 build and the 192-atom periodic ice) for the choice
+// between an FP64 kernel and a tensor-core regrouping: the FP64 kernels of term 1 (k_X12, 1.14
+// TFLOP/s), of Z (k_Z, 1.13) and of T (k_T, 1.16), and the sliced GEMM with its slicing kernels
+// (1.4 and 1.3 PFLOP/s issued).  (At 0.75 PFLOP/s, the rate of an earlier GEMM,
+// a 12-atom perovskite kept its heaviest middle atom on k_Z: 128.3 ms, and 127.2 on the tensor cores.)
+constexpr double FP64_RATE_T1 = 1.14e12, FP64_RATE_Z = 1.13e12, FP64_RATE_T = 1.16e12, TC_RATE = 1.3e15;
 
 // Middle atoms within this distance of a group's first atom join its problem (2.5 A).
 constexpr double GROUP_R = 2.5 / 0.529177210903;
