@@ -284,11 +284,11 @@ def max_over_ranks(x, world, dev):
 
 
 # DRAM bytes (read + write) per MMA of k_gemm_sliced (one 128 x 80 x 16 product of one slice
-# pair): ncu dram__bytes_read.sum + dram__bytes_write.sum over the 13 GEMM launches of a
-# (H2O)64 cluster build (192 atoms; 1.59e11 bytes for 4.65e8 MMAs, three builds 337-343),
+# pair): ncu dram__bytes_read.sum + dram__bytes_write.sum over the 7 GEMM launches of a
+# (H2O)64 cluster build (192 atoms; 8.4e10 bytes for 3.22e8 MMAs, two builds 261-262),
 # scaled to a launch of the bench workload by its MMA count (None: not measured for the
 # kernel as it stands)
-GEMM_DRAM_BYTES_PER_STAGE_PAIR = 340.0
+GEMM_DRAM_BYTES_PER_STAGE_PAIR = 261.0
 GEMM_STAGE_PAIR_FLOPS = 2.0 * 128 * 80 * 16
 
 

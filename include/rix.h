@@ -188,10 +188,11 @@ rix_status rix_layout_sizes(const rix_ctx *ctx, int64_t *c_elems, int64_t *v_ele
 rix_status rix_set_CV(rix_ctx *ctx, const double *C_dev, const double *V_dev, void *stream);
 
 /* Autotuner (no counterpart in the paper's code path beyond its auto-tuned
- * Fock-matrix block size): picks the shared-memory tile budget of the three
- * FP64 contraction kernels (terms 1+2, the term-4 intermediate Z, terms 3+4)
- * by timing four candidates on a slice of this system's own work items with
- * the density matrix D_dev (device, packed).  Needs rix_set_CV first.
+ * Fock-matrix block size): picks the shared-memory tile budget of the FP64
+ * contraction kernels (terms 1+2, the term-4 intermediate Z; terms 3+4 stage
+ * nothing and keep their entry as it is) by timing four candidates on a slice of
+ * this system's own work items with the density matrix D_dev (device, packed).
+ * Needs rix_set_CV first.
  * cache_path (may be NULL): a text file of "key x12 z x34" lines; a line
  * whose key (device name and list sizes) matches is applied without timing,
  * and a new choice is appended.  chosen (may be NULL) receives the three

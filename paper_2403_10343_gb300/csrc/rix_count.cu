@@ -4,10 +4,12 @@
 // include every product.  The build then skips the products whose C, V or D
 // block is below the screening threshold tau (Sec. "Screening": a block is
 // negligible when its largest element is below tau), and which blocks of D are
-// negligible is known only once D is.  These kernels walk the same product
-// lists as the FP64 stage kernels, apply the same tests to the same flags and
+// negligible is known only once D is.  These kernels walk the product lists of
+// the grouping, apply the tests of the stage kernels to the same flags and
 // add up 2 x multiply-adds of every product that is kept, so that a stage's
-// throughput can be quoted on the work it actually does.  Every count is an
+// throughput can be quoted on that work.  (A build may do less: it takes the
+// cheaper half of term 4, and the FP64 kernels also skip the products of a T or
+// Z block that screening left empty, which these counts include.)  Every count is an
 // integer below 2^53 and every partial sum is exact in FP64, so the atomic
 // order does not matter.
 #include "rix_internal.h"
