@@ -1124,7 +1124,7 @@ __device__ __forceinline__ bool dig_live(const Acc &, const typename Acc::Row &,
 
 // W warps per row (eight warps to a CTA): four where the plan has few rows.
 template <class Acc, int W>
-__global__ void __launch_bounds__(256) k_slice_exp(int64_t n0, int64_t n, Acc acc, int *e, float *wsq) {
+__global__ void __launch_bounds__(256) k_slice_exp(int64_t n0, int64_t n, Acc acc, int *e, uint64_t *wsq) {
   __shared__ int red[8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t w = n0 + blockIdx.x * (int64_t)(8 / W) + warp / W;
@@ -1149,17 +1149,18 @@ __global__ void __launch_bounds__(256) k_slice_exp(int64_t n0, int64_t n, Acc ac
   }
   if (in && warp % W == 0 && lane == 0) {
     e[(acc.is_b ? R.pr.eboff : R.pr.eaoff) + R.r] = m;
-    wsq[(acc.is_b ? R.pr.eboff : R.pr.eaoff) + R.r] = 0.f;
+    wsq[(acc.is_b ? R.pr.eboff : R.pr.eaoff) + R.r] = 0;
   }
 }
 
 // K values [kper blockIdx.y, + kper) of the rows (kper a multiple of 32): a plan with few rows
-// spreads its K over the grid's y.  wsq: the sum of the squares of a row's digits, all slices (an
-// upper bound: 2^-6 covers the FP32 rounding of up to 2^18 additions per thread, K = 131,072), which
-// decides how long the GEMM may accumulate; the exponent pass has set it to 0.
+// spreads its K over the grid's y.  wsq: the sum of the squares of a row's digits, all slices, which
+// decides how long the GEMM may accumulate; the exponent pass has set it to 0.  It is a whole number,
+// summed exactly, so that the decision depends neither on the split nor on the order of the atomics
+// (where the fixed point drops bits, K > 2,048 at six slices, a sum depends on its groups).
 template <class Acc, int S>
 __global__ void __launch_bounds__(256, 4)
-    k_slice_dig(int64_t n0, int64_t n, Acc acc, __nv_bfloat16 *planes, const int *e, float *wsq, int kper) {
+    k_slice_dig(int64_t n0, int64_t n, Acc acc, __nv_bfloat16 *planes, const int *e, uint64_t *wsq, int kper) {
   const int64_t g8 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (g8 * 8 >= n) return;  // n is a multiple of 8 (problems pad to whole tiles)
@@ -1171,42 +1172,45 @@ __global__ void __launch_bounds__(256, 4)
   const int nkt = R.pr.Kpad / KC;
   char *base = (char *)planes + (acc.is_b ? R.pr.boff : R.pr.aoff);
   const int rt = R.r / trows, rr = R.r % trows;
-  float W = 0.f;
+  uint32_t W32 = 0;  // below 2^32: kper is at most 2^18
   for (int k0 = blockIdx.y * kper + (lane >> 3) * 8; k0 < kend; k0 += 32) {
     if (!dig_live(acc, R, k0)) continue;  // a stage the GEMM skips: its tile is never read
     // the eight loads first (independent, so their latencies overlap), then the digits
     double v[8];
     load8(acc, R, k0, v);
     uint32_t pk[4][S];
+    float sq = 0.f;  // exact: at most 8 (128^2 + 7 64^2)
 #pragma unroll
-    for (int j = 0; j < 4; j++) digit_pairs<S>(v[2 * j], v[2 * j + 1], m, pk[j], W);
+    for (int j = 0; j < 4; j++) digit_pairs<S>(v[2 * j], v[2 * j + 1], m, pk[j], sq);
+    W32 += __float2uint_rn(sq);
     const int64_t off = ((int64_t)rt * nkt + k0 / KC) * S * tbytes + tile_off(rr, k0 % KC);
 #pragma unroll
     for (int t = 0; t < S; t++)
       *reinterpret_cast<uint4 *>(base + t * tbytes + off) = make_uint4(pk[0][t], pk[1][t], pk[2][t], pk[3][t]);
   }
+  unsigned long long W = W32;
   W += __shfl_xor_sync(0xffffffffu, W, 8);
   W += __shfl_xor_sync(0xffffffffu, W, 16);
   if (lane < 8) {
-    float *d = wsq + (acc.is_b ? R.pr.eboff : R.pr.eaoff) + R.r;
-    W *= 1.f + 1.f / 64.f;
-    if (gridDim.y > 1) atomicAdd(d, W);
+    uint64_t *d = wsq + (acc.is_b ? R.pr.eboff : R.pr.eaoff) + R.r;
+    if (gridDim.y > 1) atomicAdd((unsigned long long *)d, W);
     else *d = W;
   }
 }
 
-// Largest wsq of every row tile in [a0, a1) and column tile in [b0, b1), one warp per tile.
-__global__ void k_tile_wsq(int64_t a0, int64_t a1, int64_t b0, int64_t b1, const float *wA, const float *wB, float *tA,
-                           float *tB) {
+// Largest wsq of every row tile in [a0, a1) and column tile in [b0, b1), rounded up to FP32, one
+// warp per tile.
+__global__ void k_tile_wsq(int64_t a0, int64_t a1, int64_t b0, int64_t b1, const uint64_t *wA, const uint64_t *wB,
+                           float *tA, float *tB) {
   const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   const bool is_b = w >= a1 - a0;
   const int64_t tile = is_b ? b0 + (w - (a1 - a0)) : a0 + w;
   if (is_b && tile >= b1) return;
   const int n = is_b ? TN : TM;
-  const float *src = (is_b ? wB : wA) + tile * n;
+  const uint64_t *src = (is_b ? wB : wA) + tile * n;
   float m = 0.f;
-  for (int i = lane; i < n; i += 32) m = fmaxf(m, src[i]);
+  for (int i = lane; i < n; i += 32) m = fmaxf(m, __ull2float_ru(src[i]));
   for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
   if (lane == 0) (is_b ? tB : tA)[tile] = m;
 }
@@ -1214,7 +1218,7 @@ __global__ void k_tile_wsq(int64_t a0, int64_t a1, int64_t b0, int64_t b1, const
 // exponents and digit planes of rows [n0, n0 + n) (n a multiple of 8): the exponent pass,
 // then the digit pass
 template <class Acc>
-void slice_rows(int64_t n0, int64_t n, const Acc &acc, int S, __nv_bfloat16 *planes, int *e, float *wsq, int kmax,
+void slice_rows(int64_t n0, int64_t n, const Acc &acc, int S, __nv_bfloat16 *planes, int *e, uint64_t *wsq, int kmax,
                 cudaStream_t st);
 
 // k_slice_dig over rows [n0, n0 + n) (n a multiple of 8, K at most kmax) for S slices.  A warp
@@ -1222,11 +1226,11 @@ void slice_rows(int64_t n0, int64_t n, const Acc &acc, int S, __nv_bfloat16 *pla
 // are split, down to 32 per warp ((H2O)8: the digits of terms 2 and 3+4 were 130 us per launch on
 // 130 warps, 13 us now).
 template <class Acc>
-void launch_slice_dig(int64_t n0, int64_t n, const Acc &acc, int S, __nv_bfloat16 *planes, const int *e, float *wsq,
+void launch_slice_dig(int64_t n0, int64_t n, const Acc &acc, int S, __nv_bfloat16 *planes, const int *e, uint64_t *wsq,
                       int kmax, cudaStream_t st) {
   const int64_t warps = n / 8, k32 = (kmax + 31) / 32;
   const int64_t ny = std::min<int64_t>(k32, (152 * 32 + warps - 1) / warps);
-  const int kper = (int)((k32 + ny - 1) / ny) * 32;
+  const int kper = std::min((int)((k32 + ny - 1) / ny) * 32, 1 << 18);
   const dim3 grid((unsigned)((warps * 32 + 255) / 256), (unsigned)((kmax + kper - 1) / kper));
   switch (S) {
     case 1: k_slice_dig<Acc, 1><<<grid, 256, 0, st>>>(n0, n, acc, planes, e, wsq, kper); break;
@@ -1241,7 +1245,7 @@ void launch_slice_dig(int64_t n0, int64_t n, const Acc &acc, int S, __nv_bfloat1
 }
 
 template <class Acc>
-void slice_rows(int64_t n0, int64_t n, const Acc &acc, int S, __nv_bfloat16 *planes, int *e, float *wsq, int kmax,
+void slice_rows(int64_t n0, int64_t n, const Acc &acc, int S, __nv_bfloat16 *planes, int *e, uint64_t *wsq, int kmax,
                 cudaStream_t st) {
   if (n <= 0) return;
   if (n < 152 * 32) k_slice_exp<Acc, 4><<<(unsigned)((n + 1) / 2), 256, 0, st>>>(n0, n, acc, e, wsq);
@@ -1330,7 +1334,7 @@ __device__ __forceinline__ void load8(const SrcAcc &acc, SrcAcc::Row &R, int k0,
 // the product of the two maximising entries: the same FP64 product, hence the same
 // exponent, as the element-wise pass, from na + nb loads per member instead of
 // na nb products.
-__global__ void k_kron_exp(int64_t n0, int64_t n, SrcAcc acc, int *e, float *wsq) {
+__global__ void k_kron_exp(int64_t n0, int64_t n, SrcAcc acc, int *e, uint64_t *wsq) {
   const int64_t w = n0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (w >= n0 + n) return;
   const SrcAcc::Row R = acc.row(w);
@@ -1348,7 +1352,7 @@ __global__ void k_kron_exp(int64_t n0, int64_t n, SrcAcc acc, int *e, float *wsq
     m = max(m, exp_of(sr.flag & XHALF ? 0.5 * (mv * md) : mv * md));
   }
   e[R.pr.eaoff + R.r] = m;
-  wsq[R.pr.eaoff + R.r] = 0.f;
+  wsq[R.pr.eaoff + R.r] = 0;
 }
 
 // Per row tile r of a grouped plan, for this build: bit c of its K-stage mask is set
@@ -1403,7 +1407,8 @@ __global__ void k_flag_set(int n, const int32_t *idx, uint8_t *flags) {
 
 // Sums of the squares of the digits of every packed row and column, and the largest per tile.
 struct rix_digit_sums {
-  float *a = nullptr, *b = nullptr, *ta = nullptr, *tb = nullptr;
+  uint64_t *a = nullptr, *b = nullptr;
+  float *ta = nullptr, *tb = nullptr;
   rix_status alloc(rix_ctx *ctx, int64_t rows, int64_t cols) {
     rix_status s;
     if ((s = rix_alloc(ctx, &a, std::max<int64_t>(rows, 1))) != RIX_OK) return s;
@@ -1414,7 +1419,7 @@ struct rix_digit_sums {
   // whether a plan's tiles can be longer than a group
   static bool needed(int kmax) { return kmax > rixtc::GROUP * rixtc::KC; }
   // device bytes of `rows` packed rows and `cols` columns (whole tiles)
-  static int64_t bytes(int64_t rows, int64_t cols) { return 4 * (rows + cols + rows / rixtc::TM + cols / rixtc::TN); }
+  static int64_t bytes(int64_t rows, int64_t cols) { return 8 * (rows + cols) + 4 * (rows / rixtc::TM + cols / rixtc::TN); }
   // the tiles of packed rows [r0, r1) and columns [c0, c1), into the GEMM's arguments
   void tiles(int64_t r0, int64_t r1, int64_t c0, int64_t c1, int kmax, cudaStream_t st, rixtc::GemmArgs &ga) const {
     const int64_t a0 = r0 / rixtc::TM, a1 = r1 / rixtc::TM, b0 = c0 / rixtc::TN, b1 = c1 / rixtc::TN;
@@ -2384,7 +2389,7 @@ __global__ void k_rowexp(int64_t t0, const int64_t *off2, const int64_t *roff2, 
 // row: the rows of a warp are neighbours in every block, so its loads are contiguous (a warp per
 // row, lanes over g, took 4.0 ms per build of the 192-atom ice cell, 1.1 ms now).
 __global__ void k_t1_exp(int64_t n0, int64_t n, T1RowAcc acc, const int64_t *segR, const int *rexp,
-                         int64_t rbase, int *e, float *wsq) {
+                         int64_t rbase, int *e, uint64_t *wsq) {
   const int64_t w = n0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (w >= n0 + n) return;
   const T1RowAcc::Row R = acc.row(w);
@@ -2400,7 +2405,7 @@ __global__ void k_t1_exp(int64_t n0, int64_t n, T1RowAcc acc, const int64_t *seg
     }
   }
   e[R.pr.eaoff + R.r] = m;
-  wsq[R.pr.eaoff + R.r] = 0.f;
+  wsq[R.pr.eaoff + R.r] = 0;
 }
 
 }  // namespace rixtc
@@ -2982,7 +2987,7 @@ __global__ void k_dcolexp(int64_t np, const int32_t *pA, const int32_t *pB, cons
 // D(B', G'_t) of the column's T block (its product list) of their column-k maxima,
 // which is the largest exponent over the column's K values (the rest are zero).
 __global__ void k_tt_colexp(int64_t n0, int64_t n, TTColAcc acc, const int64_t *dcoff, const int *dcolexp,
-                            int *e, float *wsq) {
+                            int *e, uint64_t *wsq) {
   const int64_t w = n0 + ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (w >= n0 + n) return;
@@ -2997,7 +3002,7 @@ __global__ void k_tt_colexp(int64_t n0, int64_t n, TTColAcc acc, const int64_t *
   for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
   if (lane == 0) {
     e[R.pr.eboff + R.r] = m;
-    wsq[R.pr.eboff + R.r] = 0.f;
+    wsq[R.pr.eboff + R.r] = 0;
   }
 }
 
