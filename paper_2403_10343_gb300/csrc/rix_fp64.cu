@@ -1042,7 +1042,9 @@ std::string tune_key(const rix_ctx *ctx) {
   cudaGetDevice(&dev);
   cudaGetDeviceProperties(&prop, dev);
   char buf[512];
-  snprintf(buf, sizeof buf, "%s|nat=%d|np=%lld|n2=%lld|nk=%lld|prec=%d|blk=%d|", prop.name, ctx->nat,
+  // k2: the kernels the tiles were timed with; a choice made for others (96 KB a CTA, where k_X12
+  // now takes 32 KB) is not theirs
+  snprintf(buf, sizeof buf, "%s|k2|nat=%d|np=%lld|n2=%lld|nk=%lld|prec=%d|blk=%d|", prop.name, ctx->nat,
            (long long)ctx->np, (long long)ctx->n2, (long long)ctx->nk, (int)ctx->opt.precision, ctx->nblk);
   std::string k(buf);
   for (char &c : k)
