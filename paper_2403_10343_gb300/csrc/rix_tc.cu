@@ -16,8 +16,9 @@
 // Slice s is stored pre-scaled by 2^-7(s-1) (exact in BF16), so a product
 // carries its own power of two.  Six FP32 accumulators in tensor memory take
 // the products with s+t = 2, 3, 4, 5, 6 and s+t >= 7: by those bounds the
-// first five hold integers (times 2^-7(s+t-2)) below 2^24 over a group of 576
-// K values (longer where the operands' digits are known to be small), so the tensor cores accumulate them exactly; the sixth holds
+// first five hold integers (times 2^-7(s+t-2)) below 2^24 over a group of 512
+// K values (longer where the operands' digits are known to be small), so the tensor cores accumulate
+// them exactly; so does the sixth up to six slices, where it holds one diagonal.  With more it holds
 // terms at least 2^-35 below the leading one, where the tensor cores' FP32
 // accumulation costs about 2^-53 of the row x column x K scale.  After each
 // group the accumulators are folded into a 64-bit fixed-point sum per output
@@ -45,18 +46,20 @@ namespace rixtc {
 constexpr int TM = 128;         // output rows per tile (one TMEM lane each)
 constexpr int TN = 80;          // output columns per tile
 constexpr int KC = 16;          // K per pipeline stage (one MMA K step)
-// Accumulation groups of GROUP K stages (576 K values, the most that stays exact whatever the
-// digits are; a tile whose digits are known to be small enough is one group, see
-// TileInfo::group).  Accumulator a < NACC-1
+// Accumulation groups of GROUP K stages (512 K values, the most that stays exact at six slices
+// whatever the digits are; a tile whose digits are known to be small enough is one group, see
+// TileInfo::group).  Accumulator a < NACC-1, and at six slices the last one too,
 // holds diagonal a: pairs (0, a) and (a, 0) with a leading digit (<= 128)
 // and a balanced one (<= 64), and a - 1 pairs of balanced digits (a = 0: the
-// one pair of leading digits), so its sum stays an integer below 2^24.
-constexpr int GROUP = 36;
+// one pair of leading digits), so its sum stays an integer of at most 2^24.  (Groups of 576,
+// exact in the first five accumulators only, lose units of the sixth for 0.3 % of the 12-atom
+// perovskite's build, 126.9 and 127.3 ms; the water and ice builds take the same time.)
+constexpr int GROUP = 32;
 constexpr int64_t diag_bound(int a) {  // largest |sum over one K value| of diagonal a
   return a == 0 ? 128 * 128 : 2 * 128 * 64 + (int64_t)(a - 1) * 64 * 64;
 }
-constexpr bool exact_group(int a) { return diag_bound(a) * GROUP * KC < ((int64_t)1 << 24); }
-static_assert(exact_group(0) && exact_group(1) && exact_group(2) && exact_group(3) && exact_group(4),
+constexpr bool exact_group(int a) { return diag_bound(a) * GROUP * KC <= ((int64_t)1 << 24); }
+static_assert(exact_group(0) && exact_group(1) && exact_group(2) && exact_group(3) && exact_group(4) && exact_group(5),
               "accumulation groups must stay exact");
 constexpr int NACC = 6;         // accumulators: s+t = 2 .. 6 and s+t >= 7 (480 TMEM columns)
 // Sixteen drain warps (4-19, four to a 32-lane quadrant of tensor memory, 20 columns each): with
