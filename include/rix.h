@@ -392,6 +392,12 @@ rix_status rix_stage_times(rix_ctx *ctx, double *ms, int32_t n, int32_t *n_build
  * *chunks x 2 x 128 x 80 x 16.  Synchronises on the last event; resets the
  * counts.  EUNSUPPORTED otherwise. */
 rix_status rix_gemm_profile(rix_ctx *ctx, double *ms, int64_t *launches, int64_t *chunks);
+/* Output tiles that those launches computed and the accumulation groups that they
+ * took for them, since the previous call of this function (a tile is one group
+ * where the operands' digits keep its partial sums exact, else one per 512 K
+ * values).  Call it before rix_gemm_profile, which forgets the events that this
+ * call waits for.  EUNSUPPORTED as above. */
+rix_status rix_gemm_groups(rix_ctx *ctx, int64_t *tiles, int64_t *groups);
 
 const char *rix_strerror(rix_status s);
 const char *rix_last_error(const rix_ctx *ctx);

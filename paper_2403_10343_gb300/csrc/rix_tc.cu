@@ -578,7 +578,8 @@ struct GemmArgs {
   // members that meet a kept block of the tile's rows); stages without a bit are skipped
   const unsigned long long *kmask = nullptr;
   const int64_t *kmask_off = nullptr;
-  unsigned long long *chunks = nullptr;  // profiling: 128 x 80 x 16 MMAs issued (K stages x K steps x slice pairs)
+  // profiling: 128 x 80 x 16 MMAs issued (K stages x K steps x slice pairs), tiles, accumulation groups
+  unsigned long long *chunks = nullptr;
   unsigned long long *X128 = nullptr;  // deterministic mode: X additions as 128-bit fixed point (2 words each)
   // batched mode: the largest digit sum of squares of every row and column tile (wsq)
   const float *tA = nullptr, *tB = nullptr;
@@ -719,6 +720,7 @@ __global__ void __launch_bounds__(NTHR, 1) k_gemm_sliced(GemmArgs g) {
   if (warp == 0 && lane == 0) {
     // ------------------------------------------------------------ producer
     uint32_t cg = 0;  // stages issued by this CTA
+    uint32_t nt = 0, ng = 0;  // tiles and accumulation groups of them
     int st = 0;
     uint32_t ph = 1;  // parity of the ring's previous round (the first one passes at once)
     bool aborted = false;
@@ -730,6 +732,7 @@ __global__ void __launch_bounds__(NTHR, 1) k_gemm_sliced(GemmArgs g) {
       const char *ga = (const char *)ti.gA + (int64_t)ti.mt * nk * (S * A_TILE);
       const char *gb = (const char *)ti.gB + (int64_t)ti.nt * nk * (S * B_TILE);
       int lc = 0, gl = 0;  // live stages of the tile so far, and of the open group
+      nt++;
       for (int w = 0; w < (nk + 63) / 64 && !aborted; w++) {
         unsigned long long m = nk - 64 * w < 64 ? (1ull << (nk - 64 * w)) - 1 : ~0ull;
         if (ti.km) m &= ti.km[w];  // an all-zero B tile or row block: neither copied nor multiplied
@@ -741,6 +744,7 @@ __global__ void __launch_bounds__(NTHR, 1) k_gemm_sliced(GemmArgs g) {
             break;
           }
           lc++;
+          ng += gl == 0;
           st_flags[st] = (gl == 0 ? ST_OPEN : 0u) | (gl == ti.group - 1 || lc == ti.nlive ? ST_LAST : 0u);
           if (++gl == ti.group) gl = 0;
           uint8_t *sa = smem + st * stage_bytes;
@@ -762,8 +766,11 @@ __global__ void __launch_bounds__(NTHR, 1) k_gemm_sliced(GemmArgs g) {
       end_posted = 1;
     }
     issued_chunks = cg;
-    if (g.chunks && cg)
+    if (g.chunks && cg) {
       atomicAdd(g.chunks, (unsigned long long)cg * (unsigned long long)(S * (S + 1) / 2) * (KC / 16));
+      atomicAdd(g.chunks + 1, (unsigned long long)nt);
+      atomicAdd(g.chunks + 2, (unsigned long long)ng);
+    }
   } else if (warp == 1 && lane == 0) {
     // ------------------------------------------------------------ MMA issuer
     bool issued = false;
@@ -2051,8 +2058,8 @@ rix_status rix_mixed_plan(rix_ctx *ctx, const std::vector<int64_t> &ptrZ) {
   if (ctx->opt.deterministic) {
     if ((s = rix_alloc(ctx, &ctx->d_X128, 2 * ctx->offK[ctx->nk])) != RIX_OK) return s;
   }
-  if ((s = rix_alloc(ctx, &ctx->d_gemm_chunks, 1)) != RIX_OK) return s;
-  RIX_CUDA_TRY(ctx, cudaMemset(ctx->d_gemm_chunks, 0, sizeof(unsigned long long)));
+  if ((s = rix_alloc(ctx, &ctx->d_gemm_chunks, 3)) != RIX_OK) return s;
+  RIX_CUDA_TRY(ctx, cudaMemset(ctx->d_gemm_chunks, 0, 3 * sizeof(unsigned long long)));
   ctx->mx_buf_bytes = buf;
   ctx->stats.tensor_flops = tflops;
   ctx->have_mx = true;
@@ -3365,5 +3372,17 @@ extern "C" rix_status rix_gemm_profile(rix_ctx *ctx, double *ms, int64_t *launch
   RIX_CUDA_TRY(ctx, cudaMemcpy(&c, ctx->d_gemm_chunks, sizeof c, cudaMemcpyDeviceToHost));
   RIX_CUDA_TRY(ctx, cudaMemset(ctx->d_gemm_chunks, 0, sizeof c));
   *chunks = (int64_t)c;
+  return RIX_OK;
+}
+
+extern "C" rix_status rix_gemm_groups(rix_ctx *ctx, int64_t *tiles, int64_t *groups) {
+  if (!ctx || !tiles || !groups) return RIX_EINVAL;
+  if (ctx->opt.profile < 2 || !ctx->have_mx) return RIX_EUNSUPPORTED;
+  if (!ctx->gemm_ev.empty()) RIX_CUDA_TRY(ctx, cudaEventSynchronize(ctx->gemm_ev.back()));
+  unsigned long long c[2] = {0, 0};
+  RIX_CUDA_TRY(ctx, cudaMemcpy(c, ctx->d_gemm_chunks + 1, sizeof c, cudaMemcpyDeviceToHost));
+  RIX_CUDA_TRY(ctx, cudaMemset(ctx->d_gemm_chunks + 1, 0, sizeof c));
+  *tiles = (int64_t)c[0];
+  *groups = (int64_t)c[1];
   return RIX_OK;
 }

@@ -90,6 +90,7 @@ def load():
     lib.rix_fit_C.argtypes = [P, P, P, ctypes.c_double, P, P]
     lib.rix_gemm_profile.argtypes = [P, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_int64),
                                      ctypes.POINTER(ctypes.c_int64)]
+    lib.rix_gemm_groups.argtypes = [P, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int64)]
     lib.rix_bloch.argtypes = [P, P, ctypes.c_int32, P, P, P]
     lib.rix_build_K_spin.argtypes = [P, ctypes.c_int32, P, P, P]
     lib.rix_energy_spin.argtypes = [P, ctypes.c_int32, P, P, P, P]
@@ -104,7 +105,7 @@ def load():
               "rix_backward", "rix_fold_gamma", "rix_stats", "rix_stage_times", "rix_gemm_sliced",
               "rix_autotune", "rix_count_flops", "rix_check", "rix_test_stalled_gemm", "rix_bloch",
               "rix_build_K_spin", "rix_energy_spin", "rix_build_K_delta", "rix_force_stress",
-              "rix_gemm_profile", "rix_fit_C"):
+              "rix_gemm_profile", "rix_gemm_groups", "rix_fit_C"):
         getattr(lib, f).restype = I
     _lib = lib
     return lib
@@ -379,6 +380,13 @@ def gemm_profile(ctx):
     ms, n, ch = ctypes.c_double(), ctypes.c_int64(), ctypes.c_int64()
     _check(load().rix_gemm_profile(ctx, ctypes.byref(ms), ctypes.byref(n), ctypes.byref(ch)), ctx)
     return ms.value, n.value, ch.value
+
+
+def gemm_groups(ctx):
+    """rix_gemm_groups: (tiles, accumulation groups) of the sliced-GEMM launches since the last call."""
+    nt, ng = ctypes.c_int64(), ctypes.c_int64()
+    _check(load().rix_gemm_groups(ctx, ctypes.byref(nt), ctypes.byref(ng)), ctx)
+    return nt.value, ng.value
 
 
 def destroy(ctx):
