@@ -104,7 +104,8 @@ typedef struct {
   int32_t precision;               /* rix_precision */
   int32_t n_slices;                /* mixed mode: BF16 slices per operand, 1..8 (0 = default, 5; the
                                       regrouped plans take one more) */
-  int64_t max_workspace_bytes;     /* 0 = no limit beyond the device's free memory */
+  int64_t max_workspace_bytes;     /* 0 = no limit beyond the device's free memory (small arrays then
+                                      share allocations of 1 MB) */
   int32_t verbose;                 /* 0 = silent */
   int32_t profile;                 /* 1 = record a CUDA event after every stage of rix_build_K
                                       (skipped while the stream is being captured into a graph);
@@ -146,7 +147,8 @@ typedef struct {
   double flops_stage[6];           /* T, U2, X12 (terms 1+2), Z (term 4), X34, symmetrise */
   double min_bytes;                /* 8 (nnz C + V + D) + 8 nnz K */
   double tensor_flops;             /* mixed mode: tensor-core FLOPs issued per build */
-  int64_t workspace_bytes;         /* library-owned device memory */
+  int64_t workspace_bytes;         /* library-owned device memory (the unused ends of shared
+                                      allocations included) */
   int32_t n_row_blocks;            /* row blocks of the memory plan (1 = all intermediates resident) */
   double flops_term2;              /* the term-2 part of flops_stage[2] (on the tensor cores when mixed) */
   double tensor_flops_stage[5];    /* mixed mode: tensor FLOPs issued per build for terms 3+4, term 2,
