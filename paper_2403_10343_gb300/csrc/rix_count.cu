@@ -119,7 +119,7 @@ __global__ void k_cnt_X34(int64_t np, const double *f34, const uint8_t *keepC, d
 
 unsigned grid_for(int64_t n) {
   const int64_t b = (n + CNT_THREADS - 1) / CNT_THREADS;
-  return (unsigned)std::max<int64_t>(1, std::min<int64_t>(b, 152 * 16));
+  return (unsigned)std::max<int64_t>(1, std::min<int64_t>(b, rix::SMS * 16));
 }
 
 }  // namespace

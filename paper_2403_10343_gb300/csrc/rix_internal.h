@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "../../include/rix.h"
+#include "rix_rules.h"
 
 #define RIX_CUDA_TRY(ctx, call)                                                  \
   do {                                                                            \

@@ -774,7 +774,7 @@ static rix_status build_lists(rix_ctx *ctx) {
           c.push_back(len * std::min(pt, NA(a) - p0) * per);
         }
       }
-      if (cap == CAP_MIN || it.size() >= (cap == CAP_MAX ? 32 : 4) * 152) return (int32_t)cap;
+      if (cap == CAP_MIN || it.size() >= (size_t)(cap == CAP_MAX ? 32 : 4) * SMS) return (int32_t)cap;
       it.clear();
       c.clear();
     }
@@ -788,7 +788,7 @@ static rix_status build_lists(rix_ctx *ctx) {
       const int64_t qt = std::max<int64_t>(1, ctx->cap_U / (NB(a) * NB(g)));
       for (int64_t q0 = 0; q0 < NA(g); q0 += qt) itU.push_back(make_int2((int)p, (int)q0));
     }
-    if (ctx->cap_U == CAP_MIN || itU.size() >= 4 * 152) break;
+    if (ctx->cap_U == CAP_MIN || itU.size() >= 4 * SMS) break;
   }
   // launch order: most expensive first (longest processing time first)
   auto order_by = [](std::vector<int2> &it, const std::vector<double> &cost) {
@@ -813,7 +813,7 @@ static rix_status build_lists(rix_ctx *ctx) {
       cX12.push_back((double)(ptrX12[s + 1] - ptrX12[s]) * (t1 + (double)NA(a) * NB(a) * NB(e)));
     }
   // A cluster of 2^c CTAs per output (1 to 16) where the longest output of its component
-  // would otherwise take more than half of an even share of the stage on the 152 SMs: its CTA
+  // would otherwise take more than half of an even share of the stage on the SMs: its CTA
   // would run on alone at the end.  (Two waters, at most 8 -> 16 CTAs: terms 1+2 168 -> 107 us,
   // terms 3+4 27 -> 20 us.)
   auto clusters = [&](const std::vector<int32_t> &ord, const std::vector<double> &c, auto atom) {
@@ -825,7 +825,7 @@ static rix_status build_lists(rix_ctx *ctx) {
     }
     std::vector<int> cls(ctx->ncomp, 0);
     for (int m = 0; m < ctx->ncomp; m++)
-      while (cls[m] + 1 < rix_ctx::NCLS && 2.0 * top[m] * 152 > tot[m] * (1 << cls[m])) cls[m]++;
+      while (cls[m] + 1 < rix_ctx::NCLS && 2.0 * top[m] * SMS > tot[m] * (1 << cls[m])) cls[m]++;
     return cls;
   };
   const std::vector<int> cls12 = clusters(ordX12, cX12, [&](int32_t s) { return atomA2[s]; });

@@ -1239,7 +1239,7 @@ template <class Acc>
 void launch_slice_dig(int64_t n0, int64_t n, const Acc &acc, int S, __nv_bfloat16 *planes, const int *e, uint64_t *wsq,
                       int kmax, cudaStream_t st) {
   const int64_t warps = n / 8, k32 = (kmax + 31) / 32;
-  const int64_t ny = std::min<int64_t>(k32, (152 * 32 + warps - 1) / warps);
+  const int64_t ny = std::min<int64_t>(k32, (rix::SMS * 32 + warps - 1) / warps);
   const int kper = std::min((int)((k32 + ny - 1) / ny) * 32, 1 << 18);
   const dim3 grid((unsigned)((warps * 32 + 255) / 256), (unsigned)((kmax + kper - 1) / kper));
   switch (S) {
@@ -1258,7 +1258,7 @@ template <class Acc>
 void slice_rows(int64_t n0, int64_t n, const Acc &acc, int S, __nv_bfloat16 *planes, int *e, uint64_t *wsq, int kmax,
                 cudaStream_t st) {
   if (n <= 0) return;
-  if (n < 152 * 32) k_slice_exp<Acc, 4><<<(unsigned)((n + 1) / 2), 256, 0, st>>>(n0, n, acc, e, wsq);
+  if (n < rix::SMS * 32) k_slice_exp<Acc, 4><<<(unsigned)((n + 1) / 2), 256, 0, st>>>(n0, n, acc, e, wsq);
   else k_slice_exp<Acc, 1><<<(unsigned)((n + 7) / 8), 256, 0, st>>>(n0, n, acc, e, wsq);
   launch_slice_dig(n0, n, acc, S, planes, e, wsq, kmax, st);
 }
