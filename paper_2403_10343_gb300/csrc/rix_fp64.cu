@@ -769,8 +769,6 @@ rix_status last(rix_ctx *ctx, const char *what) {
   return e == cudaSuccess ? RIX_OK : fail_cuda(ctx, what, e);
 }
 
-bool g_attr_done = false;
-
 }  // namespace
 
 rix_status rix_launch_pairs(rix_ctx *ctx, const double *d_xyz, const double *d_cell, const int nr[3],
@@ -813,27 +811,66 @@ rix_status rix_launch_symcheck(rix_ctx *ctx, cudaStream_t st) {
   return last(ctx, "k_symcheck");
 }
 
+// Shared memory up to SM_MAX doubles for the kernels that stage tiles, and clusters of 16 CTAs, which
+// are beyond the portable size.  Set for every context, on its device.
+rix_status rix_fp64_attrs(rix_ctx *ctx) {
+  auto set = [&](auto *kernel, int smem, bool cluster) {
+    cudaError_t e = cudaSuccess;
+    if (smem) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess && cluster) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e;
+  };
+  RIX_CUDA_TRY(ctx, set(k_X12<1>, SM_MAX * 8, true));
+  RIX_CUDA_TRY(ctx, set(k_X12<XMAXE>, SM_MAX * 8, true));
+  RIX_CUDA_TRY(ctx, set(k_X34<1>, 0, true));
+  RIX_CUDA_TRY(ctx, set(k_X34<XMAXE>, 0, true));
+  RIX_CUDA_TRY(ctx, set(k_T, TCOL * 64 * 8, false));
+  RIX_CUDA_TRY(ctx, set(k_Z, SM_MAX * 8, false));
+  return RIX_OK;
+}
+
 namespace {
 
-void set_attrs() {
-  if (!g_attr_done) {
-    // clusters of 16 CTAs are beyond the portable size
-    cudaFuncSetAttribute(k_X12<1>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(k_X12<XMAXE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(k_X34<1>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(k_X34<XMAXE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(k_X12<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_MAX * 8);
-    cudaFuncSetAttribute(k_X12<XMAXE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_MAX * 8);
-    cudaFuncSetAttribute(k_T, cudaFuncAttributeMaxDynamicSharedMemorySize, TCOL * 64 * 8);
-    cudaFuncSetAttribute(k_Z, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_MAX * 8);
-    g_attr_done = true;
-  }
+// the configuration of count outputs, each shared by a cluster of ns CTAs (at: its attribute)
+cudaLaunchConfig_t split_config(int64_t count, int ns, int smem, cudaStream_t st, cudaLaunchAttribute *at) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(count * ns));
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = ns;
+  at->val.clusterDim.y = at->val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = ns > 1 ? 1 : 0;
+  return cfg;
 }
+
+// whether the device (or the part of it that the context has) runs clusters of ns CTAs of the kernel
+template <class... P>
+bool cluster_fits(void (*kernel)(P...), int ns, int smem) {
+  cudaLaunchAttribute at;
+  const cudaLaunchConfig_t cfg = split_config(1, ns, smem, 0, &at);
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess) return n > 0;
+  cudaGetLastError();
+  return false;
+}
+
+}  // namespace
+
+int rix_cluster_limit(int want) {
+  return fitting_class(want, [](int ns) {  // k_X12 with the largest tile that the autotuner may choose
+    return cluster_fits(k_X12<1>, ns, SM_MAX * 8) && cluster_fits(k_X12<XMAXE>, ns, SM_MAX * 8) &&
+           cluster_fits(k_X34<1>, ns, 0) && cluster_fits(k_X34<XMAXE>, ns, 0);
+  });
+}
+
+namespace {
 
 // Z(B;E') for the Z work items [first, first + count) of block b.
 rix_status launch_Z_items(rix_ctx *ctx, const double *D, int b, int64_t first, int64_t count, int smb,
                           cudaStream_t st) {
-  set_attrs();
   if (!count) return RIX_OK;
   k_Z<<<(unsigned)count, NT, smb * 8, st>>>(ctx->d_itZ + ctx->segZ[b] + first, ctx->d_ptrZ, ctx->d_LZ,
                                             ctx->d_atomA2, ctx->d_atomB2, ctx->d_off2, ctx->d_pB, ctx->d_nb,
@@ -847,17 +884,8 @@ rix_status launch_Z_items(rix_ctx *ctx, const double *D, int b, int64_t first, i
 // a launch of count outputs, each shared by a cluster of ns CTAs
 template <class... P, class... A>
 cudaError_t launch_split(void (*kernel)(P...), int64_t count, int ns, int smem, cudaStream_t st, A... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(count * ns));
-  cfg.blockDim = dim3(NT);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
   cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = ns;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = ns > 1 ? 1 : 0;
+  const cudaLaunchConfig_t cfg = split_config(count, ns, smem, st, &at);
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
@@ -879,7 +907,6 @@ int64_t n_X12(const rix_ctx *ctx, int b) {
 
 // terms 1+2 for the output blocks [first, first + count) of block b's launch order.
 rix_status launch_X12_items(rix_ctx *ctx, int b, int64_t first, int64_t count, int smb, cudaStream_t st) {
-  set_attrs();
   smb = std::max(smb, 64 * 64);  // one column entry of 64 functions over 64 rows, or a 64 x 64 output
   const int64_t *seg = &ctx->segX12[rix_ctx::NCLS * b];
   for (int c = 0; c < rix_ctx::NCLS; c++) {  // the class's part of [first, first + count)
@@ -939,7 +966,6 @@ int32_t rix_x34_launches(const rix_ctx *ctx) {
 // of their row atoms; k_T stores the others, if there are any ((H2O)8, all on the tensor cores:
 // a launch of CTAs that return at once took 11 of 1,390 us).
 rix_status rix_launch_T_block(rix_ctx *ctx, const double *D, int b, cudaStream_t st) {
-  set_attrs();
   const int64_t nT = ctx->segT[b + 1] - ctx->segT[b];
   const bool tc = ctx->have_mx && ctx->n_ttc > 0;
   if (tc) {
@@ -974,7 +1000,6 @@ rix_status rix_launch_Z_block(rix_ctx *ctx, const double *D, int b, cudaStream_t
 }
 
 rix_status rix_fp64_build(rix_ctx *ctx, const double *D, double *K, cudaStream_t st, int accumulate) {
-  set_attrs();
   rix_status s;
   if ((s = rix_prof_mark(ctx, 0, st)) != RIX_OK) return s;
   if ((s = rix_launch_flags(ctx, D, ctx->d_offD, ctx->np, ctx->d_keepD, st, ctx->d_normD)) != RIX_OK) return s;
@@ -1107,7 +1132,6 @@ extern "C" rix_status rix_autotune(rix_ctx *ctx, const double *D, const char *ca
     }
   }
   rix_status s;
-  set_attrs();
   if ((s = rix_launch_flags(ctx, D, ctx->d_offD, ctx->np, ctx->d_keepD, st)) != RIX_OK) return s;
   if ((s = launch_live(ctx, st)) != RIX_OK) return s;
   RIX_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_X, 0, sizeof(double) * ctx->offK[ctx->nk], st));

@@ -326,6 +326,8 @@ int32_t rix_tt_launches(const rix_ctx *ctx);
 // FP64 path launches (rix_fp64.cu)
 rix_status rix_fp64_build(rix_ctx *ctx, const double *D, double *K, cudaStream_t st, int accumulate = 0);
 int32_t rix_x12_launches(const rix_ctx *ctx);  // of one build
+rix_status rix_fp64_attrs(rix_ctx *ctx);        // the kernels' launch attributes on the context's device
+int rix_cluster_limit(int want);                // the largest launch class up to want that the device takes
 int32_t rix_x34_launches(const rix_ctx *ctx);  // per block of middle atoms
 rix_status rix_launch_T_block(rix_ctx *ctx, const double *D, int b, cudaStream_t st);
 rix_status rix_launch_Z_block(rix_ctx *ctx, const double *D, int b, cudaStream_t st);

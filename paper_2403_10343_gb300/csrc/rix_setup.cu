@@ -812,10 +812,8 @@ static rix_status build_lists(rix_ctx *ctx) {
       const double t1 = pae >= 0 && ctx->rep1[pae] ? (double)NA(e) * NB(a) * (NA(a) + NB(e)) : 0.0;
       cX12.push_back((double)(ptrX12[s + 1] - ptrX12[s]) * (t1 + (double)NA(a) * NB(a) * NB(e)));
     }
-  // A cluster of 2^c CTAs per output (1 to 16) where the longest output of its component
-  // would otherwise take more than half of an even share of the stage on the SMs: its CTA
-  // would run on alone at the end.  (Two waters, at most 8 -> 16 CTAs: terms 1+2 168 -> 107 us,
-  // terms 3+4 27 -> 20 us.)
+  // The launch class of a component's outputs is that of its longest one (cluster_class), as far
+  // as the device takes clusters of that size.
   auto clusters = [&](const std::vector<int32_t> &ord, const std::vector<double> &c, auto atom) {
     std::vector<double> tot(ctx->ncomp, 0.0), top(ctx->ncomp, 0.0);
     for (size_t i = 0; i < ord.size(); i++) {
@@ -824,8 +822,10 @@ static rix_status build_lists(rix_ctx *ctx) {
       top[m] = std::max(top[m], c[i]);
     }
     std::vector<int> cls(ctx->ncomp, 0);
-    for (int m = 0; m < ctx->ncomp; m++)
-      while (cls[m] + 1 < rix_ctx::NCLS && 2.0 * top[m] * SMS > tot[m] * (1 << cls[m])) cls[m]++;
+    int want = 0;
+    for (int m = 0; m < ctx->ncomp; m++) want = std::max(want, cls[m] = cluster_class(top[m], tot[m], rix_ctx::NCLS - 1));
+    const int limit = rix_cluster_limit(want);
+    for (int &c : cls) c = std::min(c, limit);
     return cls;
   };
   const std::vector<int> cls12 = clusters(ordX12, cX12, [&](int32_t s) { return atomA2[s]; });
@@ -1220,6 +1220,7 @@ extern "C" rix_status rix_setup(const rix_system *sys, const rix_options *opt, r
   }
   *(volatile int *)ctx->h_err = 0;
   if ((s = rix_noalloc_attach(ctx)) != RIX_OK) return fail(s);
+  if ((s = rix_fp64_attrs(ctx)) != RIX_OK) return fail(s);
   if ((s = build_lists(ctx)) != RIX_OK) return fail(s);
   ctx->stats.workspace_bytes = (int64_t)ctx->dev_bytes;
   *out = ctx;
