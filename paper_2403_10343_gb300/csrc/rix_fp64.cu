@@ -872,6 +872,7 @@ namespace {
 rix_status launch_Z_items(rix_ctx *ctx, const double *D, int b, int64_t first, int64_t count, int smb,
                           cudaStream_t st) {
   if (!count) return RIX_OK;
+  smb = std::max(smb, ctx->max_nel);  // one row of F, nbG x nbE: a cached budget may be smaller
   k_Z<<<(unsigned)count, NT, smb * 8, st>>>(ctx->d_itZ + ctx->segZ[b] + first, ctx->d_ptrZ, ctx->d_LZ,
                                             ctx->d_atomA2, ctx->d_atomB2, ctx->d_off2, ctx->d_pB, ctx->d_nb,
                                             ctx->d_na, ctx->d_C, ctx->d_offC, ctx->d_V, ctx->d_offV, D, ctx->d_offD,
