@@ -142,8 +142,9 @@ typedef struct {
 typedef struct {
   int64_t n_atoms, n_pairs, n_pairs2, n_kblocks;
   int64_t c_elems, v_elems, d_elems, k_elems;
-  double flops_fp64;               /* algorithmic FLOPs of one rix_build_K (unpadded products; terms 1
-                                      and 4 counted once per pair / K block, as the build runs them) */
+  double flops_fp64;               /* algorithmic FLOPs of one rix_build_K (unpadded products; term 1
+                                      counted once per pair, in the orientation that the build runs, term
+                                      4 once per K block with every Z product: rix_count_flops) */
   double flops_stage[6];           /* T, U2, X12 (terms 1+2), Z (term 4), X34, symmetrise */
   double min_bytes;                /* 8 (nnz C + V + D) + 8 nnz K */
   double tensor_flops;             /* mixed mode: tensor-core FLOPs issued per build */
@@ -282,7 +283,7 @@ rix_status rix_force_stress(rix_ctx *ctx, int32_t c, const double *dEdC_dev, con
  * from the on-site blocks V(I,I,0), V(J,J,0) and the pair block V(I,J,n).
  * V_dev: packed V (RIX_LIST_V layout), eri_dev: the three-centre integrals
  * (ij|nu) in the packed C layout, C_dev: output, packed C (all device).  Each
- * representative pair is factored by Cholesky and solved on the device; its
+ * representative pair is factored (L D L^T) and solved on the device; its
  * partner receives the transposed numbers, so C is exactly pair-symmetric
  * (rix_set_CV accepts it).  lambda >= 0 shifts the metric's diagonal (a
  * Tikhonov fit) for metrics that are numerically singular; EINVAL if a shifted

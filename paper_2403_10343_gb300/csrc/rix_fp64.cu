@@ -17,8 +17,8 @@
 // V and D stated after Eqs. 12a-12d; the paper's "2G"), and terms 1 and 4 are symmetric by
 // themselves, so the last line restores all four terms exactly.
 //
-// Each kernel is output-stationary: one CTA owns an output block (or a row
-// tile of it), walks its product list and keeps the sums in registers, so no
+// Each kernel is output-stationary: one CTA (or a cluster of them) owns an output
+// block or a row tile of it, walks its product list and keeps the sums in registers, so no
 // atomics are needed and every run sums in the same order.
 #include <cooperative_groups.h>
 
@@ -315,9 +315,11 @@ __global__ void __launch_bounds__(NT) k_U2(const int2 *items, const int32_t *pA,
 // products that need no staging run without a barrier.  Where a system has few or very
 // uneven outputs, a cluster of ns CTAs shares one output (the launch classes of rix_ctx).
 // R elements per thread: 1 up to 256 elements, else 16 (and one group).
-// GB300, one group with staged operands and now: (H2O)64 terms 1+2 652 and 309 ms (1.14 TFLOP/s
-// of the products it keeps, FP64 pipe 1.25), 24-atom ice cell terms 3+4 245 and 115 ms (1.13);
-// (H2O)8, split over 2^c CTAs, terms 1+2 5.34 and 1.99 ms.
+// GB300, one group with staged operands, with these kernels at first, and now with the cheaper
+// orientation of term 1 and empty T and Z blocks skipped: (H2O)64 terms 1+2 652, 309 and 267 ms (1.15
+// TFLOP/s of the products it keeps, FP64 pipe 1.25), 24-atom ice cell terms 3+4 245, 115 and
+// 61 ms; (H2O)8, split over 2^c CTAs, terms 1+2 5.34, 1.99 and 1.75 ms.  K blocks above 256 elements (12-atom
+// perovskite, up to 1,521): the whole FP64 build 1,483 and 700 ms.
 struct Split {
   int ng, grp, el0;  // groups of the CTA, this thread's group (ng: no work) and first element
   int part, parts;   // share of this thread's group among the shares of the whole cluster

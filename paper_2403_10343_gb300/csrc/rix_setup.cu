@@ -381,8 +381,8 @@ static void find_components(rix_ctx *ctx) {
 // (na nb per row atom and nb_B na_G nb_G per column), which makes Z the larger one by far
 // except where few atoms lie within the cutoff.  (GB300, mixed, K blocks halved and Z halved:
 // (H2O)64 cluster 169.3 and 123.0 ms, 192-atom ice cell 379 and 330 ms, 12-atom perovskite 239
-// and 210 ms.  FP64: the 24-atom ice cell, whose K blocks outweigh Z (245 and 31 ms), stays with
-// the halved K blocks.)
+// and 210 ms.  FP64: the 24-atom ice cell, whose K blocks outweigh Z (61 ms halved, Z 29 ms in
+// full), stays with the halved K blocks.)
 static std::vector<uint8_t> choose_term4(rix_ctx *ctx) {
   const int nat = ctx->nat;
   const bool mixed = ctx->opt.precision == RIX_MIXED_BF16;

@@ -1529,7 +1529,7 @@ struct PlanHost {
 // Slices per operand when rix_options.n_slices is 0: with balanced digits five
 // slices (six for the regrouped plans) keep the mixed build within 1e-8 in K and
 // 1e-6 Ha in E_x on the water, ice and perovskite workloads measured (largest
-// difference 1.1e-7 Ha, the 1,536-atom perovskite).
+// difference 1.7e-7 Ha, the 1,536-atom perovskite).
 constexpr int DEFAULT_SLICES = 5;
 
 // Slices per plan: the regrouped forms (term 1 as T x C, Z with Kronecker rows)
