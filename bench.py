@@ -426,6 +426,9 @@ def roofline(precision, r):
         alg = tensor_alg_flops(stats)
         t = gm["ms_per_build"] * 1e-3
         peak = pk_peaks["bf16_tflops_sustained"]
+        # the sustained peak is power-limited: its clock, where recorded, belongs beside the fractions of it
+        mhz = (pk_peaks.get("clocks_under_load") or {}).get("sm_mhz_median")
+        at = f", at a median SM clock of {mhz:.0f} MHz" if mhz else ""
         issued = gm["stage_pairs_per_build"] * GEMM_STAGE_PAIR_FLOPS
         per_launch = gm["stage_pairs_per_build"] / max(1.0, gm["launches_per_build"])
         traffic = None if GEMM_DRAM_BYTES_PER_STAGE_PAIR is None else GEMM_DRAM_BYTES_PER_STAGE_PAIR * per_launch
@@ -434,7 +437,7 @@ def roofline(precision, r):
                 "traffic_unit": "bytes per launch",
                 "traffic_source": "ncu DRAM bytes per 128x80x16 MMA over the GEMM launches of the 192-atom cluster "
                                   "build, times the MMAs of an average launch here",
-                "peak_source": f"bf16 sustained (a kernel timed inside a long step), {src}",
+                "peak_source": f"bf16 sustained (a kernel timed inside a long step), {src}{at}",
                 "alg_flops_per_build": alg, "kernel_ms_per_build": gm["ms_per_build"],
                 "launches_per_build": gm["launches_per_build"],
                 "issued_bf16_flops_per_build": issued, "issued_tflops": issued / t / 1e12,
